@@ -352,31 +352,96 @@ SVM_HD double xd_round(const XdAcc &acc, int unit)
     g.w2 = acc.w2 ^ s;
     g.w3 = acc.w3 ^ s;
     xd_add4(g, s & 1u, 0u, 0u, 0u);
-    uint32_t a, b, c, rest;
-    int top;
-    if (g.w3) {
-        a = g.w3; b = g.w2; c = g.w1; rest = g.w0; top = 3;
-    } else if (g.w2) {
-        a = g.w2; b = g.w1; c = g.w0; rest = 0u; top = 2;
-    } else if (g.w1) {
-        a = g.w1; b = g.w0; c = 0u; rest = 0u; top = 1;
-    } else if (g.w0) {
-        a = g.w0; b = 0u; c = 0u; rest = 0u; top = 0;
-    } else {
-        return 0.0;
-    }
-    const int lz = count_leading_zeros32(a);
-    const uint32_t h = xd_funnel(b, a, lz), mid = xd_funnel(c, b, lz), low = c << lz;
+    // selects, not branches: lanes whose leading limbs differ stay together
+    const bool b3 = g.w3 != 0u, b2 = g.w2 != 0u, b1 = g.w1 != 0u;
+    const uint32_t a = b3 ? g.w3 : (b2 ? g.w2 : (b1 ? g.w1 : g.w0));
+    const uint32_t b = b3 ? g.w2 : (b2 ? g.w1 : (b1 ? g.w0 : 0u));
+    const uint32_t c = b3 ? g.w1 : (b2 ? g.w0 : 0u);
+    const uint32_t rest = b3 ? g.w0 : 0u;
+    const int top = b3 ? 96 : (b2 ? 64 : (b1 ? 32 : 0));
+    const int lz = count_leading_zeros32(a);   // 32 when the sum is 0
+    const uint32_t h = xd_funnel(b, a, lz & 31), mid = xd_funnel(c, b, lz & 31), low = c << (lz & 31);
     uint64_t mant = ((uint64_t)h << 21) | (mid >> 11);   // leading one at bit 52
     const bool half = (mid >> 10) & 1u;
     const bool sticky = ((mid & 0x3ffu) | low | rest) != 0u;
-    int e = 32 * top + 31 - lz + unit;   // |a| 2^unit = 1.f 2^e
-    if (half && (sticky || (mant & 1u))) {
-        mant += 1;
-        if (mant >> 53) { mant >>= 1; e += 1; }
+    const int e = top + 31 - lz + unit;   // |a| 2^unit = 1.f 2^e
+    mant += (half && (sticky || (mant & 1u))) ? 1u : 0u;
+    // the leading one adds the exponent field's last unit, a carry out of the
+    // rounding the one above it
+    const uint64_t bits = ((uint64_t)(e + 1022) << 52) + mant;
+    return a ? bits_to_double(bits | ((uint64_t)(s & 1u) << 63)) : 0.0;
+}
+
+// x / y correctly rounded (nearest, ties to even), in integer arithmetic:
+// this part's FP64 pipe takes one operation of a warp per 64 cycles, and a
+// division is about nine dependent ones (561 cycles measured for one warp).
+// Long division of the significands in radix 2^30 (two digits), the digits
+// from a 32-bit reciprocal of the divisor's leading 32 bits: the special
+// function unit's 23 bits, one Newton step (r <- r + r (1 - r d)). Write X, Y
+// for the 53-bit significands. The quotient Q of X 2^60 / Y is off by at most
+// 10 units (bounds at each line), and has 60 or 61 bits, 7 or 8 more than a
+// double: it rounds like the exact quotient unless those bits lie within 10
+// units of one half, when the remainder decides. Subnormal, infinite, zero
+// or NaN operands and results near the ends of the exponent range go to the
+// division operator.
+SVM_HD double div_int(double x, double y)
+{
+    const uint64_t bx = double_to_bits(x), by = double_to_bits(y);
+    const int ex = (int)(bx >> 52) & 0x7ff, ey = (int)(by >> 52) & 0x7ff;
+    const int eq = ex - ey + 1022;   // exponent field for a quotient in [1/2, 1) of the scale
+    if ((unsigned)(ex - 1) >= 2046u || (unsigned)(ey - 1) >= 2046u || (unsigned)(eq - 1) >= 2044u) return x / y;
+    const uint64_t X = (bx & 0x000fffffffffffffull) | 0x0010000000000000ull;
+    const uint64_t Y = (by & 0x000fffffffffffffull) | 0x0010000000000000ull;
+    const uint32_t yh = (uint32_t)(Y >> 21);   // in [2^31, 2^32)
+    // g ~ 1 / F, F = yh / 2^31 cut to 24 bits, in (1/2, 1]: relative error below 2^-21
+    uint32_t r;
+    {
+        const uint32_t fb = 0x3f800000u | ((yh >> 8) & 0x007fffffu);
+        float F;
+#if defined(__CUDA_ARCH__)
+        F = __uint_as_float(fb);
+        const float gf = __fdividef(1.0f, F);
+#else
+        memcpy(&F, &fb, sizeof F);
+        const float gf = 1.0f / F;
+#endif
+        uint32_t gb = float_to_bits(gf);
+#if defined(SVM_DIV_SEED_ULP)
+        gb += (uint32_t)(SVM_DIV_SEED_ULP);   // host check: the seed's error
+#endif
+        gb = gb < 0x3f000000u ? 0x3f000000u : gb;   // an approximate 1 / F may end just below 1/2
+        r = gb >= 0x3f800000u ? 0xffffffffu : (0x800000u | (gb & 0x007fffffu)) << 8;   // ~ 2^63 / yh
     }
-    const uint64_t bits = ((uint64_t)(e + 1023) << 52) | (mant & 0x000fffffffffffffull);
-    return bits_to_double(bits | ((uint64_t)(s & 1u) << 63));
+    // Newton: r <= 2^63 / yh afterwards, less by at most 3 (it cannot pass 2^32 - 1)
+    const int64_t err = (int64_t)(0x8000000000000000ull - (uint64_t)r * yh);
+    r += (uint32_t)(int32_t)(((int64_t)(int32_t)(r >> 1) * (int64_t)(int32_t)(err >> 12)) >> 50);
+    // first digit: X 2^30 / Y, off by at most 3; the remainder is below 2^55 in magnitude
+    const uint32_t q1 = (uint32_t)(((uint64_t)(uint32_t)(X >> 21) * r) >> 33);
+    const int64_t rem1 = (int64_t)((X << 30) - (uint64_t)q1 * Y);
+    // second digit: rem1 2^30 / Y, off by at most 10 (rem1 cut to its upper bits)
+    const int32_t q2 = (int32_t)(((int64_t)(int32_t)(rem1 >> 24) * (int64_t)(int32_t)(r >> 1)) >> 29);
+    uint64_t Q = ((uint64_t)q1 << 30) + (uint64_t)(int64_t)q2;
+    const int up = (int)(Q >> 60) & 1;   // Q in [2^60, 2^61): the quotient is at least 1
+    const uint32_t half = 64u << up;
+    const uint32_t low = (uint32_t)Q & (2u * half - 1u);
+    uint64_t mant = (Q + half) >> (7 + up);
+    if (low - half + 10u <= 20u) {
+        // the exact quotient (Q, rem): X 2^60 = Q Y + rem, 0 <= rem < Y
+        int64_t rem = (int64_t)(((uint64_t)rem1 << 30) - (uint64_t)(int64_t)q2 * Y);
+        while (rem < 0) {
+            rem += (int64_t)Y;
+            --Q;
+        }
+        while (rem >= (int64_t)Y) {
+            rem -= (int64_t)Y;
+            ++Q;
+        }
+        const uint32_t lo2 = (uint32_t)Q & (2u * half - 1u);
+        mant = Q >> (7 + up);
+        if (lo2 > half || (lo2 == half && (rem != 0 || (mant & 1u)))) mant += 1;
+    }
+    const uint64_t bits = ((uint64_t)(eq + up - 1) << 52) + mant;
+    return bits_to_double(bits | ((bx ^ by) & 0x8000000000000000ull));
 }
 
 }  // namespace svmgb

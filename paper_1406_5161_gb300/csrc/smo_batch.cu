@@ -58,6 +58,7 @@ struct BatchShared {
     BatchFinish wfin[kWarps];
     double du, dl, au_new, al_new;
     unsigned char st_u, st_l;
+    PairPre pre;
     int job;
 };
 
@@ -183,6 +184,11 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             if (!first) {
                 if (!dless(thr, low.f - up.f)) { status_code = 0; break; }
                 if (iter >= J.max_iter) { status_code = 1; break; }
+                // the pair step's part that K(up, low) does not enter
+                if (warp == kPreWarp) {
+                    const PairPre p = pair_pre<MODE == MODE_FP64>(up, low, C);
+                    if (lane == 0) sh.pre = p;
+                }
                 // ---- 1. targets into the shared-memory buffer
                 if (dense) {
                     if constexpr (MODE == MODE_MIXED) {
@@ -249,63 +255,37 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
 #pragma unroll
                         for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
                     }
-                    if (lane == 0) {
-                        double kul, rinv = 0.0;
-                        if constexpr (MODE == MODE_BINARY) {
-                            int dist = up.len + low.len - 2 * s;
-                            dist = dist < 0 ? 0 : dist;
-                            kul = ktab[dist];
-                            rinv = rtab[dist];
-                        } else if constexpr (MODE == MODE_FP64) {
-                            double d2 = up.nrm + low.nrm - 2.0 * s;
-                            kul = exp_neg_fx(gamma * dpos(d2), expfx_s);
+                    const PairPre pre = sh.pre;
+                    bool curved;
+                    double q;
+                    if constexpr (MODE == MODE_BINARY) {
+                        int dist = up.len + low.len - 2 * s;
+                        dist = dist < 0 ? 0 : dist;
+                        const double eta = 2.0 - 2.0 * ktab[dist], rinv = rtab[dist];
+                        curved = bits_less(1e-12, eta);
+                        const double q0 = pre.slope * rinv;
+                        const double rr = fma(-eta, q0, pre.slope);
+                        q = fma(rr, rinv, q0);
+                    } else {
+                        double kul;
+                        if constexpr (MODE == MODE_FP64) {
+                            kul = exp_neg_fx(gamma * dpos(fma(-2.0, s, pre.nsum)), expfx_s);
                         } else {
-                            float d2 = (float)up.nrm + (float)low.nrm - 2.0f * s;
-                            kul = (double)__expf(-gammaf * fmaxf(d2, 0.f));
+                            const float d2 = norm_f32(up.nrm) + norm_f32(low.nrm) - 2.0f * s;
+                            kul = widen_f32(__expf(-gammaf * fmaxf(d2, 0.f)));
                         }
-                        const bool yu_neg = up.y < 0, yl_neg = low.y < 0;
-                        const double au = up.a, al = low.a;
                         const double eta = 2.0 - 2.0 * kul;
-                        const bool opposite = yu_neg != yl_neg;
-                        double Lo, Hi;
-                        if (opposite) {
-                            const double x = al - au;
-                            Lo = dless(x, 0.0) ? 0.0 : x;
-                            const double h = C + al - au;
-                            Hi = dless(h, C) ? h : C;
-                        } else {
-                            const double x = al + au - C;
-                            Lo = dless(x, 0.0) ? 0.0 : x;
-                            const double h = al + au;
-                            Hi = dless(h, C) ? h : C;
-                        }
-                        const double slope = neg_if(up.f - low.f, yl_neg);
-                        double aln;
-                        if (dless(1e-12, eta)) {
-                            double q;
-                            if constexpr (MODE == MODE_BINARY) {
-                                const double q0 = slope * rinv;
-                                const double rr = fma(-eta, q0, slope);
-                                q = fma(rr, rinv, q0);
-                            } else {
-                                q = slope / eta;
-                            }
-                            const double t = al + q;
-                            aln = dless(t, Lo) ? Lo : (dless(Hi, t) ? Hi : t);
-                        } else {
-                            aln = dless(0.0, slope) ? Hi : Lo;
-                        }
-                        double aun = au + neg_if(al - aln, opposite);
-                        if (dless(aln, snap)) aln = 0.0;
-                        if (dless(c_snap, aln)) aln = C;
-                        if (dless(aun, snap)) aun = 0.0;
-                        if (dless(c_snap, aun)) aun = C;
-                        sh.du = neg_if(aun - au, yu_neg);
-                        sh.dl = neg_if(aln - al, yl_neg);
-                        sh.au_new = aun;
-                        sh.al_new = aln;
-                        sh.st_u = status_of(!yu_neg, aun, C);
-                        sh.st_l = status_of(!yl_neg, aln, C);
+                        curved = bits_less(1e-12, eta);
+                        q = div_int(pre.slope, curved ? eta : 1.0);
+                    }
+                    const PairStep ps = pair_solve(pre, up, low, curved, q, C, snap, c_snap);
+                    if (lane == 0) {
+                        sh.du = ps.du;
+                        sh.dl = ps.dl;
+                        sh.au_new = ps.au;
+                        sh.al_new = ps.al;
+                        sh.st_u = status_of(up.y > 0, ps.au, C);
+                        sh.st_l = status_of(low.y > 0, ps.al, C);
                     }
                     __syncwarp();
                     step_bar_arrive(kThreads);
@@ -341,8 +321,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                             kl = exp_neg_fx(gamma * dpos(d2l), expfx_s);
                         } else {
                             const float nf = normf[g];
-                            float d2u = (float)up.nrm + nf - 2.0f * su;
-                            float d2l = (float)low.nrm + nf - 2.0f * sl;
+                            float d2u = norm_f32(up.nrm) + nf - 2.0f * su;
+                            float d2l = norm_f32(low.nrm) + nf - 2.0f * sl;
                             // widened exactly by integer operations (a conversion
                             // instruction would take a slot of the FP64 pipe)
                             ku = widen_f32(__expf(-gammaf * fmaxf(d2u, 0.f)));
@@ -636,7 +616,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 sd.f = fj[r];
                 sd.a = aj[r];
                 if constexpr (MODE == MODE_FP64) sd.nrm = norm[g];
-                else if constexpr (MODE == MODE_MIXED) sd.nrm = (double)normf[g];
+                else if constexpr (MODE == MODE_MIXED) sd.nrm = norm_bits(normf[g]);
                 else sd.nrm = 0.0;
                 if (dense) {
                     sd.p0 = g;

@@ -48,6 +48,7 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxCluster = 16;    // largest thread-block cluster launched (non-portable size)
 constexpr int kKcThread = 32;      // the kernel-row cache's directory keeper (lane 0 of warp 1)
+constexpr int kPreWarp = kWarps - 1;   // computes the pair step's bounds beside warp 0
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p)
 {
@@ -68,6 +69,11 @@ __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_re
 // named barrier 1 between the pair-step warp (arrives) and the row warps (wait)
 __device__ __forceinline__ void step_bar_arrive(int n) { asm volatile("bar.arrive 1, %0;" ::"r"(n) : "memory"); }
 __device__ __forceinline__ void step_bar_sync(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
+
+// named barrier 3 between the warp that computes the pair step's bounds
+// (arrives) and the pair-step warp (waits), for rows that need no target fill
+__device__ __forceinline__ void pre_bar_arrive() { asm volatile("bar.arrive 3, 64;" ::: "memory"); }
+__device__ __forceinline__ void pre_bar_sync() { asm volatile("bar.sync 3, 64;" ::: "memory"); }
 
 __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v)
 {
@@ -272,6 +278,97 @@ __device__ __forceinline__ uint8_t status_of(bool ypos, double a, double C)
     return (uint8_t)(set | (ypos ? 0x80 : 0));
 }
 
+// a < b on the bit patterns: right when a or b is >= 0 (finite, or a NaN the
+// caller treats alike), with -0 below +0
+__device__ __forceinline__ bool bits_less(double a, double b)
+{
+    return __double_as_longlong(a) < __double_as_longlong(b);
+}
+// The FP32 squared norm of a mixed-mode candidate travels as its bits in the
+// FP64 field (a conversion either way would take a slot of the FP64 pipe).
+__device__ __forceinline__ double norm_bits(float v) { return __hiloint2double(0, __float_as_int(v)); }
+__device__ __forceinline__ float norm_f32(double v) { return __int_as_float(__double2loint(v)); }
+
+// ---- the pair step, Eqs. (alphaup) / (rho)
+//
+// The step is one warp's chain of FP64 operations, which on this part issue
+// one per 64 cycles whatever their dependences, with 40 more for each value
+// that integer selects read. So it is cut to what follows from K(up, low):
+// the part before it (PairPre) runs in another warp, on another scheduler's
+// FP64 pipe, while the target rows load; the quotient is divided in integer
+// arithmetic (div_int); clamps and snaps compare bit patterns as signed
+// integers (every bound is >= 0); and a step that ends at 0 or C, or keeps
+// alpha_low' unsnapped, takes its difference from a value at hand. On one
+// cluster (2,000 dense rows, FP64, no row cached) the part after the inner
+// product, most of it the exponential and this, took 4,290 cycles of a step
+// before and 3,070 now. Every FP64 operation is the oracle's, on the same
+// operands.
+struct PairPre {
+    double lo, hi;      // [L, H] of alpha_low'
+    double cu, cl;      // C - alpha_up, C - alpha_low
+    double slope;       // y_low (f_up - f_low)
+    double nsum;        // ||x_up||^2 + ||x_low||^2 (FP64 rows)
+};
+struct PairStep {
+    double au, al;      // alpha_up', alpha_low'
+    double du, dl;      // y_up (alpha_up' - alpha_up), y_low (alpha_low' - alpha_low)
+};
+
+__device__ __forceinline__ double pair_slope(const Side &up, const Side &low)
+{
+    const bool neg = low.y < 0;
+    return (neg ? low.f : up.f) - (neg ? up.f : low.f);
+}
+
+// opposite labels: L = max(0, al - au), H = min(C, (C + al) - au); equal
+// labels: L = max(0, (al + au) - C), H = min(C, al + au)
+template <bool NORMS>
+__device__ __forceinline__ PairPre pair_pre(const Side &up, const Side &low, double C)
+{
+    PairPre p;
+    const bool opposite = (up.y < 0) != (low.y < 0);
+    const double au = up.a, al = low.a;
+    const double v1 = al + (opposite ? neg_if(au, true) : au);
+    const double w = (opposite ? C : v1) + (opposite ? al : neg_if(C, true));
+    const double h3 = w - au;
+    const double xl = opposite ? v1 : w, xh = opposite ? h3 : v1;
+    p.lo = bits_less(xl, 0.0) ? 0.0 : xl;
+    p.hi = bits_less(xh, C) ? xh : C;
+    p.slope = pair_slope(up, low);
+    p.cu = C - au;
+    p.cl = C - al;
+    p.nsum = NORMS ? up.nrm + low.nrm : 0.0;
+    return p;
+}
+
+// q = slope / eta when curved (eta > 1e-12), else the end-point rule; the
+// joint clip, then alphas within 1e-12 C of a bound set to it
+__device__ __forceinline__ PairStep pair_solve(const PairPre &p, const Side &up, const Side &low, bool curved,
+                                               double q, double C, double snap, double c_snap)
+{
+    PairStep r;
+    const bool yu_neg = up.y < 0, yl_neg = low.y < 0;
+    const bool opposite = yu_neg != yl_neg;
+    const double au = up.a, al = low.a;
+    const double t = al + q;
+    const bool at_lo = curved ? bits_less(t, p.lo) : !bits_less(0.0, p.slope);
+    const bool at_hi = curved ? bits_less(p.hi, t) : true;
+    const double alc = at_lo ? p.lo : (at_hi ? p.hi : t);
+    const double d = al - alc;
+    // alpha_up' from the clipped, not yet snapped alpha_low'
+    const double auc = au + neg_if(d, opposite);
+    const bool l0 = bits_less(alc, snap), lc = bits_less(c_snap, alc);
+    const bool u0 = bits_less(auc, snap), uc = bits_less(c_snap, auc);
+    r.al = l0 ? 0.0 : (lc ? C : alc);
+    r.au = u0 ? 0.0 : (uc ? C : auc);
+    const double dl = l0 ? neg_if(al, true) : (lc ? p.cl : neg_if(d, true));
+    const double dn = auc - au;
+    const double du = u0 ? neg_if(au, true) : (uc ? p.cu : dn);
+    r.dl = neg_if(dl, yl_neg);
+    r.du = neg_if(du, yu_neg);
+    return r;
+}
+
 // Selection keys: the I_up side minimises f, the I_low side maximises it;
 // both become a minimum over (key, index), so ties go to the lowest index.
 __device__ __forceinline__ unsigned long long key_up(double f) { return dkey(f); }
@@ -423,6 +520,7 @@ struct Shared {
     double du, dl;        // y_up * delta alpha_up, y_low * delta alpha_low
     double au_new, al_new;
     unsigned char st_u, st_l;
+    PairPre pre;
     int flag_timeout;
 };
 
@@ -626,14 +724,16 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
             up.p0 = A.indptr[up.i];
             up.len = (int)(A.indptr[up.i + 1] - up.p0);
             up.y = A.y[up.i];
-            up.nrm = MODE == MODE_MIXED ? (double)A.normf[up.i] : (MODE == MODE_FP64 ? A.norm[up.i] : 0.0);
+            if constexpr (MODE == MODE_MIXED) up.nrm = norm_bits(A.normf[up.i]);
+            if constexpr (MODE == MODE_FP64) up.nrm = A.norm[up.i];
             load_mask(up);
         }
         if (low.i >= 0 && low.i < A.n) {
             low.p0 = A.indptr[low.i];
             low.len = (int)(A.indptr[low.i + 1] - low.p0);
             low.y = A.y[low.i];
-            low.nrm = MODE == MODE_MIXED ? (double)A.normf[low.i] : (MODE == MODE_FP64 ? A.norm[low.i] : 0.0);
+            if constexpr (MODE == MODE_MIXED) low.nrm = norm_bits(A.normf[low.i]);
+            if constexpr (MODE == MODE_FP64) low.nrm = A.norm[low.i];
             load_mask(low);
         }
     }
@@ -731,10 +831,9 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
         else A.alpha[lo + r] = v;
     };
     auto NRM = [&](int r) -> double {
-        if constexpr (MODE == MODE_BINARY || BITS) return 0.0;
-        else if constexpr (RES) return (double)nrm_s[r];
-        else if constexpr (MODE == MODE_FP64) return A.norm[lo + r];
-        else return (double)A.normf[lo + r];
+        if constexpr (MODE != MODE_FP64) return 0.0;
+        else if constexpr (RES) return nrm_s[r];
+        else return A.norm[lo + r];
     };
     // mixed mode: the FP32 norm as it is stored (no round trip through the
     // FP64 pipe, whose conversions cost as much as its arithmetic here)
@@ -755,7 +854,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
     int prev_len_u = 0, prev_len_l = 0;
     // optional per-phase cycle counts of CTA 0 (one clock read per phase)
     const bool timed = A.phase_times && cta == 0;
-    uint64_t tp = (timed && tid == 0) ? clock64() : 0;
+    uint64_t tp = timed ? clock64() : 0;
     // with phase_times every CTA counts the cycles from step start to publish
     const bool busy_on = A.phase_times && A.cta_cycles;
     uint64_t cta_t0 = 0, busy = 0;
@@ -770,7 +869,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
         int *tcl = tcol + (size_t)(buf * 2 + 1) * maxnnz;
         bool shrink_now = false;
         const double bup_sel = up.f, blow_sel = WSS ? beta_low : low.f;   // values that chose this pair
-        if (busy_on && tid == 0) cta_t0 = clock64();
+        if (busy_on) cta_t0 = clock64();
         if (!first) {
             if (!gap_open) { exit_reason = 0; break; }
             if (iter >= A.iter_limit) { exit_reason = 1; break; }
@@ -838,6 +937,13 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                     kc_pf1 = hl_ ? -1 : sl_;
                 }
             }
+            // the pair step's part that K(up, low) does not enter, beside the
+            // target fill (rows of at most 224 entries leave this warp free)
+            if (warp == kPreWarp) {
+                const PairPre p = pair_pre<MODE == MODE_FP64>(up, low, C);
+                if (lane == 0) sh.pre = p;
+                if constexpr (BITS) pre_bar_arrive();
+            }
             // ---- 1. targets: x_up into .x / byte 0, x_low into .y / byte 1
             //         (bit-mask modes: the masks came with the exchange); x_up
             //         by the first half of the threads and x_low by the
@@ -869,7 +975,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
             }
             row_visits += total;
             if constexpr (!BITS) __syncthreads();
-            if (timed && tid == 0) { uint64_t t = clock64(); ph[0] += t - tp; tp = t; }
+            if (timed) { uint64_t t = clock64(); ph[0] += t - tp; tp = t; }
         }
 
         // ---- 2. the pair step (warp 0) runs while warps 1.. compute the
@@ -931,29 +1037,39 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
 #pragma unroll
                     for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
                 }
-                if (timed && tid == 0) { uint64_t t = clock64(); ph[6] += t - tp; tp = t; }
-                if (lane == 0) {
+                if (timed) { uint64_t t = clock64(); ph[6] += t - tp; tp = t; }
+                {
+                    // (every lane, so that the warp stays together)
                     // kernel value K(up, low) and, from the tables on binary
                     // input, eta = 2 - 2K with the correctly rounded 1 / eta
-                    double kul, rinv = 0.0, eta;
+                    double kul, rinv = 0.0, eta, q;
                     bool curved;
+                    PairPre pre;
                     if constexpr (MODE == MODE_BINARY || BITS) {
                         int dist = BITS ? s : up.len + low.len - 2 * s;
                         dist = dist < 0 ? 0 : dist;
-                        kul = ktab[dist];
                         rinv = rtab[dist];
                         eta = etab[dist];
                         curved = __double_as_longlong(rinv) != 0;   // eta > 1e-12
+                        // slope / eta from the correctly rounded 1/eta of
+                        // the table: one Markstein correction gives the
+                        // correctly rounded quotient
+                        const double slope = pair_slope(up, low);
+                        const double q0 = slope * rinv;
+                        const double r = fma(-eta, q0, slope);
+                        q = fma(r, rinv, q0);
+                        if constexpr (BITS) pre_bar_sync();
+                        pre = sh.pre;
                     } else {
+                        pre = sh.pre;
                         if (A.kernel == KERNEL_RBF) {
                             if constexpr (MODE == MODE_FP64) {
                                 // the fixed-point exp, as in the row pass
-                                double d2 = up.nrm + low.nrm - 2.0 * s;
-                                kul = kul_cached ? kul_c
-                                                 : exp_neg_fx(A.gamma * dpos(d2), expfx_s);
+                                if (kul_cached) kul = kul_c;
+                                else kul = exp_neg_fx(A.gamma * dpos(fma(-2.0, s, pre.nsum)), expfx_s);
                             } else {
-                                float d2 = (float)up.nrm + (float)low.nrm - 2.0f * s;
-                                kul = (double)__expf(-gammaf * fmaxf(d2, 0.f));
+                                float d2 = norm_f32(up.nrm) + norm_f32(low.nrm) - 2.0f * s;
+                                kul = widen_f32(__expf(-gammaf * fmaxf(d2, 0.f)));
                             }
                             eta = 2.0 - 2.0 * kul;   // K(x,x) = 1
                         } else {
@@ -966,72 +1082,28 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                             } else {
                                 const float c0 = (float)A.coef0;
                                 kul = (double)kernel_of_dot(A.kernel, gammaf, c0, A.degree, (float)s);
-                                kuu = (double)kernel_of_dot(A.kernel, gammaf, c0, A.degree, (float)up.nrm);
-                                kll = (double)kernel_of_dot(A.kernel, gammaf, c0, A.degree, (float)low.nrm);
+                                kuu = (double)kernel_of_dot(A.kernel, gammaf, c0, A.degree, norm_f32(up.nrm));
+                                kll = (double)kernel_of_dot(A.kernel, gammaf, c0, A.degree, norm_f32(low.nrm));
                             }
                             eta = __dsub_rn(__dadd_rn(kuu, kll), __dmul_rn(2.0, kul));
                         }
-                        curved = dless(1e-12, eta);
+                        curved = bits_less(1e-12, eta);
+                        q = div_int(pre.slope, curved ? eta : 1.0);
                     }
-                    // Eq. (alphaup) with rho = -eta (Eq. rho), K(x,x) = 1,
-                    // clipped to the feasible segment [L, H]; end-point rule
-                    // for a flat curvature. Each FP64 operation is the
-                    // oracle's (same operands, same order). On this part a
-                    // warp's FP64 instructions issue about one per 64 cycles,
-                    // so signs y = +-1 are applied by choosing operands, and
-                    // comparisons, clamps and snaps work on integer keys.
-                    const bool yu_neg = up.y < 0, yl_neg = low.y < 0;
-                    const double au = up.a, al = low.a;
-                    const bool opposite = yu_neg != yl_neg;
-                    // slope = y_low (f_up - f_low)
-                    const double slope = (yl_neg ? low.f : up.f) - (yl_neg ? up.f : low.f);
-                    // [L, H]: opposite labels L = max(0, al - au),
-                    // H = min(C, (C + al) - au); equal labels L = max(0,
-                    // (al + au) - C), H = min(C, al + au)
-                    const double v1 = al + (opposite ? neg_if(au, true) : au);
-                    const double w = (opposite ? C : v1) + (opposite ? al : neg_if(C, true));
-                    const double h3 = w - au;
-                    const double xL = opposite ? v1 : w, xH = opposite ? h3 : v1;
-                    const double Lo = dless(xL, 0.0) ? 0.0 : xL;
-                    const double Hi = dless(xH, C) ? xH : C;
-                    double alc;
-                    if (curved) {
-                        double q;
-                        if constexpr (MODE == MODE_BINARY || BITS) {
-                            // slope / eta from the correctly rounded 1/eta of
-                            // the table: one Markstein correction gives the
-                            // correctly rounded quotient
-                            const double q0 = slope * rinv;
-                            const double r = fma(-eta, q0, slope);
-                            q = fma(r, rinv, q0);
-                        } else {
-                            q = slope / eta;
-                        }
-                        const double t = al + q;
-                        const unsigned long long kt = dkey(t);
-                        alc = kt < dkey(Lo) ? Lo : (dkey(Hi) < kt ? Hi : t);
-                    } else {
-                        alc = dless(0.0, slope) ? Hi : Lo;
+                    const PairStep ps = pair_solve(pre, up, low, curved, q, C, snap, c_snap);
+                    if (lane == 0) {
+                        sh.du = ps.du;
+                        sh.dl = ps.dl;
+                        sh.au_new = ps.au;
+                        sh.al_new = ps.al;
+                        sh.st_u = status_of(up.y > 0, ps.au, C);
+                        sh.st_l = status_of(low.y > 0, ps.al, C);
                     }
-                    // alpha_up' = au + s (al - alpha_low'), s = y_up y_low,
-                    // from the clipped (not yet snapped) alpha_low'
-                    const double aunc = fma(opposite ? -1.0 : 1.0, al - alc, au);
-                    const unsigned long long ka = dkey(alc), ku = dkey(aunc);
-                    const unsigned long long ks = dkey(snap), kc = dkey(c_snap);
-                    const double aln = ka < ks ? 0.0 : (kc < ka ? C : alc);
-                    const double aun = ku < ks ? 0.0 : (kc < ku ? C : aunc);
-                    // y_up (alpha_up' - au) and y_low (alpha_low' - al)
-                    sh.du = (yu_neg ? au : aun) - (yu_neg ? aun : au);
-                    sh.dl = (yl_neg ? al : aln) - (yl_neg ? aln : al);
-                    sh.au_new = aun;
-                    sh.al_new = aln;
-                    sh.st_u = status_of(!yu_neg, aun, C);
-                    sh.st_l = status_of(!yl_neg, aln, C);
                 }
                 __syncwarp();
                 if constexpr (BITS && RES) step_bar_sync(kThreads);   // warp 0 joins the f updates
                 else step_bar_arrive(kThreads);
-                if (timed && tid == 0) { uint64_t t = clock64(); ph[1] += t - tp; tp = t; }
+                if (timed) { uint64_t t = clock64(); ph[1] += t - tp; tp = t; }
             }
         } else if constexpr (BITS && RES) {
             // ---- 3. row pass, bit-mask rows held on chip, in two sweeps
@@ -1068,7 +1140,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
             KT *kc_ru = kc_step ? static_cast<KT *>(A.kc) + (size_t)sh.kc_su * A.kc_ld : nullptr;
             KT *kc_rl = kc_step ? static_cast<KT *>(A.kc) + (size_t)sh.kc_sl * A.kc_ld : nullptr;
             const bool skip_sums = kc_hu && kc_hl;
-            const float up_nrmf = (float)up.nrm, low_nrmf = (float)low.nrm;
+            const float up_nrmf = norm_f32(up.nrm), low_nrmf = norm_f32(low.nrm);   // mixed rows
             // streamed segment with no row shrunk: its active list is the
             // identity (lists are reset to it and compacted in order), so the
             // row index needs no load
@@ -1510,7 +1582,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
             const uint8_t sb = GETST(r);
             sd.f = GETF(r);
             sd.a = GETA(r);
-            sd.nrm = NRM(r);
+            if constexpr (MODE == MODE_MIXED) sd.nrm = norm_bits(NRMF(r));
+            else sd.nrm = NRM(r);
             sd.p0 = RES ? base + p0 : p0;
             sd.i = (int)(lo + r);
             sd.len = (int)(p1 - p0);
@@ -1565,7 +1638,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
             }
             cnt = kept;
         }
-        if (timed && tid == 0) { uint64_t t = clock64(); ph[2] += t - tp; tp = t; }
+        if (timed) { uint64_t t = clock64(); ph[2] += t - tp; tp = t; }
         // tagged slot of the exchange through global memory, per leader (per
         // CTA in a flat launch) and epoch parity
         auto tslot = [&](int par, int c) {
@@ -1621,10 +1694,10 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                     CandFull *dst = cluster.map_shared_rank(sh.ccand, 0);
                     dst[crank] = cf;
                 }
-                if (lane == 0) {
-                    if (busy_on) busy += clock64() - cta_t0;
-                    if (timed) { uint64_t t = clock64(); ph[phs] += t - tp; tp = t; }
-                }
+                // (clocks are read by whole warps: a lane apart would run the
+                // collectives that follow one lane at a time)
+                if (busy_on) busy += clock64() - cta_t0;
+                if (timed) { uint64_t t = clock64(); ph[phs] += t - tp; tp = t; }
             }
             // the previous step's target rows are cleared while others wait
             if (!BITS && !gx && prev_valid && warp >= 8) {
@@ -1895,7 +1968,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
             }
         };
         exchange(false);
-        if (timed && tid == 0) { uint64_t t = clock64(); ph[4] += t - tp; tp = t; }
+        if (timed) { uint64_t t = clock64(); ph[4] += t - tp; tp = t; }
         if (sh.res.flag) break;
         prev_valid = first ? 0 : 1;
         prev_len_u = up.len;
@@ -1972,7 +2045,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                         if constexpr (MODE == MODE_FP64)
                             kuu = kernel_of_dot(A.kernel, A.gamma, A.coef0, A.degree, up.nrm);
                         else if constexpr (MODE == MODE_MIXED)
-                            kuu = (double)kernel_of_dot(A.kernel, gammaf, (float)A.coef0, A.degree, (float)up.nrm);
+                            kuu = (double)kernel_of_dot(A.kernel, gammaf, (float)A.coef0, A.degree, norm_f32(up.nrm));
                     }
                     constexpr int RPW = 32 / LPR;
                     const int gl = lane & (LPR - 1);
@@ -2026,7 +2099,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                                     const double d2 = up.nrm + NRM(r) - 2.0 * su;
                                     kut = exp_neg_fx(A.gamma * dpos(d2), expfx_s);
                                 } else {
-                                    const float d2 = (float)up.nrm + NRMF(r) - 2.0f * su;
+                                    const float d2 = norm_f32(up.nrm) + NRMF(r) - 2.0f * su;
                                     kut = widen_f32(__expf(-gammaf * fmaxf(d2, 0.f)));
                                 }
                                 eta = 2.0 - 2.0 * kut;   // K(x,x) = 1
@@ -2038,7 +2111,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                                 } else {
                                     const float c0 = (float)A.coef0;
                                     kut = (double)kernel_of_dot(A.kernel, gammaf, c0, A.degree, (float)su);
-                                    ktt = (double)kernel_of_dot(A.kernel, gammaf, c0, A.degree, (float)NRM(r));
+                                    ktt = (double)kernel_of_dot(A.kernel, gammaf, c0, A.degree, NRMF(r));
                                 }
                                 eta = __dsub_rn(__dadd_rn(kuu, ktt), __dmul_rn(2.0, kut));
                             }
@@ -2048,7 +2121,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                 }
                 cta_reduce(true, gk, gi, gr, gk, gi, gr, gneg);
                 exchange(true);
-                if (timed && tid == 0) { uint64_t t = clock64(); ph[7] += t - tp; tp = t; }
+                if (timed) { uint64_t t = clock64(); ph[7] += t - tp; tp = t; }
                 if (sh.res.flag) break;
                 low = sh.res.low;
             }
@@ -2057,7 +2130,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
             A.trace[2 * iter] = up.i == INT_MAX ? -1 : (A.gmap ? A.gmap[up.i] : up.i);
             A.trace[2 * iter + 1] = low.i == INT_MAX ? -1 : (A.gmap ? A.gmap[low.i] : low.i);
         }
-        if (timed && tid == 0) { uint64_t t = clock64(); ph[5] += t - tp; tp = t; }
+        if (timed) { uint64_t t = clock64(); ph[5] += t - tp; tp = t; }
     }
     cluster.sync();   // no CTA leaves while its shared memory may still be written
 
