@@ -38,6 +38,21 @@
 
 namespace svmgb {
 
+// The rare ends of the functions below, out of line on the device: inlined at
+// every use they doubled the code a step of the SMO kernel runs through, which
+// its instruction caches do not hold.
+#if defined(__CUDACC__)
+static __device__ __noinline__ double exp_library(double y) { return exp(y); }
+static __device__ __noinline__ double div_library(double x, double y) { return x / y; }
+#endif
+#if defined(__CUDA_ARCH__)
+#define SVM_EXP_LIBRARY svmgb::exp_library
+#define SVM_DIV_LIBRARY svmgb::div_library
+#else
+#define SVM_EXP_LIBRARY exp
+#define SVM_DIV_LIBRARY(x, y) ((x) / (y))
+#endif
+
 SVM_HD double bits_to_double(uint64_t b)
 {
 #if defined(__CUDA_ARCH__)
@@ -151,7 +166,7 @@ constexpr uint64_t kExpfxBits700 = 0x4085e00000000000ull;   // the bits of 700.0
 SVM_HD double exp_neg_fx(double y, const uint64_t *T)
 {
     const uint64_t b = double_to_bits(y);
-    if (b > kExpfxBits700) return exp(-y);   // y < 0, y > 700 or NaN
+    if (b > kExpfxBits700) return SVM_EXP_LIBRARY(-y);   // y < 0, y > 700 or NaN
     // y = m 2^(be - 1075), so y 2^64 = m << sh, sh = be - 1011 <= 21
     const int be = (int)(b >> 52);
     const uint64_t m = (b & 0x000fffffffffffffull) | (be ? 0x0010000000000000ull : 0ull);
@@ -374,7 +389,8 @@ SVM_HD double xd_round(const XdAcc &acc, int unit)
 
 // x / y correctly rounded (nearest, ties to even), in integer arithmetic:
 // this part's FP64 pipe takes one operation of a warp per 64 cycles, and a
-// division is about nine dependent ones (561 cycles measured for one warp).
+// division is about nine dependent ones (561 cycles measured for one warp;
+// this 350).
 // Long division of the significands in radix 2^30 (two digits), the digits
 // from a 32-bit reciprocal of the divisor's leading 32 bits: the special
 // function unit's 23 bits, one Newton step (r <- r + r (1 - r d)). Write X, Y
@@ -384,13 +400,32 @@ SVM_HD double xd_round(const XdAcc &acc, int unit)
 // units of one half, when the remainder decides. Subnormal, infinite, zero
 // or NaN operands and results near the ends of the exponent range go to the
 // division operator.
-SVM_HD double div_int(double x, double y)
+//
+// div_head prepares the dividend (ahead of the divisor where that comes late);
+// ok: it is a normal number whose quotient by any y in [2^-64, 2^64] is one.
+struct DivHead {
+    uint64_t X;    // significand
+    int e;         // exponent field
+    int ok;
+    double x;
+};
+SVM_HD DivHead div_head(double x)
 {
-    const uint64_t bx = double_to_bits(x), by = double_to_bits(y);
-    const int ex = (int)(bx >> 52) & 0x7ff, ey = (int)(by >> 52) & 0x7ff;
-    const int eq = ex - ey + 1022;   // exponent field for a quotient in [1/2, 1) of the scale
-    if ((unsigned)(ex - 1) >= 2046u || (unsigned)(ey - 1) >= 2046u || (unsigned)(eq - 1) >= 2044u) return x / y;
-    const uint64_t X = (bx & 0x000fffffffffffffull) | 0x0010000000000000ull;
+    DivHead h;
+    const uint64_t bx = double_to_bits(x);
+    h.X = (bx & 0x000fffffffffffffull) | 0x0010000000000000ull;
+    h.e = (int)(bx >> 52) & 0x7ff;
+    h.ok = h.e >= 100 && h.e <= 1900;
+    h.x = x;
+    return h;
+}
+
+// y: a normal number with the quotient's exponent field in range
+SVM_HD double div_tail(const DivHead &h, double y)
+{
+    const uint64_t by = double_to_bits(y);
+    const int ey = (int)(by >> 52) & 0x7ff;
+    const uint64_t X = h.X;
     const uint64_t Y = (by & 0x000fffffffffffffull) | 0x0010000000000000ull;
     const uint32_t yh = (uint32_t)(Y >> 21);   // in [2^31, 2^32)
     // g ~ 1 / F, F = yh / 2^31 cut to 24 bits, in (1/2, 1]: relative error below 2^-21
@@ -440,8 +475,17 @@ SVM_HD double div_int(double x, double y)
         mant = Q >> (7 + up);
         if (lo2 > half || (lo2 == half && (rem != 0 || (mant & 1u)))) mant += 1;
     }
-    const uint64_t bits = ((uint64_t)(eq + up - 1) << 52) + mant;
-    return bits_to_double(bits | ((bx ^ by) & 0x8000000000000000ull));
+    const uint64_t bits = ((uint64_t)(h.e - ey + 1021 + up) << 52) + mant;
+    return bits_to_double(bits | ((double_to_bits(h.x) ^ by) & 0x8000000000000000ull));
+}
+
+SVM_HD double div_int(double x, double y)
+{
+    const DivHead h = div_head(x);
+    const int ey = (int)(double_to_bits(y) >> 52) & 0x7ff;
+    if ((unsigned)(h.e - 1) >= 2046u || (unsigned)(ey - 1) >= 2046u || (unsigned)(h.e - ey + 1021) >= 2044u)
+        return SVM_DIV_LIBRARY(x, y);
+    return div_tail(h, y);
 }
 
 }  // namespace svmgb

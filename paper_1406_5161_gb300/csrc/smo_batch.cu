@@ -185,10 +185,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 if (!dless(thr, low.f - up.f)) { status_code = 0; break; }
                 if (iter >= J.max_iter) { status_code = 1; break; }
                 // the pair step's part that K(up, low) does not enter
-                if (warp == kPreWarp) {
-                    const PairPre p = pair_pre<MODE == MODE_FP64>(up, low, C);
-                    if (lane == 0) sh.pre = p;
-                }
+                if (warp >= kPre0) pair_pre<MODE == MODE_FP64>(&sh.pre, warp - kPre0, lane, up, low, C);
                 // ---- 1. targets into the shared-memory buffer
                 if (dense) {
                     if constexpr (MODE == MODE_MIXED) {
@@ -263,8 +260,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                         dist = dist < 0 ? 0 : dist;
                         const double eta = 2.0 - 2.0 * ktab[dist], rinv = rtab[dist];
                         curved = bits_less(1e-12, eta);
-                        const double q0 = pre.slope * rinv;
-                        const double rr = fma(-eta, q0, pre.slope);
+                        const double q0 = pre.slope.x * rinv;
+                        const double rr = fma(-eta, q0, pre.slope.x);
                         q = fma(rr, rinv, q0);
                     } else {
                         double kul;
@@ -276,7 +273,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                         }
                         const double eta = 2.0 - 2.0 * kul;
                         curved = bits_less(1e-12, eta);
-                        q = div_int(pre.slope, curved ? eta : 1.0);
+                        q = pair_quotient<true>(pre.slope, curved ? eta : 1.0);
                     }
                     const PairStep ps = pair_solve(pre, up, low, curved, q, C, snap, c_snap);
                     if (lane == 0) {

@@ -48,7 +48,8 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxCluster = 16;    // largest thread-block cluster launched (non-portable size)
 constexpr int kKcThread = 32;      // the kernel-row cache's directory keeper (lane 0 of warp 1)
-constexpr int kPreWarp = kWarps - 1;   // computes the pair step's bounds beside warp 0
+constexpr int kPreWarps = 3;       // the last warps, which compute the pair step's bounds beside warp 0
+constexpr int kPre0 = kWarps - kPreWarps;
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p)
 {
@@ -70,10 +71,17 @@ __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_re
 __device__ __forceinline__ void step_bar_arrive(int n) { asm volatile("bar.arrive 1, %0;" ::"r"(n) : "memory"); }
 __device__ __forceinline__ void step_bar_sync(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
 
-// named barrier 3 between the warp that computes the pair step's bounds
-// (arrives) and the pair-step warp (waits), for rows that need no target fill
-__device__ __forceinline__ void pre_bar_arrive() { asm volatile("bar.arrive 3, 64;" ::: "memory"); }
-__device__ __forceinline__ void pre_bar_sync() { asm volatile("bar.sync 3, 64;" ::: "memory"); }
+// named barrier 3 between the warps that compute the pair step's bounds
+// (arrive) and the pair-step warp (waits)
+__device__ __forceinline__ void pre_bar_arrive() { asm volatile("bar.arrive 3, %0;" ::"n"(32 * (kPreWarps + 1)) : "memory"); }
+__device__ __forceinline__ void pre_bar_sync() { asm volatile("bar.sync 3, %0;" ::"n"(32 * (kPreWarps + 1)) : "memory"); }
+// named barrier 4 after the target fill: the bounds' warps only arrive (their
+// FP64 chains must not hold up the others) and pick the result up later from
+// warp 0 on barrier 5
+__device__ __forceinline__ void fill_bar_arrive() { asm volatile("bar.arrive 4, %0;" ::"n"(kThreads) : "memory"); }
+__device__ __forceinline__ void fill_bar_sync() { asm volatile("bar.sync 4, %0;" ::"n"(kThreads) : "memory"); }
+__device__ __forceinline__ void filled_arrive() { asm volatile("bar.arrive 5, %0;" ::"n"(32 * (kPreWarps + 1)) : "memory"); }
+__device__ __forceinline__ void filled_sync() { asm volatile("bar.sync 5, %0;" ::"n"(32 * (kPreWarps + 1)) : "memory"); }
 
 __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v)
 {
@@ -145,6 +153,18 @@ __device__ __forceinline__ void st_cluster_v4(uint32_t a, uint4 v)
     asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z),
                  "r"(v.w)
                  : "memory");
+}
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_cluster_u16(uint32_t a)
+{
+    uint16_t v;
+    asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
+    return v;
 }
 // asynchronous store into a CTA of the cluster that counts its bytes on that
 // CTA's mbarrier (no fence on the sending side)
@@ -234,6 +254,7 @@ static_assert(offsetof(Side, f) == 0 && offsetof(Side, i) == 32 && offsetof(Side
 // global exchange slots: each candidate and each flag on lines of its own
 constexpr size_t kCandStride = 256;
 static_assert(sizeof(CandFull) <= kCandStride, "candidate slot too small");
+static_assert(offsetof(CandFull, count) == 2 * sizeof(Side), "a candidate is copied as 8-byte words");
 // a leader's tagged slot: the first 48 bytes of both winning sides and the
 // cluster's active count, 25 data words in 13 pairs
 constexpr int kTagPairs = 13;
@@ -294,19 +315,14 @@ __device__ __forceinline__ float norm_f32(double v) { return __int_as_float(__do
 // The step is one warp's chain of FP64 operations, which on this part issue
 // one per 64 cycles whatever their dependences, with 40 more for each value
 // that integer selects read. So it is cut to what follows from K(up, low):
-// the part before it (PairPre) runs in another warp, on another scheduler's
-// FP64 pipe, while the target rows load; the quotient is divided in integer
-// arithmetic (div_int); clamps and snaps compare bit patterns as signed
-// integers (every bound is >= 0); and a step that ends at 0 or C, or keeps
-// alpha_low' unsnapped, takes its difference from a value at hand. On one
-// cluster (2,000 dense rows, FP64, no row cached) the part after the inner
-// product, most of it the exponential and this, took 4,290 cycles of a step
-// before and 3,070 now. Every FP64 operation is the oracle's, on the same
-// operands.
+// the part before it (PairPre) runs in three other warps, on other
+// schedulers' FP64 pipes, while the target rows load; the quotient is divided
+// in integer arithmetic (div_tail); clamps and snaps compare bit patterns as
+// signed integers (every bound is >= 0). Every FP64 operation is the oracle's,
+// on the same operands.
 struct PairPre {
     double lo, hi;      // [L, H] of alpha_low'
-    double cu, cl;      // C - alpha_up, C - alpha_low
-    double slope;       // y_low (f_up - f_low)
+    DivHead slope;      // y_low (f_up - f_low), prepared for its division by eta
     double nsum;        // ||x_up||^2 + ||x_low||^2 (FP64 rows)
 };
 struct PairStep {
@@ -320,53 +336,70 @@ __device__ __forceinline__ double pair_slope(const Side &up, const Side &low)
     return (neg ? low.f : up.f) - (neg ? up.f : low.f);
 }
 
-// opposite labels: L = max(0, al - au), H = min(C, (C + al) - au); equal
-// labels: L = max(0, (al + au) - C), H = min(C, al + au)
+// One part per warp (part 0, 1, 2), written by its lane 0. Opposite labels:
+// L = max(0, al - au), H = min(C, (C + al) - au); equal labels:
+// L = max(0, (al + au) - C), H = min(C, al + au).
 template <bool NORMS>
-__device__ __forceinline__ PairPre pair_pre(const Side &up, const Side &low, double C)
+__device__ __forceinline__ void pair_pre(PairPre *out, int part, int lane, const Side &up, const Side &low, double C)
 {
-    PairPre p;
-    const bool opposite = (up.y < 0) != (low.y < 0);
     const double au = up.a, al = low.a;
-    const double v1 = al + (opposite ? neg_if(au, true) : au);
-    const double w = (opposite ? C : v1) + (opposite ? al : neg_if(C, true));
-    const double h3 = w - au;
-    const double xl = opposite ? v1 : w, xh = opposite ? h3 : v1;
-    p.lo = bits_less(xl, 0.0) ? 0.0 : xl;
-    p.hi = bits_less(xh, C) ? xh : C;
-    p.slope = pair_slope(up, low);
-    p.cu = C - au;
-    p.cl = C - al;
-    p.nsum = NORMS ? up.nrm + low.nrm : 0.0;
-    return p;
+    const bool opposite = (up.y < 0) != (low.y < 0);
+    if (part == 0) {
+        const double v1 = al + (opposite ? neg_if(au, true) : au);
+        const double xl = opposite ? v1 : v1 - C;
+        if (lane == 0) out->lo = bits_less(xl, 0.0) ? 0.0 : xl;
+    } else if (part == 1) {
+        const double v1 = (opposite ? C : au) + al;
+        const double xh = opposite ? v1 - au : v1;
+        if (lane == 0) out->hi = bits_less(xh, C) ? xh : C;
+    } else {
+        const DivHead slope = div_head(pair_slope(up, low));
+        const double nsum = NORMS ? up.nrm + low.nrm : 0.0;
+        if (lane == 0) {
+            out->slope = slope;
+            out->nsum = nsum;
+        }
+    }
 }
 
-// q = slope / eta when curved (eta > 1e-12), else the end-point rule; the
-// joint clip, then alphas within 1e-12 C of a bound set to it
+// q = slope / eta when curved (eta > 1e-12), else the end-point rule; the joint
+// clip; alpha_up' from the clipped, not yet snapped alpha_low'; then alphas
+// within 1e-12 C of a bound set to it
 __device__ __forceinline__ PairStep pair_solve(const PairPre &p, const Side &up, const Side &low, bool curved,
                                                double q, double C, double snap, double c_snap)
 {
     PairStep r;
     const bool yu_neg = up.y < 0, yl_neg = low.y < 0;
-    const bool opposite = yu_neg != yl_neg;
     const double au = up.a, al = low.a;
     const double t = al + q;
-    const bool at_lo = curved ? bits_less(t, p.lo) : !bits_less(0.0, p.slope);
+    const bool at_lo = curved ? bits_less(t, p.lo) : !bits_less(0.0, p.slope.x);
     const bool at_hi = curved ? bits_less(p.hi, t) : true;
     const double alc = at_lo ? p.lo : (at_hi ? p.hi : t);
     const double d = al - alc;
-    // alpha_up' from the clipped, not yet snapped alpha_low'
-    const double auc = au + neg_if(d, opposite);
-    const bool l0 = bits_less(alc, snap), lc = bits_less(c_snap, alc);
-    const bool u0 = bits_less(auc, snap), uc = bits_less(c_snap, auc);
-    r.al = l0 ? 0.0 : (lc ? C : alc);
-    r.au = u0 ? 0.0 : (uc ? C : auc);
-    const double dl = l0 ? neg_if(al, true) : (lc ? p.cl : neg_if(d, true));
-    const double dn = auc - au;
-    const double du = u0 ? neg_if(au, true) : (uc ? p.cu : dn);
+    const double auc = au + neg_if(d, yu_neg != yl_neg);
+    double dl = neg_if(d, true), du = auc - au;
+    r.al = bits_less(alc, snap) ? 0.0 : (bits_less(c_snap, alc) ? C : alc);
+    r.au = bits_less(auc, snap) ? 0.0 : (bits_less(c_snap, auc) ? C : auc);
+    // a value that was exactly 0 or C, or is not snapped, has its difference
+    // already (dl is exactly alc - al)
+    if ((__double_as_longlong(r.al) != __double_as_longlong(alc)) | (__double_as_longlong(r.au) != __double_as_longlong(auc))) {
+        dl = r.al - al;
+        du = r.au - au;
+    }
     r.dl = neg_if(dl, yl_neg);
     r.du = neg_if(du, yu_neg);
     return r;
+}
+
+// slope / eta; an eta of the RBF kernel, 2 - 2 K in (1e-12, 2], needs no check
+template <bool RBF>
+__device__ __forceinline__ double pair_quotient(const DivHead &slope, double eta)
+{
+    if (RBF) {
+        if (!slope.ok) return div_library(slope.x, eta);
+        return div_tail(slope, eta);
+    }
+    return div_int(slope.x, eta);
 }
 
 // Selection keys: the I_up side minimises f, the I_low side maximises it;
@@ -519,8 +552,8 @@ struct Shared {
     int scan_tot;
     double du, dl;        // y_up * delta alpha_up, y_low * delta alpha_low
     double au_new, al_new;
-    unsigned char st_u, st_l;
     PairPre pre;
+    int stop;             // the gap is closed, the step is not taken
     int flag_timeout;
 };
 
@@ -536,16 +569,16 @@ __device__ __forceinline__ void tgt_clear(typename RowMath<MODE>::Tgt &t)
 // with exact inner products, (m, b + te_off) as two ints in the double's
 // place (te_off = bias + t, so that a row entry's b - t plus it is the shift
 // k = b_x + b_z + bias)
+__device__ __forceinline__ double xd_entry(float v, bool xd, int tmin, int te_off)
+{
+    if (!xd) return widen_f32(v);
+    const uint32_t u = __float_as_uint(v);
+    return __hiloint2double(xd_exp(u, tmin) + te_off, xd_mant(u));
+}
 template <int SIDE>
 __device__ __forceinline__ void xd_put(double2 &t, float v, bool xd, int tmin, int te_off)
 {
-    double w;
-    if (xd) {
-        const uint32_t u = __float_as_uint(v);
-        w = __hiloint2double(xd_exp(u, tmin) + te_off, xd_mant(u));
-    } else {
-        w = (double)v;
-    }
+    const double w = xd_entry(v, xd, tmin, te_off);
     if (SIDE == 0) t.x = w;
     else t.y = w;
 }
@@ -741,6 +774,14 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
     // asynchronous stores whose bytes each CTA counts on its own mbarrier
     // (one per epoch parity; the CTA's own arrival sets the expected bytes)
     constexpr bool solo = SOLO;
+    // first-order rule: the stopping test (an FP64 subtraction) is evaluated
+    // beside the pair step instead of in the exchange, and a step of a closed
+    // gap is left before it changes anything
+    constexpr bool DEFER = !WSS;
+    // one cluster, first-order rule: the candidates' rows are read from the
+    // CTAs' shared memory (p0 of a side is then an offset in its owner's
+    // segment)
+    constexpr bool LEAN = SOLO && !WSS;
     if (tid == 0) {
         side_empty(sh.none[0], true);
         side_empty(sh.none[1], false);
@@ -759,6 +800,21 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
         cluster.sync();
     } else {
         __syncthreads();
+    }
+
+    if constexpr (LEAN) {
+        // a pair handed over from an earlier launch: its rows' owners
+        auto locate = [&](Side &sd) {
+            if (sd.i < 0 || sd.i >= A.n) { sd.i = INT_MAX; return; }
+            int o = (int)((int64_t)sd.i * G / A.n);
+            while (o + 1 < G && seg_lo(A.n, G, o + 1) <= sd.i) ++o;
+            sd.owner = o;
+            sd.p0 -= A.indptr[seg_lo(A.n, G, o)];
+        };
+        if (!first) {
+            locate(up);
+            locate(low);
+        }
     }
 
     // ---- accessors (segment-local row r, global sample lo + r)
@@ -847,7 +903,14 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
     const double snap = 1e-12 * C, c_snap = C - snap;
     const float gammaf = (float)A.gamma;
     unsigned epoch = 0;
-    int kc_pf0 = -1, kc_pf1 = -1;   // directory keeper: cache slots filled in the previous step
+    int kc_pf0 = -1, kc_pf1 = -1;   // cache slots filled in the previous step
+    const bool kc_direct = kc_on && A.kc_direct != 0;
+    // direct cache: this step's directory words, hits, and the epoch whose
+    // release covers K(up, low)
+    uint32_t kd_wu = 0, kd_wl = 0;
+    bool kd_hu = false, kd_hl = false;
+    unsigned kd_need = 0;
+    bool filled = false;   // this step filled its target buffer
     int exit_reason = 0;
     bool gap_open = first || dless(A.thr, low.f - up.f);   // stopping test of the pair in up / low
     int prev_valid = 0;              // buffer (1 - buf) holds the previous targets
@@ -871,49 +934,61 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
         const double bup_sel = up.f, blow_sel = WSS ? beta_low : low.f;   // values that chose this pair
         if (busy_on) cta_t0 = clock64();
         if (!first) {
-            if (!gap_open) { exit_reason = 0; break; }
-            if (iter >= A.iter_limit) { exit_reason = 1; break; }
-            if (total < A.compact_below) { exit_reason = 2; break; }
+            if constexpr (DEFER) {
+                // gap_open is known only with the pair step (below); a launch
+                // that ends for another reason tests it here first
+                if (up.i == INT_MAX || low.i == INT_MAX) { exit_reason = 0; break; }
+                if (iter >= A.iter_limit || total < A.compact_below) {
+                    exit_reason = !dless(A.thr, low.f - up.f) ? 0 : (iter >= A.iter_limit ? 1 : 2);
+                    break;
+                }
+            } else {
+                if (!gap_open) { exit_reason = 0; break; }
+                if (iter >= A.iter_limit) { exit_reason = 1; break; }
+                if (total < A.compact_below) { exit_reason = 2; break; }
+            }
             // ---- 0. kernel-row cache: this step's rows of x_up and x_low
             //         (the same decisions in every CTA; a row found here was
-            //         stored by this CTA in an earlier step of this launch)
-            // (by lane 0 of warp 1, which has no part in the target fill of
-            // short rows, so that the FP64 K(up, low) it reads from the cache
-            // arrives while the other threads fill the targets)
-            if (kc_on && tid == kKcThread) {
+            //         stored by this CTA in an earlier step of this launch).
+            //         Direct: every thread reads the two valid bits, which
+            //         thread 0 sets once all have read them (below)
+            if (kc_direct) {
+                kd_wu = kdir[up.i >> 5];
+                kd_wl = kdir[low.i >> 5];
+                kd_hu = (kd_wu >> (up.i & 31)) & 1u;
+                kd_hl = (kd_wl >> (low.i & 31)) & 1u;
+                kd_need = (kc_pf0 == up.i || kc_pf1 == up.i) ? epoch : epoch - 1u;
+                kc_pf0 = kd_hu ? -1 : up.i;
+                kc_pf1 = kd_hl ? -1 : low.i;
+            }
+            // 4-way sets: by lane 0 of warp 1, which has no part in the target
+            // fill of short rows, so that the FP64 K(up, low) it reads from the
+            // cache arrives while the other threads fill the targets
+            if (kc_on && !kc_direct && tid == kKcThread) {
                 auto lookup = [&](int i, int &slot, int &hit) {
-                    if (A.kc_direct) {
-                        const uint32_t bit = 1u << (i & 31);
-                        hit = (kdir[i >> 5] & bit) != 0;
-                        kdir[i >> 5] |= bit;
-                        slot = i;
-                    } else {
-                        const int nsets = A.kc_slots >> 2;
-                        const int set = i % nsets;
-                        uint32_t *tags = kdir + 4 * set, *stamps = kdir + A.kc_slots + 4 * set;
-                        int way = -1;
+                    const int nsets = A.kc_slots >> 2;
+                    const int set = i % nsets;
+                    uint32_t *tags = kdir + 4 * set, *stamps = kdir + A.kc_slots + 4 * set;
+                    int way = -1;
 #pragma unroll
-                        for (int w = 0; w < 4; ++w)
-                            if (tags[w] == (uint32_t)i) way = w;
-                        hit = way >= 0;
-                        if (!hit) {   // least recently used way
-                            way = 0;
+                    for (int w = 0; w < 4; ++w)
+                        if (tags[w] == (uint32_t)i) way = w;
+                    hit = way >= 0;
+                    if (!hit) {   // least recently used way
+                        way = 0;
 #pragma unroll
-                            for (int w = 1; w < 4; ++w)
-                                if (stamps[w] < stamps[way]) way = w;
-                            tags[way] = (uint32_t)i;
-                        }
-                        stamps[way] = (uint32_t)(iter + 1);
-                        slot = 4 * set + way;
+                        for (int w = 1; w < 4; ++w)
+                            if (stamps[w] < stamps[way]) way = w;
+                        tags[way] = (uint32_t)i;
                     }
+                    stamps[way] = (uint32_t)(iter + 1);
+                    slot = 4 * set + way;
                 };
                 int su_, hu_, sl_, hl_;
                 lookup(up.i, su_, hu_);
                 lookup(low.i, sl_, hl_);
                 sh.kc_su = su_; sh.kc_hu = hu_;
                 sh.kc_sl = sl_; sh.kc_hl = hl_;
-                kc_hits += hu_ + hl_;
-                kc_misses += 2 - hu_ - hl_;
                 if constexpr (MODE == MODE_FP64) {
                     if (hu_) {
                         // the entry was written by the CTA that owns x_low's
@@ -937,47 +1012,89 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                     kc_pf1 = hl_ ? -1 : sl_;
                 }
             }
-            // the pair step's part that K(up, low) does not enter, beside the
-            // target fill (rows of at most 224 entries leave this warp free)
-            if (warp == kPreWarp) {
-                const PairPre p = pair_pre<MODE == MODE_FP64>(up, low, C);
-                if (lane == 0) sh.pre = p;
-                if constexpr (BITS) pre_bar_arrive();
-            }
             // ---- 1. targets: x_up into .x / byte 0, x_low into .y / byte 1
             //         (bit-mask modes: the masks came with the exchange); x_up
             //         by the first half of the threads and x_low by the
             //         second, so that the loads of both rows are in flight
-            //         together (one round trip to L2, not two)
+            //         together. One cluster: from the shared memory of the
+            //         owners' CTAs (228 cycles a load, measured; an L2 hit
+            //         450), else from L2. FP64 rows that are both in the cache
+            //         need no targets: K(up, low) is an entry of x_up's row
+            //         (2,000 x 20 dense rows, of a step's 9,000 cycles 1,400
+            //         went by before the pair step could begin; with both
+            //         rows cached now fewer than 200).
+            const bool fill = !BITS && !(MODE == MODE_FP64 && !WSS && kd_hu && kd_hl);
             if constexpr (!BITS) {
-                constexpr int kHalf = kThreads / 2;
-                if (tid < kHalf) {
-                    for (int k = tid; k < up.len; k += kHalf) {
-                        int c = A.indices[up.p0 + k];
-                        tcu[k] = c;
-                        if constexpr (MODE == MODE_BINARY) reinterpret_cast<unsigned char *>(T + c)[0] = 1;
-                        else if constexpr (MODE == MODE_FP64) xd_put<0>(T[c], A.values[up.p0 + k], xd, xd_tmin, xd_te);
-                        else T[c].x = A.vmix[up.p0 + k];
+                if (fill) {
+                    constexpr int kHalf = kThreads / 2;
+                    const bool second = tid >= kHalf;
+                    const int len = second ? low.len : up.len;
+                    const int64_t p0 = second ? low.p0 : up.p0;
+                    int *tc = second ? tcl : tcu;
+                    uint32_t r_col = 0, r_val = 0;   // the owner CTA's entries (one cluster)
+                    if constexpr (LEAN) {
+                        const int own = second ? low.owner : up.owner;
+                        r_col = cluster_addr(smem_u32(col_s), own) + 2u * (uint32_t)p0;
+                        r_val = cluster_addr(smem_u32(val_s), own) + 4u * (uint32_t)p0;
                     }
-                } else {
-                    for (int k = tid - kHalf; k < low.len; k += kHalf) {
-                        int c = A.indices[low.p0 + k];
-                        tcl[k] = c;
-                        if constexpr (MODE == MODE_BINARY) reinterpret_cast<unsigned char *>(T + c)[1] = 1;
-                        else if constexpr (MODE == MODE_FP64) xd_put<1>(T[c], A.values[low.p0 + k], xd, xd_tmin, xd_te);
-                        else T[c].y = A.vmix[low.p0 + k];
+                    for (int k = second ? tid - kHalf : tid; k < len; k += kHalf) {
+                        int c;
+                        if constexpr (LEAN) {
+                            // (the entries of a row on chip: see COL, VAL and XCW)
+                            uint32_t w = 0;
+                            if constexpr (MODE != MODE_BINARY) w = ld_cluster_u32(r_val + 4u * (uint32_t)k);
+                            if constexpr (MODE == MODE_MIXED) c = (int)(w & 0xffffu);
+                            else c = (int)ld_cluster_u16(r_col + 2u * (uint32_t)k);
+                            if constexpr (MODE == MODE_BINARY) reinterpret_cast<unsigned char *>(T + c)[second] = 1;
+                            else if constexpr (MODE == MODE_MIXED)
+                                reinterpret_cast<float *>(T + c)[second] = __uint_as_float(w & 0xffff0000u);
+                            else
+                                reinterpret_cast<double *>(T + c)[second] =
+                                    xd ? __hiloint2double(xd_word_e(w) + xd_tmin + xd_te, xd_word_m(w))
+                                       : widen_f32(__uint_as_float(w));
+                        } else {
+                            c = A.indices[p0 + k];
+                            if constexpr (MODE == MODE_BINARY) reinterpret_cast<unsigned char *>(T + c)[second] = 1;
+                            else if constexpr (MODE == MODE_MIXED) reinterpret_cast<float *>(T + c)[second] = A.vmix[p0 + k];
+                            else reinterpret_cast<double *>(T + c)[second] = xd_entry(A.values[p0 + k], xd, xd_tmin, xd_te);
+                        }
+                        tc[k] = c;
                     }
+                    if (warp >= kPre0) fill_bar_arrive();
                 }
             }
+            // the pair step's part that K(up, low) does not enter
+            if (warp >= kPre0) {
+                pair_pre<MODE == MODE_FP64>(&sh.pre, warp - kPre0, lane, up, low, C);
+                pre_bar_arrive();
+            }
+            if (fill) {
+                if (warp >= kPre0) filled_sync();
+                else fill_bar_sync();
+                if (warp == 0) filled_arrive();
+            }
+            filled = fill;
             if (A.h > 0) {
                 counter -= 1;
                 shrink_now = counter <= 0;
             }
             row_visits += total;
-            if constexpr (!BITS) __syncthreads();
             if (timed) { uint64_t t = clock64(); ph[0] += t - tp; tp = t; }
         }
+        // this step's cache rows (both found: no row sums)
+        const bool kc_step = kc_on && !first;
+        const bool kc_hu = kc_step && (kc_direct ? kd_hu : sh.kc_hu != 0);
+        const bool kc_hl = kc_step && (kc_direct ? kd_hl : sh.kc_hl != 0);
+        bool stop = false;   // the gap is closed
 
+        // the pair's new alpha and index set, by the thread that updates its row
+        auto take_step = [&](int r, int i) -> uint8_t {
+            const double a = i == up.i ? sh.au_new : sh.al_new;
+            const uint8_t sb = status_of((i == up.i ? up.y : low.y) > 0, a, C);
+            PUTST(r, sb);
+            PUTA(r, a);
+            return sb;
+        };
         // ---- 2. the pair step (warp 0) runs while warps 1.. compute the
         //         row sums and kernel values; the f updates wait for it on a
         //         named barrier.
@@ -1003,8 +1120,22 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                     // the cache that entry is read instead (written by the
                     // owner of x_low's segment in an earlier step of this
                     // launch, visible here through the exchanges since)
-                    if (kc_on && sh.kc_hu) {
-                        kul_c = sh.kc_kul;
+                    if (kc_hu) {
+                        if (kc_direct) {
+                            // written by the CTA that owns x_low's row: see
+                            // the directory keeper above for the several
+                            // clusters' release it needs
+                            if constexpr (!SOLO) {
+                                unsigned seen = 0xffffffffu;
+                                if (lane > xwarps && lane < kWarps) seen = sh.rrel[lane];
+                                seen = __reduce_min_sync(0xffffffffu, seen);
+                                if (seen < kd_need)
+                                    wait_released(rel_flag(low.owner), kd_need, A.timeout_ns, &A.ctrl->err);
+                            }
+                            kul_c = __ldcg(static_cast<const double *>(A.kc) + (size_t)up.i * A.kc_ld + low.i);
+                        } else {
+                            kul_c = sh.kc_kul;
+                        }
                         kul_cached = true;
                     } else if (xd) {
                         // exact: the same value whatever the order or split,
@@ -1058,9 +1189,10 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                         const double q0 = slope * rinv;
                         const double r = fma(-eta, q0, slope);
                         q = fma(r, rinv, q0);
-                        if constexpr (BITS) pre_bar_sync();
+                        pre_bar_sync();
                         pre = sh.pre;
                     } else {
+                        pre_bar_sync();
                         pre = sh.pre;
                         if (A.kernel == KERNEL_RBF) {
                             if constexpr (MODE == MODE_FP64) {
@@ -1072,6 +1204,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                                 kul = widen_f32(__expf(-gammaf * fmaxf(d2, 0.f)));
                             }
                             eta = 2.0 - 2.0 * kul;   // K(x,x) = 1
+                            curved = bits_less(1e-12, eta);
+                            q = pair_quotient<true>(pre.slope, curved ? eta : 1.0);
                         } else {
                             // eta = K_uu + K_ll - 2 K_ul, K_uu from ||x_up||^2
                             double kuu, kll;
@@ -1086,9 +1220,14 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                                 kll = (double)kernel_of_dot(A.kernel, gammaf, c0, A.degree, norm_f32(low.nrm));
                             }
                             eta = __dsub_rn(__dadd_rn(kuu, kll), __dmul_rn(2.0, kul));
+                            curved = bits_less(1e-12, eta);
+                            q = pair_quotient<false>(pre.slope, curved ? eta : 1.0);
                         }
-                        curved = bits_less(1e-12, eta);
-                        q = div_int(pre.slope, curved ? eta : 1.0);
+                    }
+                    if constexpr (DEFER) {
+                        // Eq. (kktterm): f_low - f_up is the slope, up to its sign
+                        stop = !bits_less(A.thr, neg_if(pre.slope.x, low.y > 0));
+                        if (lane == 0) sh.stop = stop;
                     }
                     const PairStep ps = pair_solve(pre, up, low, curved, q, C, snap, c_snap);
                     if (lane == 0) {
@@ -1096,8 +1235,6 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                         sh.dl = ps.dl;
                         sh.au_new = ps.au;
                         sh.al_new = ps.al;
-                        sh.st_u = status_of(up.y > 0, ps.au, C);
-                        sh.st_l = status_of(low.y > 0, ps.al, C);
                     }
                 }
                 __syncwarp();
@@ -1134,21 +1271,55 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
             constexpr int kRowWarps = kWarps - 1;
             const int gl = lane & (LPR - 1);
             const int gw = lane / LPR;
-            // kernel-row cache rows of this step (both found: no row sums)
-            const bool kc_step = kc_on && !first;
-            const bool kc_hu = kc_step && sh.kc_hu, kc_hl = kc_step && sh.kc_hl;
-            KT *kc_ru = kc_step ? static_cast<KT *>(A.kc) + (size_t)sh.kc_su * A.kc_ld : nullptr;
-            KT *kc_rl = kc_step ? static_cast<KT *>(A.kc) + (size_t)sh.kc_sl * A.kc_ld : nullptr;
+            // the first row blocks go to the warps of the schedulers that the
+            // pair step's warp 0 does not use: its FP64 operations take 64
+            // cycles of their scheduler's pipe each, as theirs do
+            const int rw = (warp & 3) ? 3 * (warp >> 2) + (warp & 3) - 1 : 12 + (warp >> 2) - 1;
+            KT *kc_ru = kc_step ? static_cast<KT *>(A.kc) + (size_t)(kc_direct ? up.i : sh.kc_su) * A.kc_ld : nullptr;
+            KT *kc_rl = kc_step ? static_cast<KT *>(A.kc) + (size_t)(kc_direct ? low.i : sh.kc_sl) * A.kc_ld : nullptr;
             const bool skip_sums = kc_hu && kc_hl;
             const float up_nrmf = norm_f32(up.nrm), low_nrmf = norm_f32(low.nrm);   // mixed rows
             // streamed segment with no row shrunk: its active list is the
             // identity (lists are reset to it and compacted in order), so the
             // row index needs no load
             const bool ident = !RES && cnt == nseg;
-            double du = 0.0, dl = 0.0, au_new = 0.0, al_new = 0.0;
-            unsigned char st_u = 0, st_l = 0;
+            double du = 0.0, dl = 0.0;
             bool have_step = first;
             bool tiles_done = false;
+            // the step's results, once warp 0 has them
+            auto wait_step = [&]() {
+                if (have_step) return;
+                step_bar_sync(kThreads);
+                du = sh.du; dl = sh.dl;
+                if constexpr (DEFER) stop = sh.stop != 0;
+                have_step = true;
+            };
+            // Eq. (fup) for active-list position k (row r) from its kernel
+            // values, the pair's new alpha and index set, the shrink rule and
+            // this thread's candidates
+            auto finish_row = [&](int k, int r, double fi, uint8_t sb, double ku, double kl) {
+                const int i = (int)(lo + r);
+                if (!first) {
+                    // Eq. (fup), FP64 accumulation
+                    fi = fma(dl, kl, fma(du, ku, fi));
+                    PUTF(r, fi);
+                    if (i == up.i || i == low.i) sb = take_step(r, i);
+                }
+                const uint8_t set = set_bits(sb);
+                if (shrink_now) {
+                    // Eq. (shrink), with the thresholds that chose this pair
+                    if (((set == ST_I3 || set == ST_I4) && dless(fi, bup_sel)) ||
+                        ((set == ST_I1 || set == ST_I2) && dless(blow_sel, fi))) {
+                        SET_ACT(k, ~r);
+                        return;
+                    }
+                }
+                const unsigned long long kf = dkey(fi);
+                // a thread meets its rows in increasing index order: a
+                // strict key test keeps the lowest index of a tie
+                if (st_up(set) && kf < bku) { bku = kf; biu = i; bru = r; }
+                if (st_low(set) && ~kf < bkl) { bkl = ~kf; bil = i; brl = r; }
+            };
             if constexpr (MODE == MODE_MIXED && LPR == 16) {
                 if (A.dmat != nullptr && !kc_on) {
                     // Kernel rows on the tensor cores (mixed mode, RBF): tiles
@@ -1189,8 +1360,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                         }
                     }
                     rows_bar_sync();
-                    for (int base = (warp - 1) * 32;; base += kRowWarps * 32) {   // warp-uniform
-                        const bool round0 = base == (warp - 1) * 32;
+                    for (int base = rw * 32;; base += kRowWarps * 32) {   // warp-uniform
+                        const bool round0 = base == rw * 32;
                         if (!round0 && base >= cnt) break;
                         float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
                         if (!first) {
@@ -1244,50 +1415,100 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                                 kl = i == low.i ? 1.0 : widen_f32(__expf(-gammaf * fmaxf(low_nrmf + nrr - 2.0f * sl, 0.f)));
                             }
                         }
-                        if (!have_step) {
-                            step_bar_sync(kThreads);
-                            du = sh.du; dl = sh.dl;
-                            st_u = sh.st_u; st_l = sh.st_l;
-                            au_new = sh.au_new; al_new = sh.al_new;
-                            have_step = true;
-                        }
-                        if (valid) {
-                            const int i = (int)(lo + r);
-                            if (!first) {
-                                // Eq. (fup), FP64 accumulation
-                                fi = fma(dl, kl, fma(du, ku, fi));
-                                PUTF(r, fi);
-                                if (i == up.i) {
-                                    sb = st_u;
-                                    PUTST(r, sb);
-                                    PUTA(r, au_new);
-                                } else if (i == low.i) {
-                                    sb = st_l;
-                                    PUTST(r, sb);
-                                    PUTA(r, al_new);
-                                }
-                            }
-                            const uint8_t set = set_bits(sb);
-                            bool keep = true;
-                            if (shrink_now) {
-                                // Eq. (shrink), with the thresholds that chose this pair
-                                keep = !(((set == ST_I3 || set == ST_I4) && dless(fi, bup_sel)) ||
-                                         ((set == ST_I1 || set == ST_I2) && dless(blow_sel, fi)));
-                                if (!keep) SET_ACT(k, ~r);
-                            }
-                            if (keep) {
-                                const unsigned long long kup = key_up(fi), klo = key_low(fi);
-                                // a lane meets its rows in increasing index order
-                                if (st_up(set) && kup < bku) { bku = kup; biu = i; bru = r; }
-                                if (st_low(set) && klo < bkl) { bkl = klo; bil = i; brl = r; }
-                            }
-                        }
+                        wait_step();
+                        if (stop) break;
+                        if (valid) finish_row(k, r, fi, sb, ku, kl);
                     }
                 }
             }
+            // Rows on chip, at most one lane pair per row for the row warps:
+            // lane 2j takes x_up's kernel value of row j, lane 2j + 1 x_low's,
+            // so that the two inner products and exponentials of a row run
+            // side by side. Such small segments are bound by the length of
+            // one row's chain, not by issue (2,000 x 20 dense rows on one
+            // cluster, 125 rows a CTA, no row cached: from the pair step's end
+            // to the candidates 4,000 cycles with one lane a row, 2,600 with
+            // two). Each inner product keeps its order.
+            if constexpr (RES && LPR == 1 && (MODE == MODE_FP64 || MODE == MODE_MIXED)) {
+                if (!tiles_done && cnt <= kRowWarps * 16) {
+                    tiles_done = true;
+                    const int side = lane & 1, k = rw * 16 + (lane >> 1);
+                    const bool valid = k < cnt;
+                    int r = 0;
+                    double fi = 0.0, kv = 0.0;
+                    float kvf = 0.f;
+                    uint8_t sb = 0;
+                    if (valid) {
+                        r = ACT(k);
+                        fi = GETF(r);
+                        sb = GETST(r);
+                    }
+                    if (valid && !first) {
+                        KT *const kr = side ? kc_rl : kc_ru;
+                        const int64_t gi = lo + r;
+                        if (side ? kc_hl : kc_hu) {
+                            if constexpr (MODE == MODE_FP64) kv = kr[gi];
+                            else kvf = kr[gi];
+                        } else {
+                            int64_t p0, p1;
+                            ROWP(r, p0, p1);
+                            if constexpr (MODE == MODE_FP64) {
+                                double dot = 0.0;
+                                if (xd) {
+                                    const int2 *T2 = reinterpret_cast<const int2 *>(T) + side;
+                                    XdAcc a = xd_zero(), a2 = xd_zero();   // two chains of carries
+                                    constexpr int XB = 4;
+                                    for (int pb = (int)p0; pb < (int)p1; pb += XB) {
+                                        int cb[XB];
+                                        uint32_t ub[XB];
+#pragma unroll
+                                        for (int j = 0; j < XB; ++j) {
+                                            cb[j] = 0;
+                                            ub[j] = 0u;
+                                            if (pb + j < (int)p1) XCW(pb + j, cb[j], ub[j]);
+                                        }
+                                        int2 t[XB];
+#pragma unroll
+                                        for (int j = 0; j < XB; ++j) t[j] = T2[2 * cb[j]];
+#pragma unroll
+                                        for (int j = 0; j < XB; ++j)   // (past the row's end m is 0)
+                                            xd_add(j & 1 ? a2 : a, xd_word_m(ub[j]), t[j].x, xd_word_e(ub[j]) + t[j].y);
+                                    }
+                                    xd_add(a, a2);
+                                    dot = xd_round(a, xd_unit);
+                                } else {
+                                    const double *Td = reinterpret_cast<const double *>(T) + side;
+                                    for (int64_t p = p0; p < p1; ++p) dot = fma(widen_f32(VAL(p)), Td[2 * COL(p)], dot);
+                                }
+                                if (A.kernel != KERNEL_RBF) {
+                                    kv = kernel_of_dot(A.kernel, A.gamma, A.coef0, A.degree, dot);
+                                } else {
+                                    const double d2 = (side ? low.nrm : up.nrm) + NRM(r) - 2.0 * dot;
+                                    kv = exp_neg_fx(A.gamma * dpos(d2), expfx_s);
+                                }
+                                if (kc_step) kr[gi] = kv;
+                            } else {
+                                const float *Tf = reinterpret_cast<const float *>(T) + side;
+                                float dot = 0.f;
+                                for (int64_t p = p0; p < p1; ++p) dot = fmaf(VAL(p), Tf[2 * COL(p)], dot);
+                                if (A.kernel != KERNEL_RBF)
+                                    kvf = kernel_of_dot(A.kernel, gammaf, (float)A.coef0, A.degree, dot);
+                                else
+                                    kvf = __expf(-gammaf * fmaxf((side ? low_nrmf : up_nrmf) + NRMF(r) - 2.0f * dot, 0.f));
+                                if (kc_step) kr[gi] = kvf;
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    if constexpr (MODE == MODE_MIXED) kv = widen_f32(kvf);
+                    const double kl = __shfl_down_sync(0xffffffffu, kv, 1);
+                    wait_step();
+                    if (valid && side == 0 && !stop) finish_row(k, r, fi, sb, kv, kl);
+                }
+            }
             if (!tiles_done)
-            for (int kb = (warp - 1) * RPW;; kb += kRowWarps * RPW) {
-                const bool round0 = kb == (warp - 1) * RPW;
+            for (int kb = rw * RPW;; kb += kRowWarps * RPW) {
+                const bool round0 = kb == rw * RPW;
                 if (!round0 && kb >= cnt) break;
                 const int k = kb + gw;
                 const bool valid = k < cnt;
@@ -1314,33 +1535,58 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                         // exact inner products in integer arithmetic, each
                         // lane loading its next XB entries at once (4: fewer
                         // live registers than 8, measured 3% faster)
-                        const int4 *T4 = reinterpret_cast<const int4 *>(T);
-                        XdAcc au = xd_zero(), al = xd_zero();
                         constexpr int XB = 4;
-                        for (int64_t pb = p0 + gl; pb < p1; pb += XB * LPR) {
-                            int cb[XB];
-                            uint32_t ub[XB];
+                        if (!kc_hu && !kc_hl) {
+                            const int4 *T4 = reinterpret_cast<const int4 *>(T);
+                            XdAcc au = xd_zero(), al = xd_zero();
+                            for (int64_t pb = p0 + gl; pb < p1; pb += XB * LPR) {
+                                int cb[XB];
+                                uint32_t ub[XB];
 #pragma unroll
-                            for (int j = 0; j < XB; ++j) {
-                                const int64_t p = pb + (int64_t)j * LPR;
-                                cb[j] = 0;
-                                ub[j] = 0u;
-                                if (p < p1) XCW(p, cb[j], ub[j]);
-                            }
+                                for (int j = 0; j < XB; ++j) {
+                                    const int64_t p = pb + (int64_t)j * LPR;
+                                    cb[j] = 0;
+                                    ub[j] = 0u;
+                                    if (p < p1) XCW(p, cb[j], ub[j]);
+                                }
 #pragma unroll
-                            for (int j = 0; j < XB; ++j) {
-                                if (pb + (int64_t)j * LPR >= p1) break;
-                                const int32_t m = xd_word_m(ub[j]);
-                                const int e = xd_word_e(ub[j]);
-                                const int4 t = T4[cb[j]];
-                                xd_add(au, m, t.x, e + t.y);
-                                xd_add(al, m, t.z, e + t.w);
+                                for (int j = 0; j < XB; ++j) {
+                                    if (pb + (int64_t)j * LPR >= p1) break;
+                                    const int32_t m = xd_word_m(ub[j]);
+                                    const int e = xd_word_e(ub[j]);
+                                    const int4 t = T4[cb[j]];
+                                    xd_add(au, m, t.x, e + t.y);
+                                    xd_add(al, m, t.z, e + t.w);
+                                }
                             }
+                            xd_lane_sum<LPR>(au);
+                            xd_lane_sum<LPR>(al);
+                            su = xd_round(au, xd_unit);
+                            sl = xd_round(al, xd_unit);
+                        } else {
+                            // the other side's row is in the cache
+                            const int2 *T2 = reinterpret_cast<const int2 *>(T) + (kc_hu ? 1 : 0);
+                            XdAcc a = xd_zero();
+                            for (int64_t pb = p0 + gl; pb < p1; pb += XB * LPR) {
+                                int cb[XB];
+                                uint32_t ub[XB];
+#pragma unroll
+                                for (int j = 0; j < XB; ++j) {
+                                    const int64_t p = pb + (int64_t)j * LPR;
+                                    cb[j] = 0;
+                                    ub[j] = 0u;
+                                    if (p < p1) XCW(p, cb[j], ub[j]);
+                                }
+#pragma unroll
+                                for (int j = 0; j < XB; ++j) {
+                                    if (pb + (int64_t)j * LPR >= p1) break;
+                                    const int2 t = T2[2 * cb[j]];
+                                    xd_add(a, xd_word_m(ub[j]), t.x, xd_word_e(ub[j]) + t.y);
+                                }
+                            }
+                            xd_lane_sum<LPR>(a);
+                            su = sl = xd_round(a, xd_unit);
                         }
-                        xd_lane_sum<LPR>(au);
-                        xd_lane_sum<LPR>(al);
-                        su = xd_round(au, xd_unit);
-                        sl = xd_round(al, xd_unit);
                     }
                 } else if constexpr (BITS) {
                     // squared distances to x_up and x_low (one lane per row)
@@ -1494,52 +1740,18 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                         }
                     }
                 }
-                if (!have_step) {
-                    step_bar_sync(kThreads);
-                    du = sh.du; dl = sh.dl;
-                    st_u = sh.st_u; st_l = sh.st_l;
-                    au_new = sh.au_new; al_new = sh.al_new;
-                    have_step = true;
-                }
-                if (valid && gl == 0) {
-                    const int i = (int)(lo + r);
-                    if (!first) {
-                        // Eq. (fup), FP64 accumulation
-                        fi = fma(dl, kl, fma(du, ku, fi));
-                        PUTF(r, fi);
-                        if (i == up.i) {
-                            sb = st_u;
-                            PUTST(r, sb);
-                            PUTA(r, au_new);
-                        } else if (i == low.i) {
-                            sb = st_l;
-                            PUTST(r, sb);
-                            PUTA(r, al_new);
-                        }
-                    }
-                    const uint8_t set = set_bits(sb);
-                    bool keep = true;
-                    if (shrink_now) {
-                        // Eq. (shrink), with the thresholds that chose this pair
-                        keep = !(((set == ST_I3 || set == ST_I4) && dless(fi, bup_sel)) ||
-                                 ((set == ST_I1 || set == ST_I2) && dless(blow_sel, fi)));
-                        if (!keep) SET_ACT(k, ~r);
-                    }
-                    if (keep) {
-                        const unsigned long long kup = key_up(fi), klo = key_low(fi);
-                        // a thread meets its rows in increasing index order:
-                        // a strict key test keeps the lowest index of a tie
-                        if (st_up(set) && kup < bku) { bku = kup; biu = i; bru = r; }
-                        if (st_low(set) && klo < bkl) { bkl = klo; bil = i; brl = r; }
-                    }
-                }
+                wait_step();
+                if (stop) break;
+                if (valid && gl == 0) finish_row(k, r, fi, sb, ku, kl);
             }
         }
         if constexpr (BITS && RES) {
             // second sweep, all warps: f updates, shrink rule, candidates
-            const double du = sh.du, dl = sh.dl, au_new = sh.au_new, al_new = sh.al_new;
-            const unsigned char st_u = sh.st_u, st_l = sh.st_l;
-            for (int k = tid; k < cnt; k += kThreads) {
+            const double du = sh.du, dl = sh.dl;
+            if constexpr (DEFER) {
+                if (!first) stop = sh.stop != 0;
+            }
+            for (int k = tid; k < cnt && !stop; k += kThreads) {
                 const int r = act_s[k];
                 const int i = (int)(lo + r);
                 double fi = f_s[r];
@@ -1548,15 +1760,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                     const uint32_t dd = dist_s[k];
                     fi = fma(dl, ktab[dd >> 16], fma(du, ktab[dd & 0xffffu], fi));
                     f_s[r] = fi;
-                    if (i == up.i) {
-                        sb = st_u;
-                        st_s[r] = sb;
-                        a_s[r] = au_new;
-                    } else if (i == low.i) {
-                        sb = st_l;
-                        st_s[r] = sb;
-                        a_s[r] = al_new;
-                    }
+                    if (i == up.i || i == low.i) sb = take_step(r, i);
                 }
                 const uint8_t set = set_bits(sb);
                 bool keep = true;
@@ -1566,11 +1770,20 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                     if (!keep) act_s[k] = ~r;
                 }
                 if (keep) {
-                    const unsigned long long kup = key_up(fi), klo = key_low(fi);
+                    const unsigned long long kf = dkey(fi);
                     // increasing index order per thread: strict key test
-                    if (st_up(set) && kup < bku) { bku = kup; biu = i; bru = r; }
-                    if (st_low(set) && klo < bkl) { bkl = klo; bil = i; brl = r; }
+                    if (st_up(set) && kf < bku) { bku = kf; biu = i; bru = r; }
+                    if (st_low(set) && ~kf < bkl) { bkl = ~kf; bil = i; brl = r; }
                 }
+            }
+        }
+        if constexpr (DEFER) {
+            // every CTA sees the same pair: all leave here
+            if (stop) {
+                if (A.h > 0) counter += 1;
+                row_visits -= total;
+                exit_reason = 0;
+                break;
             }
         }
         // payload of a segment row for the exchange (read after this
@@ -1614,15 +1827,26 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                 sh.wkup[warp] = k1; sh.wiup[warp] = i1;
                 sh.wklow[warp] = k2; sh.wilow[warp] = i2;
             }
-            if (i1 != INT_MAX && iu_ == i1) {
-                Side sd = make_side(ru_);
-                if (gx) sd.f = gneg;
-                sh.wup[warp] = sd;
+            // one cluster: the sending warp reads the winners' rows itself
+            if constexpr (!LEAN) {
+                if (i1 != INT_MAX && iu_ == i1) {
+                    Side sd = make_side(ru_);
+                    if (gx) sd.f = gneg;
+                    sh.wup[warp] = sd;
+                }
+                if (i2 != INT_MAX && il_ == i2) sh.wlow[warp] = make_side(rl_);
             }
-            if (i2 != INT_MAX && il_ == i2) sh.wlow[warp] = make_side(rl_);
             __syncthreads();
         };
         cta_reduce(false, bku, biu, bru, bkl, bil, brl, 0.0);
+        // direct cache: both rows are stored from here on (all threads have
+        // read this step's bits; the exchange orders the next step's reads)
+        if (kc_direct && !first && tid == 0) {
+            const uint32_t bu = 1u << (up.i & 31), bl = 1u << (low.i & 31);
+            const bool same = (up.i >> 5) == (low.i >> 5);
+            kdir[up.i >> 5] = kd_wu | bu | (same ? bl : 0u);
+            if (!same) kdir[low.i >> 5] = kd_wl | bl;
+        }
         // ---- 5. compaction of the active list on shrink steps
         if (shrink_now) {
             int kept = 0;
@@ -1662,20 +1886,64 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                 unsigned long long k2 = lane < kWarps ? sh.wklow[lane] : kNoKey;
                 int i1 = lane < kWarps ? sh.wiup[lane] : INT_MAX;
                 int i2 = lane < kWarps ? sh.wilow[lane] : INT_MAX;
-                const unsigned long long k1s = k1, k2s = k2;
                 const int i1s = i1, i2s = i2;
                 warp_min_ki(k1, i1);
                 warp_min_ki(k2, i2);
-                const unsigned mu = __ballot_sync(0xffffffffu, i1 != INT_MAX && k1s == k1 && i1s == i1);
-                const unsigned ml = __ballot_sync(0xffffffffu, i2 != INT_MAX && k2s == k2 && i2s == i2);
-                if constexpr (solo) {
+                // the warps that hold them (an index occurs once)
+                int w1 = 0, w2 = 0;
+                if constexpr (!LEAN) {
+                    w1 = __ffs(__ballot_sync(0xffffffffu, i1s == i1)) - 1;
+                    w2 = __ffs(__ballot_sync(0xffffffffu, i2s == i2)) - 1;
+                }
+                if constexpr (LEAN) {
+                    // lanes q and 16 + q send the I_up and I_low sides of the
+                    // CTA's candidate to CTA q, read from the segment's arrays
+                    // (the first 48 bytes and the mask, the active count in
+                    // the owner's place)
+                    const bool side_low = lane >= 16;
+                    const int q = lane & 15, wi = side_low ? i2 : i1;
+                    double sf = __longlong_as_double(side_low ? 0xfff0000000000000ll : 0x7ff0000000000000ll);
+                    double sa = 0.0, snrm = 0.0;
+                    int sp0 = 0, slen = 0, sy = 0;
+                    uint4 mask[W4];
+#pragma unroll
+                    for (int w = 0; w < W4; ++w) mask[w] = make_uint4(0, 0, 0, 0);
+                    if (wi != INT_MAX) {
+                        const int r = wi - (int)lo;
+                        sf = f_s[r];
+                        sa = a_s[r];
+                        sy = y_of(st_s[r]);
+                        if constexpr (MODE == MODE_MIXED) snrm = norm_bits(NRMF(r));
+                        else if constexpr (MODE == MODE_FP64) snrm = nrm_s[r];
+                        if constexpr (BITS) {
+#pragma unroll
+                            for (int w = 0; w < W4; ++w) mask[w] = bits_s[(size_t)r * W4 + w];
+                        } else {
+                            sp0 = rp_s[r];
+                            slen = rp_s[r + 1] - sp0;
+                        }
+                    }
+                    if (q < csize) {
+                        const uint32_t dst = cluster_addr(smem_u32(side_low ? &sh.xc[par][crank].low : &sh.xc[par][crank].up), q);
+                        const uint32_t rbar = cluster_addr(smem_u32(&sh.xbar[par]), q);
+                        st_async_v4(dst, make_uint4(__double2loint(sf), __double2hiint(sf), __double2loint(sa), __double2hiint(sa)), rbar);
+                        st_async_v4(dst + 16, make_uint4(__double2loint(snrm), __double2hiint(snrm), (unsigned)sp0, 0u), rbar);
+                        st_async_v4(dst + 32, make_uint4((unsigned)wi, (unsigned)slen, (unsigned)sy, (unsigned)cnt), rbar);
+                        if constexpr (BITS) {
+#pragma unroll
+                            for (int w = 0; w < W4; ++w) st_async_v4(dst + 48 + 16 * w, mask[w], rbar);
+                        }
+                    }
+                    if (lane == 0)
+                        mbar_arrive_expect_tx(smem_u32(&sh.xbar[par]), (uint32_t)(csize * 2 * (48 + (BITS ? 16 * W4 : 0))));
+                } else if constexpr (solo) {
                     // lane q sends the CTA's candidate to CTA q: the winning
                     // warps' sides straight from shared memory, then the count
                     if (lane < csize) {
                         const uint32_t dst = cluster_addr(smem_u32(&sh.xc[par][crank]), lane);
                         const uint32_t rbar = cluster_addr(smem_u32(&sh.xbar[par]), lane);
-                        const uint4 *su = reinterpret_cast<const uint4 *>(mu ? &sh.wup[__ffs(mu) - 1] : &sh.none[0]);
-                        const uint4 *sl = reinterpret_cast<const uint4 *>(ml ? &sh.wlow[__ffs(ml) - 1] : &sh.none[1]);
+                        const uint4 *su = reinterpret_cast<const uint4 *>(i1 != INT_MAX ? &sh.wup[w1] : &sh.none[0]);
+                        const uint4 *sl = reinterpret_cast<const uint4 *>(i2 != INT_MAX ? &sh.wlow[w2] : &sh.none[1]);
                         constexpr int kSideV = (int)(sizeof(Side) / 16);
 #pragma unroll
                         for (int j = 0; j < kSideV; ++j) st_async_v4(dst + 16 * j, su[j], rbar);
@@ -1685,14 +1953,17 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                     }
                     if (lane == 0)
                         mbar_arrive_expect_tx(smem_u32(&sh.xbar[par]), (uint32_t)(csize * sizeof(CandFull)));
-                } else if (lane == 0) {
-                    CandFull cf;
-                    if (mu) cf.up = sh.wup[__ffs(mu) - 1]; else side_empty(cf.up, true);
-                    if (ml) cf.low = sh.wlow[__ffs(ml) - 1]; else side_empty(cf.low, false);
-                    cf.count = cnt;
-                    cf.pad[0] = cf.pad[1] = cf.pad[2] = 0;
-                    CandFull *dst = cluster.map_shared_rank(sh.ccand, 0);
-                    dst[crank] = cf;
+                } else {
+                    // one 8-byte word of the winning sides and the count per lane
+                    constexpr int kSideW = (int)(sizeof(Side) / 8);
+                    const bool u = lane < kSideW;
+                    const int w = u ? lane : lane - kSideW;
+                    const Side *sd = u ? (i1 != INT_MAX ? &sh.wup[w1] : &sh.none[0])
+                                       : (i2 != INT_MAX ? &sh.wlow[w2] : &sh.none[1]);
+                    unsigned long long *dst =
+                        reinterpret_cast<unsigned long long *>(cluster.map_shared_rank(sh.ccand, 0) + crank);
+                    if (lane < 2 * kSideW) dst[lane] = reinterpret_cast<const unsigned long long *>(sd)[w];
+                    else if (lane == 2 * kSideW) dst[lane] = (unsigned)cnt;   // count and padding
                 }
                 // (clocks are read by whole warps: a lane apart would run the
                 // collectives that follow one lane at a time)
@@ -1719,31 +1990,35 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                     unsigned long long k1 = kNoKey, k2 = kNoKey;
                     int i1 = INT_MAX, i2 = INT_MAX;
                     long long cc = 0;
-                    if (lane < csize && !timed_out) cand_keys(sh.xc[par][lane], k1, i1, k2, i2, cc);
+                    if (lane < csize && !timed_out) {
+                        cand_keys(sh.xc[par][lane], k1, i1, k2, i2, cc);
+                        if constexpr (LEAN) cc = sh.xc[par][lane].up.owner;
+                    }
                     if (gx) { k2 = k1; i2 = i1; }   // the gain winner's row on both sides
-                    const unsigned long long k1s = k1, k2s = k2;
                     const int i1s = i1, i2s = i2;
+                    const unsigned tot = __reduce_add_sync(0xffffffffu, (unsigned)cc);
                     warp_min_ki(k1, i1);
                     warp_min_ki(k2, i2);
-#pragma unroll
-                    for (int off = 16; off >= 1; off >>= 1) cc += __shfl_xor_sync(0xffffffffu, cc, off);
-                    const unsigned mu = __ballot_sync(0xffffffffu, i1 != INT_MAX && k1s == k1 && i1s == i1);
-                    const unsigned ml = __ballot_sync(0xffffffffu, i2 != INT_MAX && k2s == k2 && i2s == i2);
+                    // the CTAs that hold them (an index occurs once; without
+                    // any candidate lane 0, whose side is the empty one)
+                    const int w1 = __ffs(__ballot_sync(0xffffffffu, i1s == i1)) - 1;
+                    const int w2 = __ffs(__ballot_sync(0xffffffffu, i2s == i2)) - 1;
                     // the winning sides into the result, one 8-byte word per lane
-                    const Side *wsu = mu ? &sh.xc[par][__ffs(mu) - 1].up : &sh.none[0];
-                    const Side *wsl = ml ? &sh.xc[par][__ffs(ml) - 1].low : &sh.none[1];
                     constexpr int kSideW = (int)(sizeof(Side) / 8);
                     static_assert(2 * kSideW <= 32, "a side is copied by one warp");
                     if (lane < 2 * kSideW) {
                         const bool u = lane < kSideW;
                         const int w = u ? lane : lane - kSideW;
-                        reinterpret_cast<unsigned long long *>(u ? &sh.res.up : &sh.res.low)[w] =
-                            reinterpret_cast<const unsigned long long *>(u ? wsu : wsl)[w];
+                        unsigned long long v = reinterpret_cast<const unsigned long long *>(
+                            u ? &sh.xc[par][w1].up : &sh.xc[par][w2].low)[w];
+                        // the owner: the CTA whose candidate won (word 5 is (y, owner))
+                        if (LEAN && w == 5) v = (unsigned)v | ((unsigned long long)(unsigned)(u ? w1 : w2) << 32);
+                        reinterpret_cast<unsigned long long *>(u ? &sh.res.up : &sh.res.low)[w] = v;
                     }
                     if (lane == 0) {
-                        sh.res.total = cc;
+                        sh.res.total = tot;
                         sh.res.flag = timed_out;
-                        sh.res.gap_open = dless(A.thr, wsl->f - wsu->f);
+                        if constexpr (!DEFER) sh.res.gap_open = dless(A.thr, sh.xc[par][w2].low.f - sh.xc[par][w1].up.f);
                     }
                 }
                 __syncthreads();
@@ -1772,30 +2047,28 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                         long long cc = 0;
                         if (lane < csize) cand_keys(sh.ccand[lane], k1, i1, k2, i2, cc);
                         if (gx) { k2 = k1; i2 = i1; }
-                        const unsigned long long k1s = k1, k2s = k2;
                         const int i1s = i1, i2s = i2;
+                        cc = (long long)__reduce_add_sync(0xffffffffu, (unsigned)cc);
                         warp_min_ki(k1, i1);
                         warp_min_ki(k2, i2);
-#pragma unroll
-                        for (int off = 16; off >= 1; off >>= 1) cc += __shfl_xor_sync(0xffffffffu, cc, off);
-                        const unsigned mu = __ballot_sync(0xffffffffu, i1 != INT_MAX && k1s == k1 && i1s == i1);
-                        const unsigned ml = __ballot_sync(0xffffffffu, i2 != INT_MAX && k2s == k2 && i2s == i2);
+                        // the CTAs that hold them (without any candidate lane
+                        // 0, whose side is the empty one)
+                        const int w1 = __ffs(__ballot_sync(0xffffffffu, i1s == i1)) - 1;
+                        const int w2 = __ffs(__ballot_sync(0xffffffffu, i2s == i2)) - 1;
                         if (!tagged) {
                             if (lane == 0) {
                                 CandFull *out = reinterpret_cast<CandFull *>(static_cast<unsigned char *>(A.cand) +
                                                                              ((size_t)par * nlead + cid) * kCandStride);
-                                if (mu) copy_side(&out->up, &sh.ccand[__ffs(mu) - 1].up);
-                                else { Side e; side_empty(e, true); copy_side(&out->up, &e); }
-                                if (ml) copy_side(&out->low, &sh.ccand[__ffs(ml) - 1].low);
-                                else { Side e; side_empty(e, false); copy_side(&out->low, &e); }
+                                copy_side(&out->up, &sh.ccand[w1].up);
+                                copy_side(&out->low, &sh.ccand[w2].low);
                                 out->count = (int32_t)cc;
                                 st_release_u32(A.seq + ((size_t)par * nlead + cid) * kSeqStride, epoch);
                             }
                         } else if (lane < kTagPairs) {
                             // the first 48 bytes of both winning sides and the
                             // count, as tagged words (lane j: words 2j, 2j + 1)
-                            const uint32_t *wsu = reinterpret_cast<const uint32_t *>(mu ? &sh.ccand[__ffs(mu) - 1].up : &sh.none[0]);
-                            const uint32_t *wsl = reinterpret_cast<const uint32_t *>(ml ? &sh.ccand[__ffs(ml) - 1].low : &sh.none[1]);
+                            const uint32_t *wsu = reinterpret_cast<const uint32_t *>(&sh.ccand[w1].up);
+                            const uint32_t *wsl = reinterpret_cast<const uint32_t *>(&sh.ccand[w2].low);
                             auto word = [&](int q) -> uint32_t {
                                 return q < 12 ? wsu[q] : (q < 24 ? wsl[q - 12] : (q == 24 ? (uint32_t)cc : 0u));
                             };
@@ -1882,32 +2155,26 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                         unsigned long long k2 = bi == INT_MAX ? kNoKey : key_low(bf);
                         int i1 = ai, i2 = bi;
                         if (gx) { k2 = k1; i2 = i1; }
-                        warp_min_ki(k1, i1);
-                        warp_min_ki(k2, i2);
-#pragma unroll
-                        for (int off = 16; off >= 1; off >>= 1) cc += __shfl_xor_sync(0xffffffffu, cc, off);
+                        cc = (long long)__reduce_add_sync(0xffffffffu, (unsigned)cc);
                         if (tagged) {
                             // one warp holds every leader's candidate: the
                             // winning sides go from their lanes straight into
                             // the result area of every CTA of the cluster
-                            // (lane q writes CTA q's)
-                            const unsigned mu = __ballot_sync(0xffffffffu, i1 != INT_MAX && ai == i1);
-                            const unsigned ml = __ballot_sync(0xffffffffu, i2 != INT_MAX && bi == i2);
-                            const int su = mu ? __ffs(mu) - 1 : 0, sl = ml ? __ffs(ml) - 1 : 0;
-                            uint4 ru[3] = {shfl_u4(wu0, su), shfl_u4(wu1, su), shfl_u4(wu2, su)};
-                            uint4 rl[3] = {shfl_u4(wl0, sl), shfl_u4(wl1, sl), shfl_u4(wl2, sl)};
-                            if (!mu) {
-                                const uint4 *e = reinterpret_cast<const uint4 *>(&sh.none[0]);
-                                ru[0] = e[0]; ru[1] = e[1]; ru[2] = e[2];
+                            // (lane q writes CTA q's); without any candidate
+                            // lane 0 wins, whose sides are the empty ones
+                            warp_min_ki(k1, i1);
+                            warp_min_ki(k2, i2);
+                            const int su = __ffs(__ballot_sync(0xffffffffu, ai == i1)) - 1;
+                            const int sl = __ffs(__ballot_sync(0xffffffffu, bi == i2)) - 1;
+                            const uint4 ru[3] = {shfl_u4(wu0, su), shfl_u4(wu1, su), shfl_u4(wu2, su)};
+                            const uint4 rl[3] = {shfl_u4(wl0, sl), shfl_u4(wl1, sl), shfl_u4(wl2, sl)};
+                            unsigned open = 1;
+                            if constexpr (!DEFER) {
+                                const double fu = __hiloint2double((int)ru[0].y, (int)ru[0].x);
+                                const double fl = __hiloint2double((int)rl[0].y, (int)rl[0].x);
+                                open = dless(A.thr, fl - fu);
                             }
-                            if (!ml) {
-                                const uint4 *e = reinterpret_cast<const uint4 *>(&sh.none[1]);
-                                rl[0] = e[0]; rl[1] = e[1]; rl[2] = e[2];
-                            }
-                            const double fu = __hiloint2double((int)ru[0].y, (int)ru[0].x);
-                            const double fl = __hiloint2double((int)rl[0].y, (int)rl[0].x);
-                            const uint4 tail = make_uint4((unsigned)(unsigned long long)cc, (unsigned)((unsigned long long)cc >> 32),
-                                                          (unsigned)any_to, (unsigned)dless(A.thr, fl - fu));
+                            const uint4 tail = make_uint4((unsigned)cc, 0u, (unsigned)any_to, open);
                             if (lane < csize) {
                                 uint4 *o = reinterpret_cast<uint4 *>(cluster.map_shared_rank(&sh.res, lane));
                                 o[0] = ru[0]; o[1] = ru[1]; o[2] = ru[2];
@@ -1915,6 +2182,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                                 o[10] = tail;
                             }
                         } else {
+                            warp_min_ki(k1, i1);
+                            warp_min_ki(k2, i2);
                             if (lane == 0) {
                                 sh.rkup[warp] = k1; sh.riup[warp] = i1;
                                 sh.rklow[warp] = k2; sh.rilow[warp] = i2;
@@ -1957,7 +2226,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                                 if (il != INT_MAX) copy_side(&sh.res.low, &sh.rlow[wl]); else side_empty(sh.res.low, false);
                                 sh.res.total = cc;
                                 sh.res.flag = to;
-                                sh.res.gap_open = dless(A.thr, sh.res.low.f - sh.res.up.f);
+                                if constexpr (!DEFER) sh.res.gap_open = dless(A.thr, sh.res.low.f - sh.res.up.f);
                             }
                             __syncwarp();
                             if (lane > 0 && lane < csize) copy_result(cluster.map_shared_rank(&sh.res, lane), &sh.res);
@@ -1969,15 +2238,20 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
         };
         exchange(false);
         if (timed) { uint64_t t = clock64(); ph[4] += t - tp; tp = t; }
-        if (sh.res.flag) break;
-        prev_valid = first ? 0 : 1;
+        prev_valid = filled ? 1 : 0;
         prev_len_u = up.len;
         prev_len_l = low.len;
+        if (sh.res.flag) break;
         up = sh.res.up;
         low = sh.res.low;
         total = sh.res.total;
-        gap_open = sh.res.gap_open != 0;
+        if constexpr (!DEFER) gap_open = sh.res.gap_open != 0;
         if (!first) {
+            if (kc_on) {
+                const int hits = kc_direct ? (int)kd_hu + (int)kd_hl : (tid == kKcThread ? sh.kc_hu + sh.kc_hl : 0);
+                kc_hits += hits;
+                kc_misses += 2 - hits;
+            }
             ++iter;
             if (shrink_now) {
                 counter = A.h < total ? A.h : total;

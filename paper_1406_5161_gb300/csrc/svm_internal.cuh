@@ -31,8 +31,9 @@ enum { KERNEL_RBF = 0, KERNEL_LINEAR = 1, KERNEL_POLY = 2, KERNEL_SIGMOID = 3 };
 
 // linear <x,z>, polynomial (gamma <x,z> + coef0)^degree (power by repeated
 // products), sigmoid tanh(gamma <x,z> + coef0); each FP64 operation rounded
-// on its own, in this order
-__device__ __forceinline__ double kernel_of_dot(int kind, double gamma, double coef0, int degree, double dot)
+// on its own, in this order. Out of line: inlined they (the power, tanh) took
+// several times the code of the RBF path that the steps run through.
+static __device__ __noinline__ double kernel_of_dot(int kind, double gamma, double coef0, int degree, double dot)
 {
     if (kind == KERNEL_LINEAR) return dot;
     const double b = __dadd_rn(__dmul_rn(gamma, dot), coef0);
@@ -43,7 +44,7 @@ __device__ __forceinline__ double kernel_of_dot(int kind, double gamma, double c
     }
     return tanh(b);
 }
-__device__ __forceinline__ float kernel_of_dot(int kind, float gamma, float coef0, int degree, float dot)
+static __device__ __noinline__ float kernel_of_dot(int kind, float gamma, float coef0, int degree, float dot)
 {
     if (kind == KERNEL_LINEAR) return dot;
     const float b = __fadd_rn(__fmul_rn(gamma, dot), coef0);
