@@ -108,22 +108,26 @@ struct IngestInfo {
 
 // Validates the CSR structure and labels; detects binary (all 1.0) values;
 // the longest row and the exponent range of the values (one atomic per warp).
+// Eight lanes per row read its entries side by side (one thread per row: 66
+// us for 581,012 rows of 12 entries). No entry outside [0, indptr[n]) is read,
+// whatever the row pointers hold.
+constexpr int kRowLanes = 8;
 __global__ void k_validate(int64_t n, int64_t d, const int64_t *indptr, const int32_t *indices,
                            const float *values, const int8_t *y, IngestInfo *info)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int len = 0, bmax = 0, nbmin = 0, sub = 0;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kRowLanes;
+    const int gl = threadIdx.x % kRowLanes;
+    int len = 0, bmax = 0, nbmin = 0, sub = 0, pos = 0;
+    bool bp = false, nb = false, nf = false, bi = false, by = false;
     if (i < n) {
-        const int64_t p0 = indptr[i], p1 = indptr[i + 1];
-        if (p1 < p0 || (i == 0 && p0 != 0)) {
-            atomicOr(&info->bad_indptr, 1);
+        const int64_t p0 = indptr[i], p1 = indptr[i + 1], nnz = indptr[n];
+        if (p1 < p0 || (i == 0 && p0 != 0) || p0 < 0 || p1 > nnz) {
+            bp = true;
         } else {
-            int prev = -1;
-            bool nb = false, nf = false, bi = false;
-            for (int64_t p = p0; p < p1; ++p) {
-                int c = indices[p];
+            for (int64_t p = p0 + gl; p < p1; p += kRowLanes) {
+                const int c = indices[p];
+                const int prev = p > p0 ? indices[p - 1] : -1;
                 if (c <= prev || c >= d) bi = true;
-                prev = c;
                 if (values) {
                     const float v = values[p];
                     if (!isfinite(v)) nf = true;
@@ -138,26 +142,31 @@ __global__ void k_validate(int64_t n, int64_t d, const int64_t *indptr, const in
                     }
                 }
             }
-            if (bi) atomicOr(&info->bad_index, 1);
-            if (nf) atomicOr(&info->nonfinite, 1);
-            if (nb) atomicOr(&info->not_binary, 1);
             len = (int)(p1 - p0);
-            if (y) {
-                int8_t v = y[i];
-                if (v != 1 && v != -1) atomicOr(&info->bad_y, 1);
-                if (v == 1) atomicAdd(&info->npos, 1ull);
+            if (y && gl == 0) {
+                const int8_t v = y[i];
+                by = v != 1 && v != -1;
+                pos = v == 1;
             }
         }
     }
     len = __reduce_max_sync(0xffffffffu, len);
     bmax = __reduce_max_sync(0xffffffffu, bmax);
     nbmin = __reduce_max_sync(0xffffffffu, nbmin);
-    sub = __reduce_or_sync(0xffffffffu, sub);
+    const unsigned flags = __reduce_or_sync(0xffffffffu, (unsigned)sub | (unsigned)bp << 1 | (unsigned)nb << 2 |
+                                                             (unsigned)nf << 3 | (unsigned)bi << 4 | (unsigned)by << 5);
+    pos = __reduce_add_sync(0xffffffffu, pos);
     if ((threadIdx.x & 31) == 0) {
-        if (len) atomicMax(&info->maxnnz, len);
-        if (bmax) atomicMax(&info->bmax, bmax);
-        if (nbmin) atomicMax(&info->nbmin, nbmin);
-        if (sub) atomicOr(&info->subnormal, 1);
+        if (len > *(volatile int *)&info->maxnnz) atomicMax(&info->maxnnz, len);
+        if (bmax > *(volatile int *)&info->bmax) atomicMax(&info->bmax, bmax);
+        if (nbmin > *(volatile int *)&info->nbmin) atomicMax(&info->nbmin, nbmin);
+        if (flags & 1u) atomicOr(&info->subnormal, 1);
+        if (flags & 2u) atomicOr(&info->bad_indptr, 1);
+        if ((flags & 4u) && !*(volatile int *)&info->not_binary) atomicOr(&info->not_binary, 1);
+        if (flags & 8u) atomicOr(&info->nonfinite, 1);
+        if (flags & 16u) atomicOr(&info->bad_index, 1);
+        if (flags & 32u) atomicOr(&info->bad_y, 1);
+        if (pos) atomicAdd(&info->npos, (unsigned long long)pos);
     }
 }
 
@@ -498,64 +507,98 @@ __global__ void k_active_from_mark(int64_t n, int G, const uint8_t *mark, int32_
 
 // ---- deterministic, order-preserving compaction by predicate
 enum { PRED_UNMARKED = 0, PRED_ALPHA_POS = 1, PRED_MARKED = 2 };
-constexpr int kChunk = 4096;
+// Four consecutive elements per thread and one block scan per chunk (chunks of
+// 4,096 in 16 block-wide rounds, and one thread adding the chunks' counts,
+// took 27 + 10 us of a decision's 40 us before its contraction).
 constexpr int kCT = 256;
+constexpr int kPer = 4;
+constexpr int kChunk = kCT * kPer;
 
 __device__ __forceinline__ bool pred_at(int pred, int64_t i, const uint8_t *mark, const double *alpha)
 {
     return pred == PRED_UNMARKED ? mark[i] == 0 : (pred == PRED_MARKED ? mark[i] != 0 : alpha[i] > 0.0);
 }
 
-__global__ void k_count(int pred, int64_t n, const uint8_t *mark, const double *alpha, int *counts)
+// which of this thread's elements are selected, as bits
+__device__ __forceinline__ unsigned pred_bits(int pred, int64_t i0, int64_t n, const uint8_t *mark, const double *alpha)
 {
-    __shared__ int s;
-    if (threadIdx.x == 0) s = 0;
-    __syncthreads();
-    int64_t b0 = (int64_t)blockIdx.x * kChunk;
-    int c = 0;
-    for (int64_t i = b0 + threadIdx.x; i < n && i < b0 + kChunk; i += kCT) c += pred_at(pred, i, mark, alpha);
-    atomicAdd(&s, c);
-    __syncthreads();
-    if (threadIdx.x == 0) counts[blockIdx.x] = s;
+    unsigned m = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+        if (i0 + k < n && pred_at(pred, i0 + k, mark, alpha)) m |= 1u << k;
+    return m;
 }
 
+__global__ void k_count(int pred, int64_t n, const uint8_t *mark, const double *alpha, int *counts)
+{
+    const int64_t i0 = (int64_t)blockIdx.x * kChunk + kPer * threadIdx.x;
+    const unsigned m = pred_bits(pred, i0, n, mark, alpha);
+    __shared__ int wsum[kCT / 32];
+    const unsigned c = __reduce_add_sync(0xffffffffu, (unsigned)__popc(m));
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = (int)c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int w = 0; w < kCT / 32; ++w) t += wsum[w];
+        counts[blockIdx.x] = t;
+    }
+}
+
+// exclusive scan of the chunks' counts (one block)
 __global__ void k_scan(const int *counts, int nb, int *offsets, long long *total)
 {
-    if (threadIdx.x != 0) return;
-    long long acc = 0;
-    for (int b = 0; b < nb; ++b) {
-        offsets[b] = (int)acc;
-        acc += counts[b];
+    __shared__ int wsum[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    long long base = 0;
+    for (int b0 = 0; b0 < nb; b0 += blockDim.x) {
+        const int b = b0 + threadIdx.x;
+        const int c = b < nb ? counts[b] : 0;
+        int incl = c;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += o;
+        }
+        if (lane == 31) wsum[w] = incl;
+        __syncthreads();
+        int pre = 0, tot = 0;
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
+            if (k < w) pre += wsum[k];
+            tot += wsum[k];
+        }
+        if (b < nb) offsets[b] = (int)(base + pre + incl - c);
+        base += tot;
+        __syncthreads();
     }
-    *total = acc;
+    if (threadIdx.x == 0) *total = base;
 }
 
 __global__ void k_scatter(int pred, int64_t n, const uint8_t *mark, const double *alpha,
                           const int8_t *y, const int *offsets, int32_t *list, double *coef)
 {
     __shared__ int wsum[kCT / 32];
-    __shared__ int base;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (threadIdx.x == 0) base = offsets[blockIdx.x];
+    const int64_t i0 = (int64_t)blockIdx.x * kChunk + kPer * threadIdx.x;
+    const unsigned m = pred_bits(pred, i0, n, mark, alpha);
+    const int c = __popc(m);
+    int incl = c;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += o;
+    }
+    if (lane == 31) wsum[w] = incl;
     __syncthreads();
-    int64_t b0 = (int64_t)blockIdx.x * kChunk;
-    for (int64_t s0 = b0; s0 < n && s0 < b0 + kChunk; s0 += kCT) {
-        int64_t i = s0 + threadIdx.x;
-        bool p = i < n && i < b0 + kChunk && pred_at(pred, i, mark, alpha);
-        unsigned m = __ballot_sync(0xffffffffu, p);
-        if (lane == 0) wsum[w] = __popc(m);
-        __syncthreads();
-        int pre = __popc(m & ((1u << lane) - 1u));
-        for (int k = 0; k < w; ++k) pre += wsum[k];
-        int tot = 0;
-        for (int k = 0; k < kCT / 32; ++k) tot += wsum[k];
-        if (p) {
-            list[base + pre] = (int32_t)i;
-            if (coef) coef[base + pre] = alpha[i] * (double)y[i];
+    int at = offsets[blockIdx.x] + incl - c;
+    for (int k = 0; k < w; ++k) at += wsum[k];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if ((m >> k) & 1u) {
+            const int64_t i = i0 + k;
+            list[at] = (int32_t)i;
+            if (coef) coef[at] = alpha[i] * (double)y[i];
+            ++at;
         }
-        __syncthreads();
-        if (threadIdx.x == 0) base += tot;
-        __syncthreads();
     }
 }
 
@@ -724,7 +767,7 @@ void ingest(Arena &ar, const svm_csr *X, const int8_t *y, bool need_fp64, bool n
     }
     IngestInfo *info = ar.alloc<IngestInfo>(1);
     CK(cudaMemsetAsync(info, 0, sizeof(IngestInfo), st));
-    k_validate<<<grid1(X->n), 256, 0, st>>>(X->n, X->d, out.indptr, out.indices, out.values, out.y, info);
+    k_validate<<<grid1(X->n * kRowLanes), 256, 0, st>>>(X->n, X->d, out.indptr, out.indices, out.values, out.y, info);
     CK(cudaGetLastError());
     ++*launches;
     IngestInfo h;
@@ -776,7 +819,7 @@ int64_t compact(Arena &ar, int pred, int64_t n, const uint8_t *mark, const doubl
     int *offs = ar.alloc<int>(nb);
     long long *tot = ar.alloc<long long>(1);
     k_count<<<nb, kCT, 0, st>>>(pred, n, mark, alpha, counts);
-    k_scan<<<1, 32, 0, st>>>(counts, nb, offs, tot);
+    k_scan<<<1, 256, 0, st>>>(counts, nb, offs, tot);
     k_scatter<<<nb, kCT, 0, st>>>(pred, n, mark, alpha, y, offs, list, coef);
     CK(cudaGetLastError());
     *launches += 3;
@@ -784,6 +827,25 @@ int64_t compact(Arena &ar, int pred, int64_t n, const uint8_t *mark, const doubl
     CK(cudaMemcpyAsync(&h, tot, sizeof h, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     return h;
+}
+
+// a contraction with its workspace from the call's arena
+void contract(Arena &ar, const RbfContract &c, cudaStream_t st)
+{
+    const size_t b = rbf_contract_workspace_bytes(c);
+    CK(launch_rbf_contract(c, b ? ar.alloc<unsigned char>(b) : nullptr, st));
+}
+
+// tensor cores; sv: the prepared support vectors, or NULL to prepare them here
+void contract_tc(Arena &ar, const RbfContract &c, const void *sv, int *err, cudaStream_t st)
+{
+    if (!sv) {
+        void *p = ar.alloc<unsigned char>(tc_rbf_sv_bytes(c.nsv, c.d));
+        CK(tc_rbf_prepare_sv(c, p, st));
+        sv = p;
+    }
+    void *ws = ar.alloc<unsigned char>(tc_rbf_workspace_bytes(c));
+    CK(launch_rbf_contract_tc(c, sv, ws, err, st));
 }
 
 size_t smem_limit()
@@ -1156,10 +1218,12 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
             c.yq = D.y;
             c.add_scalar = 0.0;
             c.xd = D.xd;
+            // f must not depend on how many rows one reconstruction covers
+            // (the re-layout's solve is the same bit for bit)
+            c.keep_order = 1;
             if (use_tc && mode == MODE_MIXED && tc_rbf_supported((int)D.d)) {
-                void *ws = ar.alloc<unsigned char>(tc_rbf_workspace_bytes(n, w_nsv, (int)D.d));
                 int tc_err = 0;
-                CK(launch_rbf_contract_tc(c, ws, &tc_err, st));
+                contract_tc(ar, c, nullptr, &tc_err, st);
                 launches += 3;
                 CK(cudaStreamSynchronize(st));
                 if (tc_err) {
@@ -1167,7 +1231,7 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
                     throw Fail{SVM_ERR_TIMEOUT};
                 }
             } else {
-                CK(launch_rbf_contract(c, st));
+                contract(ar, c, st);
                 ++launches;
             }
         }
@@ -1589,10 +1653,12 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
             c.yq = D.y;
             c.add_scalar = 0.0;
             c.xd = D.xd;
+            // f must not depend on how many rows one reconstruction covers
+            // (the re-layout's solve is the same bit for bit)
+            c.keep_order = 1;
             if (use_tc && mode == MODE_MIXED && nsv > 0 && tc_rbf_supported((int)D.d)) {
-                void *ws = ar.alloc<unsigned char>(tc_rbf_workspace_bytes(nw, nsv, (int)D.d));
                 int tc_err = 0;
-                CK(launch_rbf_contract_tc(c, ws, &tc_err, st));
+                contract_tc(ar, c, nullptr, &tc_err, st);
                 launches += 3;
                 CK(cudaStreamSynchronize(st));
                 if (tc_err) {
@@ -1600,7 +1666,7 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
                     throw Fail{SVM_ERR_TIMEOUT};
                 }
             } else if (nw > 0) {
-                CK(launch_rbf_contract(c, st));
+                contract(ar, c, st);
                 ++launches;
             }
             if (inc_nq > 0 && inc_nd > 0) {
@@ -1611,7 +1677,7 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
                 c.nq = inc_nq;
                 c.yq = nullptr;
                 c.accumulate = 1;
-                CK(launch_rbf_contract(c, st));
+                contract(ar, c, st);
                 ++launches;
             }
             CK(cudaEventRecord(e1, st));
@@ -1721,10 +1787,11 @@ void check_kernel(const svm_kernel &K)
 // Eq. (classi) before the sign for the queries Z against support vectors:
 // rows list_sv[0 .. nsv) of DX with coefficients coef (alpha y). DX was
 // ingested for this precision; it is taken by value because norms it lacks
-// are derived into the call's arena.
+// are derived into the call's arena. tc_sv: the support vectors prepared for
+// the tensor cores, or NULL.
 void decision_eval(Arena &ar, DevCSR DX, const int32_t *list_sv, const double *coef, int64_t nsv, double b,
                    const svm_kernel &K, const svm_csr *Z, int32_t precision, cudaStream_t st, double *out,
-                   int *launches_out)
+                   int *launches_out, const void *tc_sv = nullptr)
 {
     int launches = 0;
     const bool rbf = K.kind == SVM_KERNEL_RBF;
@@ -1791,17 +1858,16 @@ void decision_eval(Arena &ar, DevCSR DX, const int32_t *list_sv, const double *c
     c.add_scalar = -b;
     c.xd = xd_pair(DX, DZ);
     if (rbf && precision == SVM_MIXED_BF16 && mode == MODE_MIXED && nsv > 0 && tc_rbf_supported((int)DX.d)) {
-        void *ws = ar.alloc<unsigned char>(tc_rbf_workspace_bytes(DZ.n, nsv, (int)DX.d));
         int tc_err = 0;
-        CK(launch_rbf_contract_tc(c, ws, &tc_err, st));
-        launches += 3;
+        contract_tc(ar, c, tc_sv, &tc_err, st);
+        launches += tc_sv ? 2 : 3;
         CK(cudaStreamSynchronize(st));
         if (tc_err) {
             set_err("a wait in the tensor-core decision kernel exceeded its limit");
             throw Fail{SVM_ERR_TIMEOUT};
         }
     } else {
-        CK(launch_rbf_contract(c, st));
+        contract(ar, c, st);
         ++launches;
     }
     if (!Z->on_device) CK(cudaMemcpyAsync(out, out_d, sizeof(double) * DZ.n, cudaMemcpyDeviceToHost, st));
@@ -1887,6 +1953,7 @@ struct ModelState {
     double b = 0.0;
     svm_kernel K{};
     int32_t precision = SVM_FP64;
+    const void *tc_sv = nullptr;    // mixed precision: the support vectors as the tensor cores read them
     std::vector<void *> mem;        // device allocations freed with the model
 };
 
@@ -1979,6 +2046,23 @@ ModelState *model_create_impl(const svm_csr *X, const int8_t *y, const double *a
         k_iota<<<grid1(m), 256, 0, st>>>(m, M->list);
         CK(cudaGetLastError());
         ++launches;
+    }
+    if (rbf && precision == SVM_MIXED_BF16 && !S.binary && m > 0 && tc_rbf_supported((int)S.d)) {
+        RbfContract c;
+        std::memset(&c, 0, sizeof c);
+        c.x_indptr = S.indptr;
+        c.x_indices = S.indices;
+        c.x_values = S.vmix;
+        c.x_normf = S.normf;
+        c.sv = M->list;
+        c.coef = M->coef;
+        c.nsv = m;
+        c.d = (int32_t)S.d;
+        c.gamma = K.gamma;
+        void *p = keep.alloc<unsigned char>(tc_rbf_sv_bytes(m, (int)S.d));
+        CK(tc_rbf_prepare_sv(c, p, st));
+        ++launches;
+        M->tc_sv = p;
     }
     CK(cudaStreamSynchronize(st));
     M->mem = std::move(keep.ptrs);
@@ -2462,7 +2546,7 @@ void srv_admit(Server &S, const std::shared_ptr<SrvJob> &J)
     }
     CK(cudaMemcpyAsync(y, J->y.data(), J->n, cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(S.info_d, 0, sizeof(IngestInfo), st));
-    k_validate<<<grid1(J->n), 256, 0, st>>>(J->n, J->d, indptr, indices, values, y, S.info_d);
+    k_validate<<<grid1(J->n * kRowLanes), 256, 0, st>>>(J->n, J->d, indptr, indices, values, y, S.info_d);
     k_norms<<<grid1(J->n), 256, 0, st>>>(J->n, indptr, values, norm, vmix, normf, S.info_d);
     k_iota<<<grid1(J->n), 256, 0, st>>>(J->n, rows);
     if (dense) k_dense_bf16<<<(unsigned)J->n, 128, 0, st>>>(J->n, (int)J->d, dpad, indptr, indices, vmix, dmat);
@@ -2686,7 +2770,7 @@ int train_fixed_impl(const svm_csr *X, const int8_t *y, const svm_params *P, dou
     // ingest checks (device buffers are read in place)
     IngestInfo *info = W.take<IngestInfo>(1);
     CK(cudaMemsetAsync(info, 0, sizeof(IngestInfo), st));
-    k_validate<<<grid1(n), 256, 0, st>>>(n, X->d, X->indptr, X->indices, X->values, y, info);
+    k_validate<<<grid1(n * kRowLanes), 256, 0, st>>>(n, X->d, X->indptr, X->indices, X->values, y, info);
     CK(cudaGetLastError());
     ++launches;
     IngestInfo h;
@@ -2924,7 +3008,7 @@ int svm_model_decision(const svm_model *model, const svm_csr *Z, void *stream, d
         cudaStream_t st = as_stream(stream);
         int launches = 0;
         Arena ar(st);
-        decision_eval(ar, M.sv, M.list, M.coef, M.nsv, M.b, M.K, Z, M.precision, st, out, &launches);
+        decision_eval(ar, M.sv, M.list, M.coef, M.nsv, M.b, M.K, Z, M.precision, st, out, &launches, M.tc_sv);
         g_launches += launches;
         return SVM_OK;
     } catch (const Fail &f) {

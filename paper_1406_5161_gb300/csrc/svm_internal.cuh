@@ -320,15 +320,22 @@ struct RbfContract {
     const int8_t *yq;          // subtract yq[row] when non-NULL
     double add_scalar;
     int32_t accumulate;        // 1: add to out[] instead of writing (CUDA-core path only)
+    int32_t keep_order;        // 1: sums in an order that does not depend on nq (no split)
     XdFormat xd;               // FP64 mode: exact inner products (xd.on) for X and Z together
 };
-cudaError_t launch_rbf_contract(const RbfContract &c, cudaStream_t st);
+// ws: rbf_contract_workspace_bytes(c) bytes (NULL when that is 0)
+size_t rbf_contract_workspace_bytes(const RbfContract &c);
+cudaError_t launch_rbf_contract(const RbfContract &c, void *ws, cudaStream_t st);
 
-// Tensor-core (tcgen05) version for MODE_MIXED inputs; d <= 256. `ws` holds
-// tc_rbf_workspace_bytes(nq, nsv, d); *err_host is written asynchronously (1
-// when a wait inside the kernel gave up) and is valid after a stream sync.
+// Tensor-core (tcgen05) version for MODE_MIXED inputs; d <= 256. `sv` holds
+// tc_rbf_sv_bytes(nsv, d), written by tc_rbf_prepare_sv (once per set of
+// support vectors, coefficients and gamma); `ws` tc_rbf_workspace_bytes(c);
+// *err_host is written asynchronously (1 when a wait inside the
+// kernel gave up) and is valid after a stream sync.
 bool tc_rbf_supported(int d);
-size_t tc_rbf_workspace_bytes(int64_t nq, int64_t nsv, int d);
-cudaError_t launch_rbf_contract_tc(const RbfContract &c, void *ws, int *err_host, cudaStream_t st);
+size_t tc_rbf_sv_bytes(int64_t nsv, int d);
+size_t tc_rbf_workspace_bytes(const RbfContract &c);
+cudaError_t tc_rbf_prepare_sv(const RbfContract &c, void *sv, cudaStream_t st);
+cudaError_t launch_rbf_contract_tc(const RbfContract &c, const void *sv, void *ws, int *err_host, cudaStream_t st);
 
 }  // namespace svmgb

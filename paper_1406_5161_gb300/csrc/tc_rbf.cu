@@ -124,6 +124,11 @@ struct TcArgs {
     double add_scalar;
     double *out;
     int *err;
+    // few query tiles: the support tiles split over gridDim.y CTAs per query
+    // tile, whose sums (part: [splits][nq]) the last CTA to finish adds in
+    // split order (done: per query tile, zeroed)
+    double *part;
+    unsigned *done;
 };
 
 // 2^x on the special-function unit (flush to zero below 2^-126)
@@ -233,7 +238,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
     __shared__ uint32_t tmem_base;
     __shared__ __align__(16) float s_xc[kMaxStages][kTile], s_coef[kMaxStages][kTile];
     __shared__ double s_acc[kTile];   // the second column half's row sums
-    __shared__ int s_fail;
+    __shared__ int s_fail, s_last;
     const volatile int *fail = &s_fail;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -262,7 +267,10 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base;
-    const int64_t ntiles = (a.nsv + kTile - 1) / kTile;
+    const int64_t ntiles_all = (a.nsv + kTile - 1) / kTile;
+    const int splits = gridDim.y;
+    const int64_t tile0 = ntiles_all * (int64_t)blockIdx.y / splits;   // this CTA's first support tile
+    const int64_t ntiles = ntiles_all * (int64_t)(blockIdx.y + 1) / splits - tile0;
 
     bool ok = true;
     int64_t issued = 0;         // producer: support tiles whose loads were issued
@@ -290,9 +298,9 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
                 unsigned char *tb = tileB + (size_t)sl * tile_all;
                 mbar_expect_tx(&bar_full[sl], (uint32_t)tile_all + 2 * kTile * 4);
                 for (int kb = 0; kb < a.kblocks; ++kb)
-                    tma_load_2d(tb + (size_t)kb * kTileBytes, &mapX, kb * kKB, (int)(t * kTile), &bar_full[sl]);
-                bulk_load(s_xc[sl], a.xc + t * kTile, kTile * 4, &bar_full[sl]);
-                bulk_load(s_coef[sl], a.coef + t * kTile, kTile * 4, &bar_full[sl]);
+                    tma_load_2d(tb + (size_t)kb * kTileBytes, &mapX, kb * kKB, (int)((tile0 + t) * kTile), &bar_full[sl]);
+                bulk_load(s_xc[sl], a.xc + (tile0 + t) * kTile, kTile * 4, &bar_full[sl]);
+                bulk_load(s_coef[sl], a.coef + (tile0 + t) * kTile, kTile * 4, &bar_full[sl]);
                 issued = t + 1;
             }
         }
@@ -449,16 +457,37 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
         }
     } else {
         // the two column halves of a row meet in shared memory (fixed order)
+        const int64_t q = q0 + my_row;
         if (warp >= 2 && half == 1) s_acc[my_row] = acc;
         __syncthreads();
-        if (warp >= 2 && half == 0) {
-            const int64_t q = q0 + my_row;
-            if (q < a.nq) {
-                const int32_t row = a.qrow[q];
-                double v = (acc + s_acc[my_row]) + a.add_scalar;
-                if (a.yq) v -= (double)a.yq[row];
-                a.out[row] = v;
+        if (warp >= 2 && half == 0) acc += s_acc[my_row];
+        bool mine = warp >= 2 && half == 0 && q < a.nq;
+        if (splits > 1) {
+            if (mine) a.part[(size_t)blockIdx.y * a.nq + q] = acc;
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) s_last = atomicAdd(a.done + blockIdx.x, 1u) == (unsigned)splits - 1u;
+            __syncthreads();
+            if (s_last) {
+                __threadfence();
+                // each half of the epilogue warps adds half of the splits
+                double v = 0.0;
+                if (warp >= 2 && q < a.nq) {
+                    const int k1 = half ? splits : splits / 2;
+                    for (int k = half ? splits / 2 : 0; k < k1; ++k) v += __ldcg(a.part + (size_t)k * a.nq + q);
+                }
+                if (warp >= 2 && half == 1) s_acc[my_row] = v;
+                __syncthreads();
+                acc = v + s_acc[my_row];
+            } else {
+                mine = false;
             }
+        }
+        if (mine) {
+            const int32_t row = a.qrow[q];
+            double v = acc + a.add_scalar;
+            if (a.yq) v -= (double)a.yq[row];
+            a.out[row] = v;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -471,28 +500,31 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
 
 // ------------------------------------------------------------- preparation
 
-// Dense BF16 rows (row-major, ld = d_pad) from CSR rows (list or all) and the
-// scaled norms used by the epilogue; padding rows are zero.
+// Dense BF16 rows (row-major, ld = d_pad, a multiple of 64) from CSR rows
+// (list or all) and the scaled norms used by the epilogue; padding rows are
+// zero. A warp per row, the row cleared with 16-byte stores (one CTA of 64
+// threads per row: 29 us for 48,868 rows of 12 entries).
 __global__ void k_densify(int64_t nrows, int64_t nrows_pad, int d_pad, const int32_t *list,
                           const int64_t *indptr, const int32_t *indices, const float *vmix,
                           const float *normf, float nscale, __nv_bfloat16 *dense, float *cnorm,
                           const double *coef_in, float *coef_out, int32_t *outrow, int out_by_row)
 {
-    const int64_t r = blockIdx.x;
+    const int lane = threadIdx.x & 31;
+    const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (r >= nrows_pad) return;
     __nv_bfloat16 *dst = dense + (size_t)r * d_pad;
-    for (int c = threadIdx.x; c < d_pad; c += blockDim.x) dst[c] = __float2bfloat16_rn(0.f);
-    __syncthreads();
+    for (int c = lane; c < d_pad / 8; c += 32) reinterpret_cast<uint4 *>(dst)[c] = make_uint4(0, 0, 0, 0);
+    __syncwarp();
     if (r < nrows) {
         const int64_t row = list ? list[r] : r;
-        for (int64_t p = indptr[row] + threadIdx.x; p < indptr[row + 1]; p += blockDim.x)
-            dst[indices[p]] = __float2bfloat16_rn(vmix[p]);
-        if (threadIdx.x == 0) {
+        const int64_t p1 = indptr[row + 1];
+        for (int64_t p = indptr[row] + lane; p < p1; p += 32) dst[indices[p]] = __float2bfloat16_rn(vmix[p]);
+        if (lane == 0) {
             cnorm[r] = nscale * normf[row];
             if (coef_out) coef_out[r] = (float)coef_in[r];
             if (outrow) outrow[r] = out_by_row ? (int32_t)row : (int32_t)r;
         }
-    } else if (threadIdx.x == 0) {
+    } else if (lane == 0) {
         cnorm[r] = 0.f;
         if (coef_out) coef_out[r] = 0.f;
     }
@@ -531,73 +563,137 @@ bool make_map(CUtensorMap *m, const void *base, int64_t rows, int d_pad)
 
 bool tc_rbf_supported(int d) { return d >= 1 && d <= kMaxKBlocks * kKB && encode_fn() != nullptr; }
 
-size_t tc_rbf_workspace_bytes(int64_t nq, int64_t nsv, int d)
+namespace {
+
+// consecutive 256-byte aligned pieces of a buffer (NULL base: sizes only)
+struct Pieces {
+    unsigned char *p;
+    size_t used = 0;
+    template <class T>
+    T *take(size_t count)
+    {
+        T *r = reinterpret_cast<T *>(p + used);
+        used += (count * sizeof(T) + 255) & ~(size_t)255;
+        return p ? r : nullptr;
+    }
+};
+
+int pad_cols(int d) { return (d + kKB - 1) / kKB * kKB; }
+int64_t pad_rows(int64_t n) { return (std::max<int64_t>(n, 1) + kTile - 1) / kTile * kTile; }
+
+// the support vectors' side: dense rows, scaled norms, coefficients
+struct SvSide {
+    __nv_bfloat16 *X;
+    float *xc, *coef;
+};
+SvSide sv_side(Pieces &p, int64_t nsv, int d)
 {
-    const int d_pad = ((d + kKB - 1) / kKB) * kKB;
-    const int64_t nq_pad = (nq + kTile - 1) / kTile * kTile;
-    const int64_t ns_pad = (nsv + kTile - 1) / kTile * kTile;
-    size_t b = 0;
-    auto add = [&](size_t x) { b += (x + 255) & ~(size_t)255; };
-    add((size_t)nq_pad * d_pad * 2);
-    add((size_t)ns_pad * d_pad * 2);
-    add((size_t)nq_pad * 4);   // zc
-    add((size_t)ns_pad * 4);   // xc
-    add((size_t)ns_pad * 4);   // coef
-    add((size_t)nq_pad * 4);   // qrow
-    add(256);                  // err
-    return b;
+    const int64_t n = pad_rows(nsv);
+    SvSide s;
+    s.X = p.take<__nv_bfloat16>((size_t)n * pad_cols(d));
+    s.xc = p.take<float>(n);
+    s.coef = p.take<float>(n);
+    return s;
+}
+struct QSide {
+    __nv_bfloat16 *Z;
+    float *zc;
+    int32_t *qrow;
+    int *err;
+    unsigned *done;
+    double *part;
+    int splits;
+};
+// Two CTAs share an SM: with fewer query tiles than that the support tiles are
+// split (48,868 support vectors, 300 queries: 3 CTAs took 377 us), at least
+// four tiles to a CTA and at most 64 CTAs to a query tile (the last one adds
+// their sums, an FP64 addition of a warp per 64 cycles).
+QSide q_side(Pieces &p, int64_t nq, int64_t nsv, int d, bool keep_order)
+{
+    int dev = 0, sms = 1;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 1;
+    const int64_t n = pad_rows(nq), tiles = n / kTile, nt = pad_rows(nsv) / kTile;
+    QSide s;
+    s.splits = keep_order ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>({2 * (int64_t)sms / tiles, nt / 4, 64}));
+    s.Z = p.take<__nv_bfloat16>((size_t)n * pad_cols(d));
+    s.zc = p.take<float>(n);
+    s.qrow = p.take<int32_t>(n);
+    s.err = p.take<int>(1 + (size_t)tiles);   // the error word, then the tiles' counters
+    s.done = reinterpret_cast<unsigned *>(s.err) + 1;
+    s.part = p.take<double>(s.splits > 1 ? (size_t)s.splits * nq : 0);
+    return s;
+}
+
+}  // namespace
+
+size_t tc_rbf_sv_bytes(int64_t nsv, int d)
+{
+    Pieces p{nullptr};
+    sv_side(p, nsv, d);
+    return p.used;
+}
+
+size_t tc_rbf_workspace_bytes(const RbfContract &c)
+{
+    Pieces p{nullptr};
+    q_side(p, c.nq, c.nsv, c.d, c.keep_order != 0);
+    return p.used;
+}
+
+// The support vectors' side of a contraction into `sv` (tc_rbf_sv_bytes).
+cudaError_t tc_rbf_prepare_sv(const RbfContract &c, void *sv, cudaStream_t st)
+{
+    Pieces p{static_cast<unsigned char *>(sv)};
+    const SvSide s = sv_side(p, c.nsv, c.d);
+    const int64_t n = pad_rows(c.nsv);
+    const float nscale = (float)(-c.gamma) * 1.4426950408889634f;
+    k_densify<<<(unsigned)(n / 8), 256, 0, st>>>(c.nsv, n, pad_cols(c.d), c.sv, c.x_indptr, c.x_indices, c.x_values,
+                                                 c.x_normf, nscale, s.X, s.xc, c.coef, s.coef, nullptr, 0);
+    return cudaGetLastError();
 }
 
 // Same contract as launch_rbf_contract (MODE_MIXED inputs: vmix values and
-// FP32 norms), on the tensor cores. `ws` must hold tc_rbf_workspace_bytes.
-cudaError_t launch_rbf_contract_tc(const RbfContract &c, void *ws, int *err_host, cudaStream_t st)
+// FP32 norms), on the tensor cores. `sv` was filled by tc_rbf_prepare_sv;
+// `ws` must hold tc_rbf_workspace_bytes.
+cudaError_t launch_rbf_contract_tc(const RbfContract &c, const void *sv, void *ws, int *err_host, cudaStream_t st)
 {
     *err_host = 0;
     if (c.nq <= 0) return cudaSuccess;
-    const int d_pad = ((c.d + kKB - 1) / kKB) * kKB;
+    if (c.nsv <= 0) return cudaErrorInvalidValue;   // (no support vectors: every sum is zero)
+    const int d_pad = pad_cols(c.d);
     const int kblocks = d_pad / kKB;
     if (kblocks > kMaxKBlocks) return cudaErrorInvalidValue;
-    const int64_t nq_pad = (c.nq + kTile - 1) / kTile * kTile;
-    const int64_t ns = c.nsv > 0 ? c.nsv : 1;
-    const int64_t ns_pad = (ns + kTile - 1) / kTile * kTile;
-    unsigned char *p = static_cast<unsigned char *>(ws);
-    auto take = [&](size_t x) {
-        unsigned char *r = p;
-        p += (x + 255) & ~(size_t)255;
-        return r;
-    };
-    auto *Zd = reinterpret_cast<__nv_bfloat16 *>(take((size_t)nq_pad * d_pad * 2));
-    auto *Xd = reinterpret_cast<__nv_bfloat16 *>(take((size_t)ns_pad * d_pad * 2));
-    auto *zc = reinterpret_cast<float *>(take((size_t)nq_pad * 4));
-    auto *xc = reinterpret_cast<float *>(take((size_t)ns_pad * 4));
-    auto *coef = reinterpret_cast<float *>(take((size_t)ns_pad * 4));
-    auto *qrow = reinterpret_cast<int32_t *>(take((size_t)nq_pad * 4));
-    auto *err = reinterpret_cast<int *>(take(256));
+    const int64_t nq_pad = pad_rows(c.nq), tiles = nq_pad / kTile;
+    Pieces pw{static_cast<unsigned char *>(ws)}, ps{static_cast<unsigned char *>(const_cast<void *>(sv))};
+    const QSide q = q_side(pw, c.nq, c.nsv, c.d, c.keep_order != 0);
+    const SvSide x = sv_side(ps, c.nsv, c.d);
     const float L2E = 1.4426950408889634f;
     const float nscale = (float)(-c.gamma) * L2E;
-    cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), st);
+    cudaError_t e = cudaMemsetAsync(q.err, 0, sizeof(int) * (1 + (size_t)tiles), st);
     if (e != cudaSuccess) return e;
-    k_densify<<<(unsigned)nq_pad, 64, 0, st>>>(c.nq, nq_pad, d_pad, c.q, c.z_indptr, c.z_indices, c.z_values,
-                                               c.z_normf, nscale, Zd, zc, nullptr, nullptr, qrow, c.out_by_row);
-    k_densify<<<(unsigned)ns_pad, 64, 0, st>>>(c.nsv, ns_pad, d_pad, c.sv, c.x_indptr, c.x_indices, c.x_values,
-                                               c.x_normf, nscale, Xd, xc, c.coef, coef, nullptr, 0);
+    k_densify<<<(unsigned)(nq_pad / 8), 256, 0, st>>>(c.nq, nq_pad, d_pad, c.q, c.z_indptr, c.z_indices, c.z_values,
+                                                      c.z_normf, nscale, q.Z, q.zc, nullptr, nullptr, q.qrow, c.out_by_row);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     CUtensorMap mz, mx;
-    if (!make_map(&mz, Zd, nq_pad, d_pad) || !make_map(&mx, Xd, ns_pad, d_pad)) return cudaErrorInvalidValue;
+    if (!make_map(&mz, q.Z, nq_pad, d_pad) || !make_map(&mx, x.X, pad_rows(c.nsv), d_pad)) return cudaErrorInvalidValue;
     TcArgs a;
     a.nq = c.nq;
     a.nsv = c.nsv;
     a.kblocks = kblocks;
-    a.zc = zc;
-    a.xc = xc;
-    a.coef = coef;
+    a.zc = q.zc;
+    a.xc = x.xc;
+    a.coef = x.coef;
     a.g2 = 2.0f * (float)c.gamma * L2E;
-    a.qrow = qrow;
+    a.qrow = q.qrow;
     a.yq = c.yq;
     a.add_scalar = c.add_scalar;
     a.out = c.out;
-    a.err = err;
+    a.err = q.err;
+    a.part = q.part;
+    a.done = q.done;
     // query tile + a ring of support tiles: 4 slots at d <= 64, else 2; at
     // least 80 KiB so that at most 2 CTAs share an SM: their 2 x 256
     // tensor-memory columns then fit the SM's 512 without waiting
@@ -605,16 +701,10 @@ cudaError_t launch_rbf_contract_tc(const RbfContract &c, void *ws, int *err_host
     const size_t smem = std::max<size_t>((size_t)(1 + a.stages) * kblocks * kTileBytes + 1024, 80 * 1024);
     e = cudaFuncSetAttribute(tc_rbf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    if (c.nsv > 0) {
-        tc_rbf_kernel<<<(unsigned)(nq_pad / kTile), kTcThreads, smem, st>>>(mz, mx, a);
-    } else {
-        // no support vectors: every sum is zero
-        return cudaErrorInvalidValue;
-    }
+    tc_rbf_kernel<<<dim3((unsigned)tiles, (unsigned)q.splits), kTcThreads, smem, st>>>(mz, mx, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(err_host, err, sizeof(int), cudaMemcpyDeviceToHost, st);
-    return e;
+    return cudaMemcpyAsync(err_host, q.err, sizeof(int), cudaMemcpyDeviceToHost, st);
 }
 
 
