@@ -1866,6 +1866,9 @@ void decision_eval(Arena &ar, DevCSR DX, const int32_t *list_sv, const double *c
             set_err("a wait in the tensor-core decision kernel exceeded its limit");
             throw Fail{SVM_ERR_TIMEOUT};
         }
+    } else if (rbf_bits_supported(c)) {
+        CK(launch_rbf_bits(c, ar.alloc<unsigned char>(rbf_bits_workspace_bytes(c)), st));
+        launches += nsv > 0 ? 3 : 2;
     } else {
         contract(ar, c, st);
         ++launches;

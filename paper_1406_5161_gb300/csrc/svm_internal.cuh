@@ -327,6 +327,12 @@ struct RbfContract {
 size_t rbf_contract_workspace_bytes(const RbfContract &c);
 cudaError_t launch_rbf_contract(const RbfContract &c, void *ws, cudaStream_t st);
 
+// Decision values of binary rows as bit masks (rbf_bits.cu): MODE_BINARY, d <=
+// 256, all rows of Z in order; ws: rbf_bits_workspace_bytes(c).
+bool rbf_bits_supported(const RbfContract &c);
+size_t rbf_bits_workspace_bytes(const RbfContract &c);
+cudaError_t launch_rbf_bits(const RbfContract &c, void *ws, cudaStream_t st);
+
 // Tensor-core (tcgen05) version for MODE_MIXED inputs; d <= 256. `sv` holds
 // tc_rbf_sv_bytes(nsv, d), written by tc_rbf_prepare_sv (once per set of
 // support vectors, coefficients and gamma); `ws` tc_rbf_workspace_bytes(c);

@@ -33,7 +33,7 @@ def _alpha(n, C):
 
 
 @pytest.mark.parametrize("m,n", CASES)
-@pytest.mark.parametrize("kind", ["fp64", "binary", "simt", "mixed"])
+@pytest.mark.parametrize("kind", ["fp64", "binary", "binary200", "simt", "mixed"])
 def test_decision_against_the_oracle(m, n, kind):
     if kind == "binary200":   # masks of eight words, ragged rows
         p = synth.random_sparse(n=n + m, d=200, density=0.08, seed=n, binary=True)
