@@ -1800,10 +1800,20 @@ void decision_eval(Arena &ar, DevCSR DX, const int32_t *list_sv, const double *c
     ingest(ar, Z, nullptr, !mixed, mixed, st, DZ, &launches, rbf);
     int mode = (DX.binary && DZ.binary) ? MODE_BINARY : (mixed ? MODE_MIXED : MODE_FP64);
     if (mode != MODE_BINARY && (DX.binary || DZ.binary)) {
-        // one side binary, the other not: derive the missing norms
+        // one side binary, the other not: the binary side's values (when it
+        // has none) and norms; the other side has its own
         for (DevCSR *D : {&DX, &DZ}) {
-            if (mode == MODE_FP64 && !D->norm) D->norm = ar.alloc<double>(D->n);
-            if (mode == MODE_MIXED && !D->vmix) {
+            if (!D->binary) continue;
+            if (!D->values && D->nnz > 0) {
+                float *v = ar.alloc<float>(D->nnz);
+                k_fill_ones<<<grid1(D->nnz), 256, 0, st>>>(D->nnz, v);
+                CK(cudaGetLastError());
+                ++launches;
+                D->values = v;
+            }
+            if (D->n < 1) continue;
+            if (mode == MODE_FP64) D->norm = ar.alloc<double>(D->n);
+            if (mode == MODE_MIXED) {
                 D->vmix = ar.alloc<float>(D->nnz);
                 D->normf = ar.alloc<float>(D->n);
             }
@@ -1996,6 +2006,15 @@ ModelState *model_create_impl(const svm_csr *X, const int8_t *y, const double *a
     S.d = DX.d;
     S.binary = DX.binary;
     S.maxnnz = DX.maxnnz;
+    // the training rows' record and exponent range (those of the support
+    // vectors lie within): later decisions take their formats from them
+    S.bmax = DX.bmax;
+    S.bmin = DX.bmin;
+    S.subnormal = DX.subnormal;
+    S.xd = DX.xd;
+    IngestInfo *info = keep.alloc<IngestInfo>(1);
+    CK(cudaMemcpyAsync(info, DX.info, sizeof(IngestInfo), cudaMemcpyDeviceToDevice, st));
+    S.info = info;
     int64_t *sub_indptr = keep.alloc<int64_t>(m + 1);
     int64_t nnz_m = 0;
     if (m > 0) {
