@@ -12,6 +12,7 @@
 #include <chrono>
 #include <condition_variable>
 #include <deque>
+#include <exception>
 #include <map>
 #include <memory>
 #include <new>
@@ -65,26 +66,128 @@ struct Fail {
         throw Fail{SVM_ERR_ARG};      \
     } while (0)
 
-// Stream-ordered device allocations released when the scope ends.
+// The library's own pool of stream-ordered device memory, one per device. The
+// default pool gives its memory back to the system at every synchronisation,
+// so each call paid for mapping it again (the 32 MB kernel-row cache of a
+// 2,000-row solve alone about 0.3 ms of 6.4). This one keeps up to
+// kPoolKeepBytes between calls and gives back the rest; what it keeps is given
+// back too when an allocation fails for want of memory. The driver orders its
+// reuse across streams and threads.
+constexpr size_t kPoolKeepBytes = (size_t)512 << 20;
+constexpr int kPoolDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kPoolDevices] = {};
+
+cudaMemPool_t device_pool()
+{
+    int dev = 0;
+    CK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kPoolDevices) return nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps props;
+        std::memset(&props, 0, sizeof props);
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        CK(cudaMemPoolCreate(&pool, &props));
+        uint64_t keep = kPoolKeepBytes;
+        CK(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+        g_pool[dev] = pool;
+    }
+    return g_pool[dev];
+}
+
+void *pool_alloc(size_t bytes, cudaStream_t st)
+{
+    void *p = nullptr;
+    cudaMemPool_t pool = device_pool();
+    if (!pool) {
+        CK(cudaMallocAsync(&p, bytes, st));
+        return p;
+    }
+    cudaError_t e = cudaMallocFromPoolAsync(&p, bytes, pool, st);
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        CK(cudaStreamSynchronize(st));
+        CK(cudaMemPoolTrimTo(pool, 0));
+        e = cudaMallocFromPoolAsync(&p, bytes, pool, st);
+    }
+    CK(e);
+    return p;
+}
+
+// Stream-ordered device allocations released when the scope ends; small ones
+// are cut from slabs.
 struct Arena {
+    static constexpr size_t kSlab = (size_t)512 << 10, kSmall = (size_t)64 << 10;
     cudaStream_t st;
     std::vector<void *> ptrs;
-    explicit Arena(cudaStream_t s) : st(s) {}
+    unsigned char *slab = nullptr;
+    size_t slab_used = 0;
+    int exceptions;
+    explicit Arena(cudaStream_t s) : st(s), exceptions(std::uncaught_exceptions()) {}
+    Arena(const Arena &) = delete;
+    Arena &operator=(const Arena &) = delete;
     template <class T>
     T *alloc(size_t count)
     {
-        void *p = nullptr;
-        if (count == 0) count = 1;
-        CK(cudaMallocAsync(&p, count * sizeof(T), st));
-        ptrs.push_back(p);
-        return static_cast<T *>(p);
+        const size_t bytes = ((count ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
+        if (bytes <= kSmall) {
+            if (!slab || slab_used + bytes > kSlab) {
+                slab = static_cast<unsigned char *>(keep(pool_alloc(kSlab, st)));
+                slab_used = 0;
+            }
+            unsigned char *p = slab + slab_used;
+            slab_used += bytes;
+            return reinterpret_cast<T *>(p);
+        }
+        return static_cast<T *>(keep(pool_alloc(bytes, st)));
     }
     ~Arena()
     {
         for (void *p : ptrs) cudaFreeAsync(p, st);
-        cudaStreamSynchronize(st);
+        // a call that ends by an exception may have copies from its own
+        // buffers in flight (one that returns has waited for its work)
+        if (std::uncaught_exceptions() > exceptions) cudaStreamSynchronize(st);
+    }
+
+private:
+    void *keep(void *p)
+    {
+        ptrs.push_back(p);
+        return p;
     }
 };
+
+// Page-locked host memory of the calling thread for small results read back
+// between launches (a copy to pageable memory is staged by the driver).
+struct HostBox {
+    static constexpr size_t kBytes = 4096;
+    void *p = nullptr;
+    bool locked = false;
+    HostBox()
+    {
+        locked = cudaHostAlloc(&p, kBytes, cudaHostAllocPortable) == cudaSuccess;
+        if (!locked) {
+            (void)cudaGetLastError();
+            p = ::operator new(kBytes);
+        }
+    }
+    ~HostBox()
+    {
+        if (locked) cudaFreeHost(p);
+        else ::operator delete(p);
+    }
+};
+enum { BOX_INFO_X = 0, BOX_INFO_Z = 256, BOX_COUNT = 512, BOX_ERR = 520 };
+template <class T>
+T *host_box(int at)
+{
+    static thread_local HostBox box;
+    return reinterpret_cast<T *>(static_cast<unsigned char *>(box.p) + at);
+}
 
 // --------------------------------------------------------------- kernels
 
@@ -104,6 +207,7 @@ struct IngestInfo {
     int nbmin;
     int subnormal;
     int pad3;
+    long long nnz;   // indptr[n]
 };
 
 // Validates the CSR structure and labels; detects binary (all 1.0) values;
@@ -121,7 +225,8 @@ __global__ void k_validate(int64_t n, int64_t d, const int64_t *indptr, const in
     bool bp = false, nb = false, nf = false, bi = false, by = false;
     if (i < n) {
         const int64_t p0 = indptr[i], p1 = indptr[i + 1], nnz = indptr[n];
-        if (p1 < p0 || (i == 0 && p0 != 0) || p0 < 0 || p1 > nnz) {
+        if (i == 0 && gl == 0) info->nnz = nnz;
+        if (p1 < p0 || (i == 0 && p0 != 0) || p0 < 0 || p1 > nnz || nnz >= ((int64_t)1 << 40)) {
             bp = true;
         } else {
             for (int64_t p = p0 + gl; p < p1; p += kRowLanes) {
@@ -721,10 +826,10 @@ __global__ void k_fill_ones(int64_t m, float *v)
     if (i < m) v[i] = 1.0f;
 }
 
-// binary_ok = false: binary rows are kept on the general (values) path,
-// with explicit 1.0 values when the matrix has none
-void ingest(Arena &ar, const svm_csr *X, const int8_t *y, bool need_fp64, bool need_mixed,
-            cudaStream_t st, DevCSR &out, int *launches, bool binary_ok = true)
+// First part of a matrix's ingest: copies (host input), the validation kernel,
+// and its record on the way to `h` (host memory of this thread). Nothing waits.
+void ingest_begin(Arena &ar, const svm_csr *X, const int8_t *y, cudaStream_t st, DevCSR &out, int *launches,
+                  IngestInfo *h)
 {
     if (!X) ARG_FAIL("matrix is NULL");
     if (X->n < 1 || X->d < 1) ARG_FAIL("n and d must be >= 1 (n=%lld d=%lld)", (long long)X->n, (long long)X->d);
@@ -733,21 +838,14 @@ void ingest(Arena &ar, const svm_csr *X, const int8_t *y, bool need_fp64, bool n
     if (!X->indptr || (!X->indices && X->n > 0)) ARG_FAIL("indptr/indices must not be NULL");
     out.n = X->n;
     out.d = X->d;
-    int64_t nnz = 0;
-    if (X->on_device) {
-        CK(cudaMemcpyAsync(&nnz, X->indptr + X->n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-    } else {
-        nnz = X->indptr[X->n];
-    }
-    if (nnz < 0 || nnz >= ((int64_t)1 << 40)) ARG_FAIL("indptr[n] out of range");
-    out.nnz = nnz;
     if (X->on_device) {
         out.indptr = X->indptr;
         out.indices = X->indices;
         out.values = X->values;
         out.y = y;
     } else {
+        const int64_t nnz = X->indptr[X->n];
+        if (nnz < 0 || nnz >= ((int64_t)1 << 40)) ARG_FAIL("indptr[n] out of range");
         int64_t *ip = ar.alloc<int64_t>(X->n + 1);
         CK(cudaMemcpyAsync(ip, X->indptr, sizeof(int64_t) * (X->n + 1), cudaMemcpyHostToDevice, st));
         int32_t *ix = ar.alloc<int32_t>(nnz);
@@ -770,13 +868,24 @@ void ingest(Arena &ar, const svm_csr *X, const int8_t *y, bool need_fp64, bool n
     k_validate<<<grid1(X->n * kRowLanes), 256, 0, st>>>(X->n, X->d, out.indptr, out.indices, out.values, out.y, info);
     CK(cudaGetLastError());
     ++*launches;
-    IngestInfo h;
-    CK(cudaMemcpyAsync(&h, info, sizeof h, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
+    CK(cudaMemcpyAsync(h, info, sizeof *h, cudaMemcpyDeviceToHost, st));
+    out.info = info;
+}
+
+// Second part, once `h` has arrived (the stream was waited for): the verdict,
+// and the data derived for the precision. binary_ok = false: binary rows are
+// kept on the general (values) path, with explicit 1.0 values when the matrix
+// has none.
+void ingest_finish(Arena &ar, const svm_csr *X, const int8_t *y, bool need_fp64, bool need_mixed, cudaStream_t st,
+                   DevCSR &out, int *launches, const IngestInfo &h, bool binary_ok = true)
+{
+    const int64_t nnz = h.nnz;
+    if (nnz < 0 || nnz >= ((int64_t)1 << 40)) ARG_FAIL("indptr[n] out of range");
     if (h.bad_indptr) ARG_FAIL("indptr is not non-decreasing from 0");
     if (h.bad_index) ARG_FAIL("column indices must be strictly increasing within a row and < d");
     if (h.nonfinite) ARG_FAIL("values must be finite");
     if (y && h.bad_y) ARG_FAIL("labels must be +1 or -1");
+    out.nnz = nnz;
     out.binary = !h.not_binary;
     if (out.binary && !binary_ok) {
         out.binary = false;
@@ -790,7 +899,6 @@ void ingest(Arena &ar, const svm_csr *X, const int8_t *y, bool need_fp64, bool n
     }
     out.maxnnz = h.maxnnz;
     out.npos = (int64_t)h.npos;
-    out.info = info;
     // input without values: every value is 1.0 (b = 127), filled or not
     out.bmax = X->values ? h.bmax : 127;
     out.bmin = X->values ? 255 - h.nbmin : 127;
@@ -802,17 +910,27 @@ void ingest(Arena &ar, const svm_csr *X, const int8_t *y, bool need_fp64, bool n
         out.normf = ar.alloc<float>(X->n);
     }
     if (out.norm || out.vmix) {
-        k_norms<<<grid1(X->n), 256, 0, st>>>(X->n, out.indptr, out.values, out.norm, out.vmix, out.normf, info);
+        k_norms<<<grid1(X->n), 256, 0, st>>>(X->n, out.indptr, out.values, out.norm, out.vmix, out.normf, out.info);
         CK(cudaGetLastError());
         ++*launches;
     }
 }
 
+void ingest(Arena &ar, const svm_csr *X, const int8_t *y, bool need_fp64, bool need_mixed, cudaStream_t st, DevCSR &out,
+            int *launches, bool binary_ok = true)
+{
+    IngestInfo *h = host_box<IngestInfo>(BOX_INFO_X);
+    ingest_begin(ar, X, y, st, out, launches, h);
+    CK(cudaStreamSynchronize(st));
+    ingest_finish(ar, X, y, need_fp64, need_mixed, st, out, launches, *h, binary_ok);
+}
+
 cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 
-// order-preserving compaction; returns the count
-int64_t compact(Arena &ar, int pred, int64_t n, const uint8_t *mark, const double *alpha,
-                const int8_t *y, int32_t *list, double *coef, cudaStream_t st, int *launches)
+// order-preserving compaction; the count is on its way to `count` (host
+// memory of this thread)
+void compact_begin(Arena &ar, int pred, int64_t n, const uint8_t *mark, const double *alpha, const int8_t *y,
+                   int32_t *list, double *coef, cudaStream_t st, int *launches, long long *count)
 {
     int nb = (int)((n + kChunk - 1) / kChunk);
     int *counts = ar.alloc<int>(nb);
@@ -823,10 +941,17 @@ int64_t compact(Arena &ar, int pred, int64_t n, const uint8_t *mark, const doubl
     k_scatter<<<nb, kCT, 0, st>>>(pred, n, mark, alpha, y, offs, list, coef);
     CK(cudaGetLastError());
     *launches += 3;
-    long long h = 0;
-    CK(cudaMemcpyAsync(&h, tot, sizeof h, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(count, tot, sizeof *count, cudaMemcpyDeviceToHost, st));
+}
+
+// ... returns the count
+int64_t compact(Arena &ar, int pred, int64_t n, const uint8_t *mark, const double *alpha,
+                const int8_t *y, int32_t *list, double *coef, cudaStream_t st, int *launches)
+{
+    long long *h = host_box<long long>(BOX_COUNT);
+    compact_begin(ar, pred, n, mark, alpha, y, list, coef, st, launches, h);
     CK(cudaStreamSynchronize(st));
-    return h;
+    return *h;
 }
 
 // a contraction with its workspace from the call's arena
@@ -1787,17 +1912,16 @@ void check_kernel(const svm_kernel &K)
 // Eq. (classi) before the sign for the queries Z against support vectors:
 // rows list_sv[0 .. nsv) of DX with coefficients coef (alpha y). DX was
 // ingested for this precision; it is taken by value because norms it lacks
-// are derived into the call's arena. tc_sv: the support vectors prepared for
-// the tensor cores, or NULL.
+// are derived into the call's arena. DZ, hz: Z after ingest_begin and its
+// record. tc_sv: the support vectors prepared for the tensor cores, or NULL.
 void decision_eval(Arena &ar, DevCSR DX, const int32_t *list_sv, const double *coef, int64_t nsv, double b,
                    const svm_kernel &K, const svm_csr *Z, int32_t precision, cudaStream_t st, double *out,
-                   int *launches_out, const void *tc_sv = nullptr)
+                   int *launches_out, DevCSR DZ, const IngestInfo &hz, const void *tc_sv = nullptr)
 {
     int launches = 0;
     const bool rbf = K.kind == SVM_KERNEL_RBF;
     const bool mixed = precision != SVM_FP64;
-    DevCSR DZ;
-    ingest(ar, Z, nullptr, !mixed, mixed, st, DZ, &launches, rbf);
+    ingest_finish(ar, Z, nullptr, !mixed, mixed, st, DZ, &launches, hz, rbf);
     int mode = (DX.binary && DZ.binary) ? MODE_BINARY : (mixed ? MODE_MIXED : MODE_FP64);
     if (mode != MODE_BINARY && (DX.binary || DZ.binary)) {
         // one side binary, the other not: the binary side's values (when it
@@ -1867,15 +1991,11 @@ void decision_eval(Arena &ar, DevCSR DX, const int32_t *list_sv, const double *c
     c.yq = nullptr;
     c.add_scalar = -b;
     c.xd = xd_pair(DX, DZ);
+    int *tc_err = nullptr;
     if (rbf && precision == SVM_MIXED_BF16 && mode == MODE_MIXED && nsv > 0 && tc_rbf_supported((int)DX.d)) {
-        int tc_err = 0;
-        contract_tc(ar, c, tc_sv, &tc_err, st);
+        tc_err = host_box<int>(BOX_ERR);
+        contract_tc(ar, c, tc_sv, tc_err, st);
         launches += tc_sv ? 2 : 3;
-        CK(cudaStreamSynchronize(st));
-        if (tc_err) {
-            set_err("a wait in the tensor-core decision kernel exceeded its limit");
-            throw Fail{SVM_ERR_TIMEOUT};
-        }
     } else if (rbf_bits_supported(c)) {
         CK(launch_rbf_bits(c, ar.alloc<unsigned char>(rbf_bits_workspace_bytes(c)), st));
         launches += nsv > 0 ? 3 : 2;
@@ -1885,6 +2005,10 @@ void decision_eval(Arena &ar, DevCSR DX, const int32_t *list_sv, const double *c
     }
     if (!Z->on_device) CK(cudaMemcpyAsync(out, out_d, sizeof(double) * DZ.n, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    if (tc_err && *tc_err) {
+        set_err("a wait in the tensor-core decision kernel exceeded its limit");
+        throw Fail{SVM_ERR_TIMEOUT};
+    }
     *launches_out += launches;
 }
 
@@ -1901,8 +2025,11 @@ int decision_impl(const svm_csr *X, const int8_t *y, const double *alpha, double
     int launches = 0;
     Arena ar(st);
     const bool mixed = precision != SVM_FP64;
-    DevCSR DX;
-    ingest(ar, X, y, !mixed, mixed, st, DX, &launches, rbf);
+    // both matrices' validation and the support vectors' compaction are under
+    // way before the first wait
+    DevCSR DX, DZ;
+    IngestInfo *hx = host_box<IngestInfo>(BOX_INFO_X), *hz = host_box<IngestInfo>(BOX_INFO_Z);
+    ingest_begin(ar, X, y, st, DX, &launches, hx);
     const int64_t n = DX.n;
     const double *alpha_d = alpha;
     if (!X->on_device) {
@@ -1912,8 +2039,12 @@ int decision_impl(const svm_csr *X, const int8_t *y, const double *alpha, double
     }
     int32_t *list_sv = ar.alloc<int32_t>(n);
     double *coef = ar.alloc<double>(n);
-    int64_t nsv = compact(ar, PRED_ALPHA_POS, n, nullptr, alpha_d, DX.y, list_sv, coef, st, &launches);
-    decision_eval(ar, DX, list_sv, coef, nsv, b, K, Z, precision, st, out, &launches);
+    long long *nsv = host_box<long long>(BOX_COUNT);
+    compact_begin(ar, PRED_ALPHA_POS, n, nullptr, alpha_d, DX.y, list_sv, coef, st, &launches, nsv);
+    ingest_begin(ar, Z, nullptr, st, DZ, &launches, hz);
+    CK(cudaStreamSynchronize(st));
+    ingest_finish(ar, X, y, !mixed, mixed, st, DX, &launches, *hx, rbf);
+    decision_eval(ar, DX, list_sv, coef, *nsv, b, K, Z, precision, st, out, &launches, DZ, *hz);
     g_launches += launches;
     return SVM_OK;
 }
@@ -3030,7 +3161,11 @@ int svm_model_decision(const svm_model *model, const svm_csr *Z, void *stream, d
         cudaStream_t st = as_stream(stream);
         int launches = 0;
         Arena ar(st);
-        decision_eval(ar, M.sv, M.list, M.coef, M.nsv, M.b, M.K, Z, M.precision, st, out, &launches, M.tc_sv);
+        DevCSR DZ;
+        IngestInfo *hz = host_box<IngestInfo>(BOX_INFO_Z);
+        ingest_begin(ar, Z, nullptr, st, DZ, &launches, hz);
+        CK(cudaStreamSynchronize(st));
+        decision_eval(ar, M.sv, M.list, M.coef, M.nsv, M.b, M.K, Z, M.precision, st, out, &launches, DZ, *hz, M.tc_sv);
         g_launches += launches;
         return SVM_OK;
     } catch (const Fail &f) {
