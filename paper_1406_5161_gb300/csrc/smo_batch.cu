@@ -39,14 +39,23 @@ __device__ __forceinline__ void st_release_sys_i32(int *p, int v)
     asm volatile("st.release.sys.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// bulk copy global -> this CTA's shared memory, counted on an mbarrier
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
 struct __align__(16) BatchFinish {
     double sum_a, sum_ayfy, sum_f0;
     long long n0, nsv;
     int pad[2];
 };
 
-// per warp: 16 k-steps x 32 lanes of packed BF16 target pairs (uint2)
-constexpr size_t kFragBytes = (size_t)kWarps * 16 * 32 * sizeof(uint2);
+// 16 k-steps x 32 lanes of packed BF16 target pairs (uint2)
+constexpr size_t kFragBytes = (size_t)16 * 32 * sizeof(uint2);
 
 struct BatchShared {
     Side wup[kWarps], wlow[kWarps];
@@ -59,6 +68,8 @@ struct BatchShared {
     double du, dl, au_new, al_new;
     unsigned char st_u, st_l;
     PairPre pre;
+    unsigned long long stage_bar[kWarps];   // packed units: a row warp's unit has landed
+    int stage_bad;                          // a wait for one gave up
     int job;
 };
 
@@ -83,8 +94,24 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
     int *tcol = reinterpret_cast<int *>(dsm + L.tcol);
     double *ktab = reinterpret_cast<double *>(dsm + L.ktab);
     const double *rtab = ktab + B.ktab_len;
+    uint2 *frag = reinterpret_cast<uint2 *>(dsm + L.total);   // mixed: the tiles' target fragments
+    uint32_t *kdir = reinterpret_cast<uint32_t *>(dsm + L.total + (MODE == MODE_MIXED ? kFragBytes : 0));
     if constexpr (MODE == MODE_FP64) {
         for (int c = tid; c < kExpfxTabLen; c += kThreads) expfx_s[c] = kExpfxTab[c];   // ordered by the cluster sync below
+    }
+    // packed rows (dense BF16 on the tensor cores): each row warp streams its
+    // units of 32 rows through a stage of its own in shared memory
+    constexpr bool PACK_MODE = MODE == MODE_MIXED && LPR == 16;
+    unsigned char *stage0 = reinterpret_cast<unsigned char *>(
+        ((uintptr_t)(kdir + B.kdir_words) + 127) & ~(uintptr_t)127);
+    uint32_t stage_parity = 0;
+    if constexpr (PACK_MODE) {
+        if (tid == 0) {
+            for (int w = 0; w < kWarps; ++w) mbar_init(smem_u32(&sh.stage_bar[w]), 1);
+            sh.stage_bad = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            fence_async_proxy();
+        }
     }
 
     for (;;) {
@@ -140,6 +167,17 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
         const double snap = 1e-12 * C, c_snap = C - snap;
         const double thr = 2.0 * J.tau;
         const int32_t *rows = J.rows;
+        // kernel-row cache of the cluster (FP64): row r's values at [r * kc_ld,
+        // + m), each CTA its own rows' part; a bit per row that is stored,
+        // kept alike in every CTA's shared memory
+        constexpr bool KC_MODE = MODE == MODE_FP64;
+        const int64_t kc_ld = ((int64_t)m + 31) & ~(int64_t)31;
+        const bool kc_on = KC_MODE && B.kc && m <= 32 * B.kdir_words && (int64_t)m * kc_ld * 8 <= B.kc_stride;
+        double *kc = kc_on ? reinterpret_cast<double *>(static_cast<unsigned char *>(B.kc) + (size_t)(blockIdx.x / csize) * B.kc_stride)
+                       : nullptr;
+        if (kc_on) {
+            for (int w = tid; w < (m + 31) / 32; w += kThreads) kdir[w] = 0;
+        }
 
         // FP64 with exact inner products (J.xd.on): target entries hold (m, b)
         // pairs as in the single-solve kernel; an absent value m = 0, b = tmin
@@ -166,7 +204,54 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             fj[r] = -(double)yr;
             sj[r] = (uint8_t)(st_of(yr, 0.0, 1.0) | (yr > 0 ? 0x80 : 0));
         }
+        // This CTA's rows in the order the tensor cores' fragments read them:
+        // unit u (32 rows), tile q, 32-column block b, half h, lane: the 8
+        // values of row 32 u + 16 q + 8 h + lane / 4 at columns 32 b + 8
+        // (lane & 3). A unit is one bulk copy, and its reads have no bank
+        // conflict; gathered row by row from the matrix in every step, the
+        // warps waited for loads 57% of the time (long scoreboard) and a round
+        // of 15 x 32 rows took 7 us.
+        const int units = (hi - lo + 31) / 32;
+        const uint32_t unit_bytes = 64u * (uint32_t)d;
+        unsigned char *pk = nullptr;
+        bool packed = false;
+        if constexpr (PACK_MODE) {
+            packed = dense && B.pack && (d & 31) == 0 && d <= 256 && (int64_t)units * unit_bytes <= B.pack_stride &&
+                     unit_bytes <= (uint32_t)B.stage_bytes;
+            if (packed) {
+                pk = static_cast<unsigned char *>(B.pack) + (size_t)blockIdx.x * B.pack_stride;
+                const int nb = d >> 5, per = nb * 128;   // 16-byte pieces of a unit
+                for (int k = tid; k < units * per; k += kThreads) {
+                    const int ln = k & 31, h = (k >> 5) & 1, qb = (k >> 6) % (2 * nb), u = k / per;
+                    const int r = lo + 32 * u + 16 * (qb / nb) + 8 * h + (ln >> 2);
+                    uint4 v = make_uint4(0, 0, 0, 0);
+                    if (r < hi)
+                        v = __ldg(reinterpret_cast<const uint4 *>(dmat + (size_t)rows[r] * d + 32 * (qb % nb) + 8 * (ln & 3)));
+                    reinterpret_cast<uint4 *>(pk)[k] = v;
+                }
+                fence_async_proxy();   // the bulk copies read them
+            }
+        }
         __syncthreads();
+        const int stage_warps = packed ? B.stage_warps : 0;
+        unsigned char *stage = stage0 + (size_t)(warp - 1) * B.stage_bytes;
+        const uint32_t stage_bar = smem_u32(&sh.stage_bar[warp]);
+        bool in_flight = false;   // a unit is on its way into this warp's stage
+        auto issue_unit = [&](int u) {
+            if (lane == 0) {
+                mbar_arrive_expect_tx(stage_bar, unit_bytes);
+                bulk_load(smem_u32(stage), pk + (size_t)u * unit_bytes, unit_bytes, stage_bar);
+            }
+            in_flight = true;
+        };
+        auto wait_unit = [&]() {
+            if (!in_flight) return;
+            const int bad = mbar_wait_bounded(stage_bar, stage_parity, 10ll * 1000 * 1000 * 1000, &sh.stage_bad);
+            if (__any_sync(0xffffffffu, bad) && lane == 0) sh.stage_bad = 1;
+            stage_parity ^= 1u;
+            in_flight = false;
+        };
+        if (warp >= 1 && warp <= stage_warps && warp - 1 < units) issue_unit(warp - 1);
 
         Side up, low;
         side_empty(up, true);
@@ -181,9 +266,17 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             Tgt *T = tbuf + (size_t)buf * dmax;
             int *tcu = tcol + (size_t)(buf * 2 + 0) * maxnnz;
             int *tcl = tcol + (size_t)(buf * 2 + 1) * maxnnz;
+            bool hu = false, hl = false;   // x_up's / x_low's kernel row is in the cache
+            uint32_t kd_wu = 0, kd_wl = 0;
             if (!first) {
                 if (!dless(thr, low.f - up.f)) { status_code = 0; break; }
                 if (iter >= J.max_iter) { status_code = 1; break; }
+                if (kc_on) {
+                    kd_wu = kdir[up.i >> 5];
+                    kd_wl = kdir[low.i >> 5];
+                    hu = (kd_wu >> (up.i & 31)) & 1u;
+                    hl = (kd_wl >> (low.i & 31)) & 1u;
+                }
                 // the pair step's part that K(up, low) does not enter
                 if (warp >= kPre0) pair_pre<MODE == MODE_FP64>(&sh.pre, warp - kPre0, lane, up, low, C);
                 // ---- 1. targets into the shared-memory buffer
@@ -302,29 +395,11 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                         have_step = true;
                     }
                 };
-                // kernel values, FP64 update of Eq. (fup), selection keys of one row
-                auto finish_row = [&](int r, int g, int len, Acc su, Acc sl, double fi, uint8_t sb) {
+                double *kcu = kc_on && !first ? kc + (size_t)up.i * kc_ld : nullptr;
+                double *kcl = kc_on && !first ? kc + (size_t)low.i * kc_ld : nullptr;
+                // FP64 update of Eq. (fup) and selection keys of one row
+                auto update_row = [&](int r, double ku, double kl, double fi, uint8_t sb) {
                     if (!first) {
-                        double ku, kl;
-                        if constexpr (MODE == MODE_BINARY) {
-                            int du2 = up.len + len - 2 * su, dl2 = low.len + len - 2 * sl;
-                            ku = ktab[du2 < 0 ? 0 : du2];
-                            kl = ktab[dl2 < 0 ? 0 : dl2];
-                        } else if constexpr (MODE == MODE_FP64) {
-                            const double nrm_i = norm[g];
-                            double d2u = up.nrm + nrm_i - 2.0 * su;
-                            double d2l = low.nrm + nrm_i - 2.0 * sl;
-                            ku = exp_neg_fx(gamma * dpos(d2u), expfx_s);
-                            kl = exp_neg_fx(gamma * dpos(d2l), expfx_s);
-                        } else {
-                            const float nf = normf[g];
-                            float d2u = norm_f32(up.nrm) + nf - 2.0f * su;
-                            float d2l = norm_f32(low.nrm) + nf - 2.0f * sl;
-                            // widened exactly by integer operations (a conversion
-                            // instruction would take a slot of the FP64 pipe)
-                            ku = widen_f32(__expf(-gammaf * fmaxf(d2u, 0.f)));
-                            kl = widen_f32(__expf(-gammaf * fmaxf(d2l, 0.f)));
-                        }
                         fi = fma(dl, kl, fma(du, ku, fi));
                         fj[r] = fi;
                         if (r == up.i) {
@@ -338,10 +413,76 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                         }
                     }
                     const uint8_t set = set_bits(sb);
-                    const unsigned long long kup = key_up(fi), klo = key_low(fi);
-                    if (st_up(set) && ki_less(kup, r, bku, biu)) { bku = kup; biu = r; bru = r; }
-                    if (st_low(set) && ki_less(klo, r, bkl, bil)) { bkl = klo; bil = r; brl = r; }
+                    const unsigned long long kf = dkey(fi);
+                    if (st_up(set) && ki_less(kf, r, bku, biu)) { bku = kf; biu = r; bru = r; }
+                    if (st_low(set) && ki_less(~kf, r, bkl, bil)) { bkl = ~kf; bil = r; brl = r; }
                 };
+                // this row's kernel values from its inner products, or from the
+                // cache; nv: the row's norm
+                auto kernel_values = [&](int r, int len, Acc su, Acc sl, double nv, double &ku, double &kl) {
+                    ku = kl = 0.0;
+                    if (first) return;
+                    if constexpr (MODE == MODE_BINARY) {
+                        int du2 = up.len + len - 2 * su, dl2 = low.len + len - 2 * sl;
+                        ku = ktab[du2 < 0 ? 0 : du2];
+                        kl = ktab[dl2 < 0 ? 0 : dl2];
+                    } else if constexpr (MODE == MODE_FP64) {
+                        if (hu) ku = kcu[r];
+                        else {
+                            ku = exp_neg_fx(gamma * dpos(up.nrm + nv - 2.0 * su), expfx_s);
+                            if (kc_on) kcu[r] = ku;
+                        }
+                        if (hl) kl = kcl[r];
+                        else {
+                            kl = exp_neg_fx(gamma * dpos(low.nrm + nv - 2.0 * sl), expfx_s);
+                            if (kc_on) kcl[r] = kl;
+                        }
+                    } else {
+                        // widened exactly by integer operations (a conversion
+                        // instruction would take a slot of the FP64 pipe)
+                        const float nf = norm_f32(nv);
+                        ku = widen_f32(__expf(-gammaf * fmaxf(norm_f32(up.nrm) + nf - 2.0f * su, 0.f)));
+                        kl = widen_f32(__expf(-gammaf * fmaxf(norm_f32(low.nrm) + nf - 2.0f * sl, 0.f)));
+                    }
+                };
+                auto row_norm = [&](int g) -> double {
+                    if constexpr (MODE == MODE_FP64) return norm[g];
+                    else if constexpr (MODE == MODE_MIXED) return norm_bits(normf[g]);
+                    else return 0.0;
+                };
+                auto finish_row = [&](int r, int g, int len, Acc su, Acc sl, double fi, uint8_t sb) {
+                    double ku, kl;
+                    kernel_values(r, len, su, sl, first ? 0.0 : row_norm(g), ku, kl);
+                    update_row(r, ku, kl, fi, sb);
+                };
+                if (hu && hl) {
+                    // both rows cached: a thread per row, coalesced
+                    if constexpr (KC_MODE) {
+                        for (int r0 = lo + tid - 32;; r0 += 4 * (kThreads - 32)) {
+                            double ku[4], kl[4], fi[4];
+                            uint8_t sb[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const int r = r0 + j * (kThreads - 32);
+                                ku[j] = kl[j] = fi[j] = 0.0;
+                                sb[j] = 0;
+                                if (r < hi) {
+                                    ku[j] = kcu[r];
+                                    kl[j] = kcl[r];
+                                    fi[j] = fj[r];
+                                    sb[j] = sj[r];
+                                }
+                            }
+                            wait_step();
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const int r = r0 + j * (kThreads - 32);
+                                if (r < hi) update_row(r, ku[j], kl[j], fi[j], sb[j]);
+                            }
+                            if (r0 - (tid - 32) + 4 * (kThreads - 32) >= hi) break;   // uniform
+                        }
+                    }
+                } else {
                 bool blocked = false;
                 if constexpr (LPR == 32) blocked = dense && d <= 256;
                 bool tiles = false;   // dense BF16 rows on the tensor cores
@@ -359,76 +500,101 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                         // the same map, so the dot products are unchanged.
                         const int g = lane >> 2, t = lane & 3;
                         const int nblk = d >> 5;
-                        // this warp's target fragments: [k-step][lane], k-step = 2 * block + h
-                        uint2 *frag = reinterpret_cast<uint2 *>(dsm + L.total) + (size_t)warp * 16 * 32;
+                        // the target fragments, [k-step][lane], k-step = 2 * block + h,
+                        // packed once per step by the row warps together
+                        for (int ks = warp - 1; ks < 2 * nblk; ks += kRowWarps) {
+                            uint32_t r0 = 0, r1 = 0;
+                            if (!first && g < 2) {
+                                const int c = 32 * (ks >> 1) + 8 * t + 4 * (ks & 1);
+                                float e[4];
 #pragma unroll
-                        for (int b = 0; b < 8; ++b) {
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                uint32_t r0 = 0, r1 = 0;
-                                if (!first && g < 2 && b < nblk) {
-                                    const int c = 32 * b + 8 * t + 4 * h;
-                                    float e[4];
-#pragma unroll
-                                    for (int x = 0; x < 4; ++x) e[x] = g == 0 ? T[c + x].x : T[c + x].y;
-                                    const __nv_bfloat162 p0 = __floats2bfloat162_rn(e[0], e[1]);
-                                    const __nv_bfloat162 p1 = __floats2bfloat162_rn(e[2], e[3]);
-                                    r0 = *reinterpret_cast<const uint32_t *>(&p0);
-                                    r1 = *reinterpret_cast<const uint32_t *>(&p1);
-                                }
-                                frag[(2 * b + h) * 32 + lane] = make_uint2(r0, r1);
+                                for (int x = 0; x < 4; ++x) e[x] = g == 0 ? T[c + x].x : T[c + x].y;
+                                const __nv_bfloat162 p0 = __floats2bfloat162_rn(e[0], e[1]);
+                                const __nv_bfloat162 p1 = __floats2bfloat162_rn(e[2], e[3]);
+                                r0 = *reinterpret_cast<const uint32_t *>(&p0);
+                                r1 = *reinterpret_cast<const uint32_t *>(&p1);
                             }
+                            frag[ks * 32 + lane] = make_uint2(r0, r1);
                         }
-                        __syncwarp();
-                        for (int base = lo + (warp - 1) * 16;; base += kRowWarps * 16) {
-                            const bool round0 = base == lo + (warp - 1) * 16;
-                            if (!round0 && base >= hi) break;
-                            const int ra = base + g, rb = base + g + 8;
-                            float acc[4] = {0.f, 0.f, 0.f, 0.f};
-                            if (!first) {
-                                const __nv_bfloat16 *pa = ra < hi ? dmat + (size_t)rows[ra] * d + 8 * t : nullptr;
-                                const __nv_bfloat16 *pb = rb < hi ? dmat + (size_t)rows[rb] * d + 8 * t : nullptr;
-                                // all blocks' loads in flight before their MMAs
+                        rows_bar_sync();
+                        // two tiles (32 rows, a unit) at a time: each row's two
+                        // sums are handed to one lane, so that the exponentials
+                        // and the FP64 updates run on whole warps
+                        const int step_warps = packed ? stage_warps : kRowWarps;
+                        for (int u = warp - 1; u < units && warp <= step_warps; u += step_warps) {
+                            const int base = lo + 32 * u;
+                            const int r = base + lane;
+                            const bool valid = r < hi;
+                            int grow = 0;
+                            double fi = 0.0, nv = 0.0;
+                            uint8_t sb = 0;
+                            if (valid) {
+                                grow = rows[r];
+                                fi = fj[r];
+                                sb = sj[r];
+                                nv = row_norm(grow);
+                            }
+                            float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+                            if (!first && packed) {
+                                wait_unit();
+                                const uint4 *sp = reinterpret_cast<const uint4 *>(stage) + lane;
 #pragma unroll
-                                for (int b0 = 0; b0 < 8; b0 += 8) {
-                                    uint4 uu[8], vv[8];
-#pragma unroll
-                                    for (int q = 0; q < 8; ++q) {
-                                        const int b = b0 + q;
-                                        uu[q] = (pa && b < nblk) ? __ldg(reinterpret_cast<const uint4 *>(pa + 32 * b)) : make_uint4(0, 0, 0, 0);
-                                        vv[q] = (pb && b < nblk) ? __ldg(reinterpret_cast<const uint4 *>(pb + 32 * b)) : make_uint4(0, 0, 0, 0);
-                                    }
-#pragma unroll
-                                    for (int q = 0; q < 8; ++q) {
-                                    const int b = b0 + q;
-                                    if (b < nblk) {
-                                        const uint4 u = uu[q], v = vv[q];
+                                for (int q = 0; q < 2; ++q) {
+#pragma unroll 4
+                                    for (int b = 0; b < nblk; ++b) {
+                                        const uint4 x = sp[((q * nblk + b) * 2) * 32], z = sp[((q * nblk + b) * 2 + 1) * 32];
                                         const uint2 f0 = frag[(2 * b) * 32 + lane], f1 = frag[(2 * b + 1) * 32 + lane];
-                                        asm volatile(
-                                            "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-                                            "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                                            : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3])
-                                            : "r"(u.x), "r"(v.x), "r"(u.y), "r"(v.y), "r"(f0.x), "r"(f0.y));
-                                        asm volatile(
-                                            "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-                                            "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                                            : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3])
-                                            : "r"(u.z), "r"(v.z), "r"(u.w), "r"(v.w), "r"(f1.x), "r"(f1.y));
+                                        mma_bf16_16816(acc[q], x.x, z.x, x.y, z.y, f0.x, f0.y);
+                                        mma_bf16_16816(acc[q], x.z, z.z, x.w, z.w, f1.x, f1.y);
                                     }
+                                }
+                                // the next unit while this one's rows are
+                                // finished (a warp's first unit again at the
+                                // end: it lands before the next step begins)
+                                __syncwarp();
+                                const int next = u + step_warps < units ? u + step_warps : warp - 1;
+                                if (next != u) {
+                                    fence_async_proxy();
+                                    issue_unit(next);
+                                }
+                            } else if (!first) {
+#pragma unroll
+                                for (int q = 0; q < 2; ++q) {
+                                    const int ia = __shfl_sync(0xffffffffu, grow, 16 * q + g);
+                                    const int ib = __shfl_sync(0xffffffffu, grow, 16 * q + g + 8);
+                                    const __nv_bfloat16 *pa = base + 16 * q + g < hi ? dmat + (size_t)ia * d + 8 * t : nullptr;
+                                    const __nv_bfloat16 *pb = base + 16 * q + g + 8 < hi ? dmat + (size_t)ib * d + 8 * t : nullptr;
+#pragma unroll 4
+                                    for (int b = 0; b < nblk; ++b) {
+                                        const uint4 x = pa ? __ldg(reinterpret_cast<const uint4 *>(pa + 32 * b)) : make_uint4(0, 0, 0, 0);
+                                        const uint4 z = pb ? __ldg(reinterpret_cast<const uint4 *>(pb + 32 * b)) : make_uint4(0, 0, 0, 0);
+                                        const uint2 f0 = frag[(2 * b) * 32 + lane], f1 = frag[(2 * b + 1) * 32 + lane];
+                                        mma_bf16_16816(acc[q], x.x, z.x, x.y, z.y, f0.x, f0.y);
+                                        mma_bf16_16816(acc[q], x.z, z.z, x.w, z.w, f1.x, f1.y);
                                     }
                                 }
                             }
-                            // lanes with t == 0 hold the two sums of rows ra and rb
-                            const bool lead = t == 0;
-                            double fa = 0.0, fb = 0.0;
-                            uint8_t sa = 0, sbb = 0;
-                            int ga = 0, gb = 0;
-                            if (lead && ra < hi) { ga = rows[ra]; fa = fj[ra]; sa = sj[ra]; }
-                            if (lead && rb < hi) { gb = rows[rb]; fb = fj[rb]; sbb = sj[rb]; }
+                            // the sums of row base + lane: tile lane >> 4, row
+                            // lane & 15, held by lane 4 (lane & 7) as (acc[2 s],
+                            // acc[2 s + 1]), s = (lane >> 3) & 1
+                            const int src = 4 * (lane & 7);
+                            const int qq = lane >> 4, ss = (lane >> 3) & 1;
+                            float su = 0.f, sl = 0.f;
+#pragma unroll
+                            for (int q = 0; q < 2; ++q) {
+#pragma unroll
+                                for (int s2 = 0; s2 < 2; ++s2) {
+                                    const float x = __shfl_sync(0xffffffffu, acc[q][2 * s2], src);
+                                    const float z = __shfl_sync(0xffffffffu, acc[q][2 * s2 + 1], src);
+                                    if (q == qq && s2 == ss) { su = x; sl = z; }
+                                }
+                            }
+                            double ku = 0.0, kl = 0.0;
+                            if (valid) kernel_values(r, d, su, sl, nv, ku, kl);
                             wait_step();
-                            if (lead && ra < hi) finish_row(ra, ga, d, acc[0], acc[1], fa, sa);
-                            if (lead && rb < hi) finish_row(rb, gb, d, acc[2], acc[3], fb, sbb);
+                            if (valid) update_row(r, ku, kl, fi, sb);
                         }
+                        wait_step();
                     }
                 } else if (blocked) {
                     if constexpr (LPR == 32 && MODE == MODE_MIXED) {
@@ -600,9 +766,12 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                                 sl += __shfl_xor_sync(0xffffffffu, sl, o);
                             }
                         }
+                        double ku = 0.0, kl = 0.0;
+                        if (valid && gl == 0) kernel_values(r, (int)(p1 - p0), su, sl, first ? 0.0 : row_norm(g), ku, kl);
                         wait_step();
-                        if (valid && gl == 0) finish_row(r, g, (int)(p1 - p0), su, sl, fi, sb);
+                        if (valid && gl == 0) update_row(r, ku, kl, fi, sb);
                     }
+                }
                 }
             }
             // payload of a job row (job-local index r)
@@ -640,6 +809,14 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 if (i2 != INT_MAX && bil == i2) sh.wlow[warp] = make_side(brl);
             }
             __syncthreads();
+            // both rows are stored from here on (all threads have read this
+            // step's bits; the cluster barriers order the next step's reads)
+            if (kc_on && !first && tid == 0) {
+                const uint32_t bu = 1u << (up.i & 31), bl = 1u << (low.i & 31);
+                const bool same = (up.i >> 5) == (low.i >> 5);
+                kdir[up.i >> 5] = kd_wu | bu | (same ? bl : 0u);
+                if (!same) kdir[low.i >> 5] = kd_wl | bl;
+            }
             // ---- 4. candidate exchange inside the cluster
             if (warp == 0) {
                 unsigned long long k1 = lane < kWarps ? sh.wkup[lane] : kNoKey;
@@ -709,6 +886,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             first = false;
         }
 
+        wait_unit();   // the stage is free and the packed rows may be rewritten
         // ---- job results: b (Section III-A) and the objective from partial sums
         {
             BatchFinish pf = {0, 0, 0, 0, 0, {0, 0}};
@@ -759,7 +937,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 R.b = t.n0 > 0 ? t.sum_f0 / (double)t.n0 : 0.5 * (up.f + low.f);
                 R.objective = t.sum_a - 0.5 * t.sum_ayfy;
                 R.iters = iter;
-                R.status = status_code;
+                R.status = PACK_MODE && sh.stage_bad ? 2 : status_code;
                 R.n_sv = (int32_t)t.nsv;
                 B.results[job] = R;
                 if (B.done) {
@@ -798,10 +976,12 @@ void *batch_fn(int mode, int lpr)
 }  // namespace
 }  // namespace smo
 
-size_t smo_batch_smem(int mode, int d, int ktab_len, int maxnnz)
+size_t smo_batch_smem(int mode, int d, int ktab_len, int maxnnz, int kdir_words)
 {
-    // mixed mode: each warp's target fragments of the tensor-core row tiles
-    return smo_layout(mode, d, ktab_len, maxnnz, 0, 0, 0).total + (mode == MODE_MIXED ? smo::kFragBytes : 0);
+    // mixed mode: the target fragments of the tensor-core row tiles; then the
+    // kernel-row cache's directory
+    return smo_layout(mode, d, ktab_len, maxnnz, 0, 0, 0).total + (mode == MODE_MIXED ? smo::kFragBytes : 0) +
+           4 * (size_t)kdir_words;
 }
 
 int smo_batch_max_clusters(int mode, int lpr, int dense, size_t smem, int cs)

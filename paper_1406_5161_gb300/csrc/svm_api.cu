@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <condition_variable>
@@ -73,7 +74,7 @@ struct Fail {
 // kPoolKeepBytes between calls and gives back the rest; what it keeps is given
 // back too when an allocation fails for want of memory. The driver orders its
 // reuse across streams and threads.
-constexpr size_t kPoolKeepBytes = (size_t)512 << 20;
+constexpr size_t kPoolKeepBytes = (size_t)4 << 30;
 constexpr int kPoolDevices = 64;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kPoolDevices] = {};
@@ -2323,7 +2324,7 @@ void batch_prepare(Arena &ar, const svm_csr *X, int precision, cudaStream_t st, 
         B.d_eff = d_pad;
     }
     B.ktab_len = B.mode == MODE_BINARY ? 2 * D.maxnnz + 1 : 0;
-    B.smem = smo_batch_smem(B.mode, B.d_eff, B.ktab_len, D.maxnnz);
+    B.smem = smo_batch_smem(B.mode, B.d_eff, B.ktab_len, D.maxnnz, 0);
     if (B.smem > smem_limit() - 12288) {
         set_err("d = %lld exceeds the shared-memory target rows of the batched solver", (long long)D.d);
         throw Fail{SVM_ERR_UNSUPPORTED};
@@ -2441,15 +2442,23 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
         J.f = f + offs[j];
         J.status = status + offs[j];
     }
+    // the work-list holds the jobs with the most rows first, so that the last
+    // ones to be taken are short (order[k]: the k-th job of the list)
+    std::vector<int> order(n_jobs);
+    for (int j = 0; j < n_jobs; ++j) order[j] = j;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return hj[a].nrows > hj[b].nrows; });
+    std::vector<BatchJobDev> list(n_jobs);
+    for (int k = 0; k < n_jobs; ++k) list[k] = hj[order[k]];
     BatchJobDev *djobs = ar.alloc<BatchJobDev>(n_jobs);
-    CK(cudaMemcpyAsync(djobs, hj.data(), sizeof(BatchJobDev) * n_jobs, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(djobs, list.data(), sizeof(BatchJobDev) * n_jobs, cudaMemcpyHostToDevice, st));
     int *bad = ar.alloc<int>(n_jobs);
     k_job_check<<<n_jobs, 256, 0, st>>>(n_jobs, djobs, D.n, bad);
     CK(cudaGetLastError());
     ++launches;
-    std::vector<int> hbad(n_jobs);
-    CK(cudaMemcpyAsync(hbad.data(), bad, sizeof(int) * n_jobs, cudaMemcpyDeviceToHost, st));
+    std::vector<int> lbad(n_jobs), hbad(n_jobs);
+    CK(cudaMemcpyAsync(lbad.data(), bad, sizeof(int) * n_jobs, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    for (int k = 0; k < n_jobs; ++k) hbad[order[k]] = lbad[k];
     for (int j = 0; j < n_jobs; ++j) {
         if (hbad[j] == 1) ARG_FAIL("job %d: row ids out of range or labels not +-1", j);
         if (hbad[j] == 2) ARG_FAIL("job %d: both classes must be present", j);
@@ -2465,6 +2474,43 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
     A.results = dres;
     A.ktab_len = P.ktab_len;
     A.maxnnz = D.maxnnz;
+
+    int64_t most_rows = 0, least_rows = INT64_MAX;
+    for (int j = 0; j < n_jobs; ++j) {
+        most_rows = std::max<int64_t>(most_rows, jobs[j].n_rows);
+        least_rows = std::min<int64_t>(least_rows, jobs[j].n_rows);
+    }
+    // a buffer of the call, or NULL where there is no room for it
+    auto try_alloc = [&](size_t bytes) -> void * {
+        try {
+            return ar.alloc<unsigned char>(bytes);
+        } catch (const Fail &) {
+            g_err.clear();
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+    };
+    // Dense BF16 rows on the tensor cores: the packed rows' buffer and the
+    // stages in shared memory (as many row warps as fit, at least half).
+    void *pack_buf = nullptr;
+    size_t pack_have = 0;
+    auto set_pack = [&](BatchArgs &a, BatchPlan &q, int l, int c, int ncl) {
+        if (P.mode != MODE_MIXED || !P.dense || l != 16 || P.d_eff % 32 != 0 || P.d_eff > 256) return;
+        const size_t unit = 64 * (size_t)P.d_eff, lim = smem_limit() - 12288;
+        if (q.smem + 128 + 8 * unit > lim) return;
+        const int64_t stride = ((most_rows + c - 1) / c + 32) / 32 * (int64_t)unit;
+        const size_t bytes = (size_t)stride * c * ncl;
+        if (bytes > pack_have) {
+            pack_buf = try_alloc(bytes);
+            pack_have = pack_buf ? bytes : 0;
+        }
+        if (!pack_buf) return;
+        a.stage_warps = (int)std::min<size_t>(15, (lim - q.smem - 128) / unit);
+        a.stage_bytes = (int)unit;
+        a.pack = pack_buf;
+        a.pack_stride = stride;
+        q.smem += 128 + (size_t)a.stage_warps * unit;
+    };
 
     // ---- launch shape: given, or picked by timing candidates on a sample
     int cs = cfg->cluster_size, lpr = cfg->lanes_per_row;
@@ -2498,7 +2544,10 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
             for (int l : lprs) {
                 const int maxc = batch_clusters(P, l, c);
                 if (maxc < 1) continue;
-                const float ms = batch_run(P, S, l, c, std::min(maxc, ns), next_job, st, &launches);
+                BatchPlan Q = P;
+                BatchArgs SQ = S;
+                set_pack(SQ, Q, l, c, std::min(maxc, ns));
+                const float ms = batch_run(Q, SQ, l, c, std::min(maxc, ns), next_job, st, &launches);
                 CK(cudaMemcpy(sres.data(), dres, sizeof(BatchResultDev) * ns, cudaMemcpyDeviceToHost));
                 int64_t it = 0;
                 for (auto &r : sres) it += r.iters;
@@ -2520,16 +2569,46 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
         cfg->lanes_per_row = lpr;
     }
     if (tune_only) return SVM_OK;
-    const int maxc = batch_clusters(P, lpr, cs);
+    int maxc = batch_clusters(P, lpr, cs);
     if (maxc < 1) {
         set_err("cluster size %d does not fit this device", cs);
         throw Fail{SVM_ERR_UNSUPPORTED};
     }
-    int ncl = std::min(maxc, n_jobs);
-    if (cfg->clusters > 0) ncl = std::min(ncl, cfg->clusters);
+    auto in_flight = [&](int most) {
+        const int k = std::min(most, n_jobs);
+        return cfg->clusters > 0 ? std::min(k, cfg->clusters) : k;
+    };
+    int ncl = in_flight(maxc);
+    // Kernel-row cache (FP64): each cluster's job keeps the kernel rows it
+    // computes, all of them when its kernel matrix fits the cluster's part of
+    // the budget (svm_train's). 45 jobs of 1,500 x 20 rows: 54 ms without, 33
+    // with it. Mixed rows gain nothing: of the rows of the 90 one-vs-one jobs
+    // (2,200-5,800 x 256) a quarter of the steps find both, 140 -> 126 ms, and
+    // mapping the 10 GB takes the difference.
+    if (P.mode == MODE_FP64) {
+        auto matrix_bytes = [&](int64_t m) { return m * ((m + 31) / 32 * 32) * 8; };
+        const int words = (int)std::min<int64_t>((most_rows + 31) / 32, 4096);
+        BatchPlan Q = P;
+        Q.smem = smo_batch_smem(P.mode, P.d_eff, P.ktab_len, D.maxnnz, words);
+        const int qmax = Q.smem <= smem_limit() - 12288 ? batch_clusters(Q, lpr, cs) : 0;
+        size_t fr = 0, tot = 0;
+        if (qmax >= maxc && cudaMemGetInfo(&fr, &tot) == cudaSuccess) {
+            const int64_t stride = std::min<int64_t>(matrix_bytes(most_rows),
+                                                     (int64_t)std::min<size_t>(fr / 2, (size_t)32 << 30) / ncl) / 256 * 256;
+            if (stride >= matrix_bytes(least_rows)) {
+                if (void *kc = try_alloc((size_t)stride * ncl)) {
+                    P.smem = Q.smem;
+                    A.kc = kc;
+                    A.kc_stride = stride;
+                    A.kdir_words = words;
+                }
+            }
+        }
+    }
+    set_pack(A, P, lpr, cs, ncl);
     const float ms = batch_run(P, A, lpr, cs, ncl, next_job, st, &launches);
-    std::vector<BatchResultDev> hres(n_jobs);
-    CK(cudaMemcpyAsync(hres.data(), dres, sizeof(BatchResultDev) * n_jobs, cudaMemcpyDeviceToHost, st));
+    std::vector<BatchResultDev> lres(n_jobs), hres(n_jobs);
+    CK(cudaMemcpyAsync(lres.data(), dres, sizeof(BatchResultDev) * n_jobs, cudaMemcpyDeviceToHost, st));
     if (X->on_device) {
         for (int j = 0; j < n_jobs; ++j)
             CK(cudaMemcpyAsync(jobs[j].alpha_out, alpha + offs[j], 8 * jobs[j].n_rows, cudaMemcpyDeviceToDevice,
@@ -2542,9 +2621,14 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
         for (int j = 0; j < n_jobs; ++j)
             std::memcpy(jobs[j].alpha_out, ha.data() + offs[j], 8 * jobs[j].n_rows);
     }
+    for (int k = 0; k < n_jobs; ++k) hres[order[k]] = lres[k];
     int64_t iters = 0;
     int rc = SVM_OK;
     for (int j = 0; j < n_jobs; ++j) {
+        if (hres[j].status == 2) {
+            set_err("a wait in the batched SMO kernel exceeded its time limit");
+            throw Fail{SVM_ERR_TIMEOUT};
+        }
         svm_result &R = results[j];
         R.b = hres[j].b;
         R.b_up = hres[j].b_up;
@@ -3302,7 +3386,7 @@ int svm_server_create(const svm_server_config *config, svm_server **out)
         Server &V = S->impl;
         V.cfg = c;
         V.mode = c.precision == SVM_FP64 ? MODE_FP64 : MODE_MIXED;
-        V.smem = smo_batch_smem(V.mode, c.max_d, 0, c.max_d);
+        V.smem = smo_batch_smem(V.mode, c.max_d, 0, c.max_d, 0);
         if (V.smem > smem_limit() - 12288) ARG_FAIL("max_d = %d does not fit the engine's shared memory", c.max_d);
         V.nclusters = smo_batch_max_clusters(V.mode, c.lanes_per_row, 0, V.smem, c.cluster_size);
         if (V.nclusters < 1) ARG_FAIL("cluster_size %d does not fit this device", c.cluster_size);

@@ -185,7 +185,7 @@ struct BatchJobDev {
 struct BatchResultDev {
     double b, b_up, b_low, objective;
     int64_t iters;
-    int32_t status;            // 0 converged, 1 iteration limit
+    int32_t status;            // 0 converged, 1 iteration limit, 2 a wait gave up
     int32_t n_sv;
 };
 
@@ -206,9 +206,22 @@ struct BatchArgs {
     const int *shutdown;       // host sets to stop the engine
     int *done;                 // per slot: set to 1 when the result is written
     int64_t idle_ns;           // an engine cluster leaves after this long without work
+    // kernel-row cache (NULL: none): kc_stride bytes per cluster, used by the
+    // FP64 jobs whose whole kernel matrix fits; kdir_words words of
+    // shared memory hold a valid bit per row
+    void *kc;
+    int64_t kc_stride;
+    int32_t kdir_words;
+    // dense BF16 rows on the tensor cores (16 lanes per row): pack_stride bytes
+    // per CTA for its rows in fragment order (NULL: rows read from the matrix),
+    // and stage_warps stages of stage_bytes in shared memory behind the rest
+    int32_t stage_warps, stage_bytes;
+    int32_t pad2;
+    void *pack;
+    int64_t pack_stride;
 };
 
-size_t smo_batch_smem(int mode, int d, int ktab_len, int maxnnz);
+size_t smo_batch_smem(int mode, int d, int ktab_len, int maxnnz, int kdir_words);
 int smo_batch_max_clusters(int mode, int lpr, int dense, size_t smem, int cs);
 cudaError_t launch_smo_batch(int mode, int lpr, int dense, const BatchArgs &a, size_t smem, int cs,
                              int nclusters, cudaStream_t st);
