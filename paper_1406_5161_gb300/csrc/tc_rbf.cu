@@ -25,6 +25,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "svm_internal.cuh"
@@ -34,7 +35,6 @@ namespace {
 
 constexpr int kTile = 128;            // rows per query tile and per SV tile (M = N)
 constexpr int kKB = 64;               // BF16 elements per 128-byte swizzle row
-constexpr int kTcThreads = 320;       // warp 0 loads, warp 1 MMA, warps 2..9 epilogue
 constexpr int kMaxKBlocks = 4;        // d_pad <= 256
 constexpr uint32_t kTileBytes = kTile * kKB * 2;   // 16 KiB per k-block tile
 constexpr long long kWaitLimit = 1ll << 26;        // mbarrier polls before giving up
@@ -157,6 +157,20 @@ __device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, un
     return r;
 }
 
+__device__ __forceinline__ void tmem_ld_x32(uint32_t *r, uint32_t addr)
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(addr)
+        : "memory");
+}
+
 __device__ __forceinline__ float ex2_approx(float x)
 {
     float y;
@@ -181,7 +195,15 @@ __device__ __forceinline__ float ex2_approx(float x)
 // acce[b]  : the epilogue has read accumulator b (one arrival per warp).
 // Tile t uses slot t % stages (round t / stages) and accumulator t & 1 (use
 // t >> 1); the k-th completion of a barrier has parity k & 1.
-constexpr int kEpiWarps = 8;
+constexpr int kEpiWarps = 8;          // epilogue warps per accumulator
+// Query tiles per CTA (RT). The epilogue's constants of a column, 8 bytes read
+// from shared memory into every lane, bound it with one tile: a warp-wide
+// 16-byte read takes 4 clocks of the SM's data path whatever its addresses, 8
+// clocks per pair and scheduler against 6.5 of issue. With two tiles a thread
+// holds a row of each and reads the constants once for both; one such CTA per
+// SM (512 tensor-memory columns), whose 16 epilogue warps take the support
+// tiles in turn, 8 each.
+__host__ __device__ constexpr int tc_threads(int rt) { return 64 + 32 * kEpiWarps * rt; }
 constexpr int kMaxStages = 4;
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
@@ -222,27 +244,46 @@ __device__ __forceinline__ bool mbar_wait_or_fail(uint64_t *bar, uint32_t parity
     }
 }
 
-__global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constant__ CUtensorMap mapZ,
-                                                            const __grid_constant__ CUtensorMap mapX,
-                                                            TcArgs a)
+// 32 columns of one row: (columns j, j + 1) partial sums in two chains; the
+// FP32 arithmetic runs on packed column pairs (f32x2), the same IEEE result in
+// each lane as the scalar form. FACTORED: see the kernel.
+template <bool FACTORED>
+__device__ __forceinline__ void epi_quad(const uint32_t *rr, const ulonglong2 &x4, const ulonglong2 &c4,
+                                         unsigned long long g2v, unsigned long long zc2, float nzc,
+                                         unsigned long long &partA, unsigned long long &partB)
+{
+    const float cap = FACTORED ? nzc : 0.f;
+    const unsigned long long xa = FACTORED ? x4.x : add_f32x2(x4.x, zc2), xb = FACTORED ? x4.y : add_f32x2(x4.y, zc2);
+    float e0, e1, e2, e3;
+    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(rr[0]), __uint_as_float(rr[1])), g2v, xa), e0, e1);
+    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(rr[2]), __uint_as_float(rr[3])), g2v, xb), e2, e3);
+    const unsigned long long k01 = pack_f32x2(ex2_approx(fminf(e0, cap)), ex2_approx(fminf(e1, cap)));
+    const unsigned long long k23 = pack_f32x2(ex2_approx(fminf(e2, cap)), ex2_approx(fminf(e3, cap)));
+    partA = fma_f32x2(c4.x, k01, partA);
+    partB = fma_f32x2(c4.y, k23, partB);
+}
+
+template <int RT>
+__global__ void __launch_bounds__(tc_threads(RT), RT == 1 ? 2 : 1)
+    tc_rbf_kernel(const __grid_constant__ CUtensorMap mapZ, const __grid_constant__ CUtensorMap mapX, TcArgs a)
 {
     extern __shared__ __align__(1024) unsigned char dsm_raw[];
     // 1024-byte alignment for the swizzled tiles
     unsigned char *dsm = reinterpret_cast<unsigned char *>(((uintptr_t)dsm_raw + 1023) & ~(uintptr_t)1023);
     const int S = a.stages;
     const size_t tile_all = (size_t)a.kblocks * kTileBytes;   // one tile, all k-blocks
-    unsigned char *tileA = dsm;                               // the query tile
-    unsigned char *tileB = dsm + tile_all;                    // [S][kblocks][16 KiB]
+    unsigned char *tileA = dsm;                               // the query tiles
+    unsigned char *tileB = dsm + RT * tile_all;               // [S][kblocks][16 KiB]
     __shared__ __align__(8) uint64_t bar_q, bar_full[kMaxStages], bar_empty[kMaxStages], bar_accf[2],
         bar_acce[2], bar_drain;
     __shared__ uint32_t tmem_base;
     __shared__ __align__(16) float s_xc[kMaxStages][kTile], s_coef[kMaxStages][kTile];
-    __shared__ double s_acc[kTile];   // the second column half's row sums
+    __shared__ double s_acc[2 * RT][RT * kTile];   // the epilogue warps' row sums, by tile turn and column half
     __shared__ int s_fail, s_last;
     const volatile int *fail = &s_fail;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t q0 = (int64_t)blockIdx.x * kTile;
+    const int64_t q0 = (int64_t)blockIdx.x * (RT * kTile);
     if (tid == 0) {
         mbar_init(&bar_q, 1);
         for (int k = 0; k < kMaxStages; ++k) {
@@ -260,7 +301,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(&tmem_base)), "r"(2 * kTile) : "memory");
+                     ::"r"(smem_u32(&tmem_base)), "r"(2 * RT * kTile) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -275,16 +316,21 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
     bool ok = true;
     int64_t issued = 0;         // producer: support tiles whose loads were issued
     bool q_issued = false;
-    const int quad = warp & 3, half = (warp - 2) >> 2;    // epilogue warps
-    const int my_row = quad * 32 + lane;                  // TMEM lane = query row in tile
-    double acc = 0.0;
+    // epilogue warps: turn (support tiles t = turn, turn + RT, ..), column half
+    // and 32-lane quadrant of tensor memory
+    const int quad = warp & 3, half = ((warp - 2) >> 2) & 1, turn = (warp - 2) >> 3;
+    const int my_row = quad * 32 + lane;                  // TMEM lane = query row in each tile
+    double acc[RT];
+#pragma unroll
+    for (int i = 0; i < RT; ++i) acc[i] = 0.0;
 
     if (warp == 0) {
         // ---- producer
         if (lane == 0) {
-            mbar_expect_tx(&bar_q, (uint32_t)tile_all);
-            for (int kb = 0; kb < a.kblocks; ++kb)
-                tma_load_2d(tileA + (size_t)kb * kTileBytes, &mapZ, kb * kKB, (int)q0, &bar_q);
+            mbar_expect_tx(&bar_q, (uint32_t)(RT * tile_all));
+            for (int i = 0; i < RT; ++i)
+                for (int kb = 0; kb < a.kblocks; ++kb)
+                    tma_load_2d(tileA + i * tile_all + (size_t)kb * kTileBytes, &mapZ, kb * kKB, (int)q0 + i * kTile, &bar_q);
             q_issued = true;
             for (int64_t t = 0; t < ntiles; ++t) {
                 const int sl = (int)(t % S);
@@ -318,9 +364,10 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const unsigned char *tb = tileB + (size_t)sl * tile_all;
-                const uint32_t dcol = tmem + (uint32_t)(b * kTile);
+                for (int i = 0; i < RT; ++i)
                 for (int kb = 0; kb < a.kblocks; ++kb) {
-                    const uint32_t sa = smem_u32(tileA + (size_t)kb * kTileBytes);
+                    const uint32_t dcol = tmem + (uint32_t)((b * RT + i) * kTile);
+                    const uint32_t sa = smem_u32(tileA + i * tile_all + (size_t)kb * kTileBytes);
                     const uint32_t sb = smem_u32(tb + (size_t)kb * kTileBytes);
 #pragma unroll
                     for (int ks = 0; ks < kKB / 16; ++ks) {
@@ -345,19 +392,28 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
         }
     } else {
         // ---- epilogue
-        const int64_t q = q0 + my_row;
-        const float zc = (q < a.nq) ? a.zc[q] : 0.f;
-        const unsigned long long zc2 = pack_f32x2(zc, zc), g2v = pack_f32x2(a.g2, a.g2);
         // The row's scaled norm factors out of the sum:
         //   sum_j c_j 2^min(g2 dot_j + xc_j + zc, 0)
         //     = 2^zc sum_j c_j 2^min(g2 dot_j + xc_j, -zc),
         // one addition less per pair; 2^zc is applied once per tile. A warp
         // with a row whose 2^-zc would leave FP32 (-zc > 120) keeps the
         // per-pair form.
-        const float nzc = -zc;
-        const bool factored = !__any_sync(0xffffffffu, nzc > 120.f);
-        const double row_scale = factored ? exp2((double)zc) : 1.0;
-        for (int64_t t = 0; t < ntiles; ++t) {
+        const unsigned long long g2v = pack_f32x2(a.g2, a.g2);
+        float nzc[RT];
+        unsigned long long zc2[RT];
+        bool factored[RT], all_factored = true;
+        double row_scale[RT];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            const int64_t q = q0 + i * kTile + my_row;
+            const float zc = (q < a.nq) ? a.zc[q] : 0.f;
+            nzc[i] = -zc;
+            zc2[i] = pack_f32x2(zc, zc);
+            factored[i] = !__any_sync(0xffffffffu, nzc[i] > 120.f);
+            all_factored &= factored[i];
+            row_scale[i] = factored[i] ? exp2((double)zc) : 1.0;
+        }
+        for (int64_t t = turn; t < ntiles; t += RT) {
             const int sl = (int)(t % S), b = (int)(t & 1);
             const int64_t r = t / S, u = t >> 1;
             const bool w_ok = mbar_wait_or_fail(&bar_accf[b], (uint32_t)(u & 1), fail) &&
@@ -367,72 +423,60 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // (columns j, j + 1) partial sums, two chains
-            unsigned long long partA = pack_f32x2(0.f, 0.f), partB = partA;
-#pragma unroll 1
-            for (int c0 = half * (kTile / 2); c0 < (half + 1) * (kTile / 2); c0 += 32) {
-                uint32_t rr[32];
-                const uint32_t addr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * kTile + c0);
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                    "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                    "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                    : "=r"(rr[0]), "=r"(rr[1]), "=r"(rr[2]), "=r"(rr[3]), "=r"(rr[4]), "=r"(rr[5]), "=r"(rr[6]),
-                      "=r"(rr[7]), "=r"(rr[8]), "=r"(rr[9]), "=r"(rr[10]), "=r"(rr[11]), "=r"(rr[12]),
-                      "=r"(rr[13]), "=r"(rr[14]), "=r"(rr[15]), "=r"(rr[16]), "=r"(rr[17]), "=r"(rr[18]),
-                      "=r"(rr[19]), "=r"(rr[20]), "=r"(rr[21]), "=r"(rr[22]), "=r"(rr[23]), "=r"(rr[24]),
-                      "=r"(rr[25]), "=r"(rr[26]), "=r"(rr[27]), "=r"(rr[28]), "=r"(rr[29]), "=r"(rr[30]),
-                      "=r"(rr[31])
-                    : "r"(addr)
-                    : "memory");
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                // the FP32 arithmetic runs on packed column pairs (f32x2),
-                // the same IEEE result in each lane as the scalar form
-                const float4 *xs = reinterpret_cast<const float4 *>(&s_xc[sl][c0]);
-                const float4 *cs = reinterpret_cast<const float4 *>(&s_coef[sl][c0]);
-                if (factored) {
+            unsigned long long part[RT][2];
 #pragma unroll
-                    for (int v = 0; v < 8; ++v) {
-                        const float4 x4 = xs[v], c4 = cs[v];   // the same address in every lane
-                        const int j = 4 * v;
-                        float e0, e1, e2, e3;
-                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(rr[j]), __uint_as_float(rr[j + 1])), g2v,
-                                               pack_f32x2(x4.x, x4.y)), e0, e1);
-                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(rr[j + 2]), __uint_as_float(rr[j + 3])),
-                                               g2v, pack_f32x2(x4.z, x4.w)), e2, e3);
-                        const unsigned long long k01 = pack_f32x2(ex2_approx(fminf(e0, nzc)), ex2_approx(fminf(e1, nzc)));
-                        const unsigned long long k23 = pack_f32x2(ex2_approx(fminf(e2, nzc)), ex2_approx(fminf(e3, nzc)));
-                        partA = fma_f32x2(pack_f32x2(c4.x, c4.y), k01, partA);
-                        partB = fma_f32x2(pack_f32x2(c4.z, c4.w), k23, partB);
+            for (int i = 0; i < RT; ++i) part[i][0] = part[i][1] = pack_f32x2(0.f, 0.f);
+            // 64 values per thread at once (one tile: the 64 columns of this
+            // half; two: 32 columns of each), so that a wait for tensor memory
+            // covers that many; the accumulator is free for the MMA once the
+            // last of them are in registers
+            constexpr int kCols = 64 / RT;
+#pragma unroll
+            for (int c0 = 0; c0 < kTile / 2; c0 += kCols) {
+                uint32_t rr[64];
+                const uint32_t addr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * RT * kTile + half * (kTile / 2) + c0);
+                tmem_ld_x32(rr, addr);
+                tmem_ld_x32(rr + 32, RT == 1 ? addr + 32 : addr + kTile);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (c0 + kCols == kTile / 2) {
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar_acce[b]);
+                }
+                const ulonglong2 *xs = reinterpret_cast<const ulonglong2 *>(&s_xc[sl][half * (kTile / 2) + c0]);
+                const ulonglong2 *cs = reinterpret_cast<const ulonglong2 *>(&s_coef[sl][half * (kTile / 2) + c0]);
+                if (all_factored) {
+#pragma unroll
+                    for (int v = 0; v < kCols / 4; ++v) {
+                        const ulonglong2 x4 = xs[v], c4 = cs[v];   // the same address in every lane
+#pragma unroll
+                        for (int i = 0; i < RT; ++i)
+                            epi_quad<true>(rr + i * kCols + 4 * v, x4, c4, g2v, zc2[i], nzc[i], part[i][0], part[i][1]);
                     }
                 } else {
 #pragma unroll
-                    for (int v = 0; v < 8; ++v) {
-                        const float4 x4 = xs[v], c4 = cs[v];
-                        const int j = 4 * v;
-                        float e0, e1, e2, e3;
-                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(rr[j]), __uint_as_float(rr[j + 1])), g2v,
-                                               add_f32x2(pack_f32x2(x4.x, x4.y), zc2)), e0, e1);
-                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(rr[j + 2]), __uint_as_float(rr[j + 3])),
-                                               g2v, add_f32x2(pack_f32x2(x4.z, x4.w), zc2)), e2, e3);
-                        const unsigned long long k01 = pack_f32x2(ex2_approx(fminf(e0, 0.f)), ex2_approx(fminf(e1, 0.f)));
-                        const unsigned long long k23 = pack_f32x2(ex2_approx(fminf(e2, 0.f)), ex2_approx(fminf(e3, 0.f)));
-                        partA = fma_f32x2(pack_f32x2(c4.x, c4.y), k01, partA);
-                        partB = fma_f32x2(pack_f32x2(c4.z, c4.w), k23, partB);
+                    for (int v = 0; v < kCols / 4; ++v) {
+                        const ulonglong2 x4 = xs[v], c4 = cs[v];
+#pragma unroll
+                        for (int i = 0; i < RT; ++i) {
+                            if (factored[i])
+                                epi_quad<true>(rr + i * kCols + 4 * v, x4, c4, g2v, zc2[i], nzc[i], part[i][0], part[i][1]);
+                            else
+                                epi_quad<false>(rr + i * kCols + 4 * v, x4, c4, g2v, zc2[i], nzc[i], part[i][0], part[i][1]);
+                        }
                     }
                 }
             }
-            float pa0, pa1, pb0, pb1;
-            unpack_f32x2(partA, pa0, pa1);
-            unpack_f32x2(partB, pb0, pb1);
-            acc += (double)((pa0 + pa1) + (pb0 + pb1)) * row_scale;
-            // this warp is done with accumulator b and with slot sl
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&bar_acce[b]);
-                mbar_arrive(&bar_empty[sl]);
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                float pa0, pa1, pb0, pb1;
+                unpack_f32x2(part[i][0], pa0, pa1);
+                unpack_f32x2(part[i][1], pb0, pb1);
+                acc[i] += (double)((pa0 + pa1) + (pb0 + pb1)) * row_scale[i];
             }
+            // this warp is done with slot sl
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_empty[sl]);
         }
     }
     if (!ok && lane == 0) {
@@ -456,44 +500,57 @@ __global__ void __launch_bounds__(kTcThreads) tc_rbf_kernel(const __grid_constan
             if (q_issued) (void)mbar_wait(&bar_q, 0);
         }
     } else {
-        // the two column halves of a row meet in shared memory (fixed order)
-        const int64_t q = q0 + my_row;
-        if (warp >= 2 && half == 1) s_acc[my_row] = acc;
+        // a row's sums (by column half and tile turn) meet in shared memory, in
+        // a fixed order; one epilogue thread per row then has its total
+        if (warp >= 2) {
+#pragma unroll
+            for (int i = 0; i < RT; ++i) s_acc[2 * turn + half][i * kTile + my_row] = acc[i];
+        }
         __syncthreads();
-        if (warp >= 2 && half == 0) acc += s_acc[my_row];
-        bool mine = warp >= 2 && half == 0 && q < a.nq;
+        const int row = tid - 64;                 // epilogue threads 0 .. RT kTile - 1
+        const int64_t q = q0 + row;
+        const bool owner = row >= 0 && row < RT * kTile;
+        bool mine = owner && q < a.nq;
+        double sum = 0.0;
+        if (owner) {
+            sum = s_acc[0][row];
+#pragma unroll
+            for (int k = 1; k < 2 * RT; ++k) sum += s_acc[k][row];
+        }
         if (splits > 1) {
-            if (mine) a.part[(size_t)blockIdx.y * a.nq + q] = acc;
+            if (mine) a.part[(size_t)blockIdx.y * a.nq + q] = sum;
             __threadfence();
             __syncthreads();
             if (tid == 0) s_last = atomicAdd(a.done + blockIdx.x, 1u) == (unsigned)splits - 1u;
             __syncthreads();
             if (s_last) {
                 __threadfence();
-                // each half of the epilogue warps adds half of the splits
+                // the epilogue's two sets of threads add half of the splits each
+                const int set = row >= RT * kTile, rw = set ? row - RT * kTile : row;
+                const int64_t qq = q0 + rw;
                 double v = 0.0;
-                if (warp >= 2 && q < a.nq) {
-                    const int k1 = half ? splits : splits / 2;
-                    for (int k = half ? splits / 2 : 0; k < k1; ++k) v += __ldcg(a.part + (size_t)k * a.nq + q);
+                if (row >= 0 && qq < a.nq) {
+                    const int k1 = set ? splits : splits / 2;
+                    for (int k = set ? splits / 2 : 0; k < k1; ++k) v += __ldcg(a.part + (size_t)k * a.nq + qq);
                 }
-                if (warp >= 2 && half == 1) s_acc[my_row] = v;
+                if (row >= 0 && set) s_acc[0][rw] = v;
                 __syncthreads();
-                acc = v + s_acc[my_row];
+                if (owner) sum = v + s_acc[0][row];
             } else {
                 mine = false;
             }
         }
         if (mine) {
-            const int32_t row = a.qrow[q];
-            double v = acc + a.add_scalar;
-            if (a.yq) v -= (double)a.yq[row];
-            a.out[row] = v;
+            const int32_t out_row = a.qrow[q];
+            double v = sum + a.add_scalar;
+            if (a.yq) v -= (double)a.yq[out_row];
+            a.out[out_row] = v;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 1) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kTile)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * RT * kTile)
                      : "memory");
     }
 }
@@ -602,7 +659,7 @@ struct QSide {
     int *err;
     unsigned *done;
     double *part;
-    int splits;
+    int splits, rt;
 };
 // Two CTAs share an SM: with fewer query tiles than that the support tiles are
 // split (48,868 support vectors, 300 queries: 3 CTAs took 377 us), at least
@@ -616,7 +673,27 @@ QSide q_side(Pieces &p, int64_t nq, int64_t nsv, int d, bool keep_order)
         sms = 1;
     const int64_t n = pad_rows(nq), tiles = n / kTile, nt = pad_rows(nsv) / kTile;
     QSide s;
-    s.splits = keep_order ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>({2 * (int64_t)sms / tiles, nt / 4, 64}));
+    // two query tiles per CTA once they give every SM one (d <= 128: their
+    // shared memory)
+    s.rt = !keep_order && (tiles + 1) / 2 >= sms && pad_cols(d) <= 2 * kKB ? 2 : 1;
+    const int64_t ctas = (tiles + s.rt - 1) / s.rt, slots = (s.rt == 2 ? 1 : 2) * (int64_t)sms;
+    s.splits = 1;
+    if (!keep_order && ctas < slots) {
+        s.splits = (int)std::max<int64_t>(1, std::min<int64_t>({slots / ctas, nt / 4, 64}));
+    } else if (!keep_order) {
+        // more CTAs than fit at once: the split, of at least 16 support tiles
+        // a CTA, whose last wave is fullest (391 CTAs on 152 SMs, 2.6 waves:
+        // 2.77 ms; split by 5, 12.9 waves: 2.52)
+        double best = 1e9;
+        for (int k = 1; k <= 8 && nt / k >= 16; ++k) {
+            const double waves = (double)(ctas * k) / (double)slots;
+            const double cost = std::ceil(waves) / waves + 0.005 * k;
+            if (cost < best) {
+                best = cost;
+                s.splits = k;
+            }
+        }
+    }
     s.Z = p.take<__nv_bfloat16>((size_t)n * pad_cols(d));
     s.zc = p.take<float>(n);
     s.qrow = p.take<int32_t>(n);
@@ -694,14 +771,23 @@ cudaError_t launch_rbf_contract_tc(const RbfContract &c, const void *sv, void *w
     a.err = q.err;
     a.part = q.part;
     a.done = q.done;
-    // query tile + a ring of support tiles: 4 slots at d <= 64, else 2; at
-    // least 80 KiB so that at most 2 CTAs share an SM: their 2 x 256
-    // tensor-memory columns then fit the SM's 512 without waiting
-    a.stages = kblocks == 1 ? 4 : 2;
-    const size_t smem = std::max<size_t>((size_t)(1 + a.stages) * kblocks * kTileBytes + 1024, 80 * 1024);
-    e = cudaFuncSetAttribute(tc_rbf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    tc_rbf_kernel<<<dim3((unsigned)tiles, (unsigned)q.splits), kTcThreads, smem, st>>>(mz, mx, a);
+    if (q.rt == 2) {
+        // two query tiles + 4 slots at d <= 64, 2 at d <= 128; one CTA per SM
+        a.stages = kblocks == 1 ? 4 : 2;
+        const size_t smem = std::max<size_t>((size_t)(2 + a.stages) * kblocks * kTileBytes + 1024, 120 * 1024);
+        e = cudaFuncSetAttribute(tc_rbf_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        tc_rbf_kernel<2><<<dim3((unsigned)((tiles + 1) / 2), (unsigned)q.splits), tc_threads(2), smem, st>>>(mz, mx, a);
+    } else {
+        // query tile + a ring of support tiles: 4 slots at d <= 64, else 2; at
+        // least 80 KiB so that at most 2 CTAs share an SM: their 2 x 256
+        // tensor-memory columns then fit the SM's 512 without waiting
+        a.stages = kblocks == 1 ? 4 : 2;
+        const size_t smem = std::max<size_t>((size_t)(1 + a.stages) * kblocks * kTileBytes + 1024, 80 * 1024);
+        e = cudaFuncSetAttribute(tc_rbf_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        tc_rbf_kernel<1><<<dim3((unsigned)tiles, (unsigned)q.splits), tc_threads(1), smem, st>>>(mz, mx, a);
+    }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return cudaMemcpyAsync(err_host, q.err, sizeof(int), cudaMemcpyDeviceToHost, st);

@@ -54,3 +54,17 @@ def test_decision_against_the_oracle(m, n, kind):
     with pkg.Model(p.X, p.y, a, 0.25, p.gamma, precision=prec) as mod:
         if kind != "fp64":
             assert np.array_equal(mod.decision(p.Z), got)
+
+
+def test_two_query_tiles_per_cta():
+    # enough queries that a CTA of the tensor-core contraction takes two tiles
+    # (a last one half empty): the rows' values in small calls, whose sums of
+    # the same 128-vector partial sums are added in another order
+    n, m = 300, 38785
+    p = synth.covtype_like(n=n, n_test=m, seed=3)
+    a = _alpha(n, p.C)
+    got = pkg.svm_decision(p.X, p.y, a, 0.25, p.gamma, p.Z, precision=pkg.SVM_MIXED_BF16)
+    bound = (n / 128 + 4) * 2.0 ** -52 * a.sum()
+    for lo, hi in ((0, 700), (19000, 19300), (m - 500, m)):
+        part = pkg.svm_decision(p.X, p.y, a, 0.25, p.gamma, p.Z.take(np.arange(lo, hi)), precision=pkg.SVM_MIXED_BF16)
+        assert np.abs(part - got[lo:hi]).max() <= bound
