@@ -640,7 +640,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
     const bool kc_on = KC_MODE && A.kc != nullptr;
     const SmoLayout L = smo_layout(MODE, d, A.ktab_len, A.maxnnz, RES ? 1 : 0, A.seg_rows_max,
                                    A.seg_nnz_max,
-                                   kc_on ? smo_kdir_bytes(A.n, A.kc_slots, A.kc_direct) : 0);
+                                   kc_on ? smo_kdir_bytes(A.n, A.kc_slots, A.kc_direct) : 0, A.dm_stride);
     uint32_t *kdir = reinterpret_cast<uint32_t *>(dsm + L.kdir);
     Tgt *tbuf = reinterpret_cast<Tgt *>(dsm + L.tgt);            // [2][d]
     int *tcol = reinterpret_cast<int *>(dsm + L.tcol);           // [2 buf][2 side][maxnnz]
@@ -718,6 +718,12 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
             }
         }
         for (int k = tid; k < cnt; k += kThreads) act_s[k] = A.act[lo + k];
+        if constexpr (MODE == MODE_MIXED && LPR == 16) {
+            const int per = A.d_pad / 8;   // 16-byte pieces of a dense row
+            for (int q = tid; A.dm_stride > 0 && q < nseg * per; q += kThreads)
+                *reinterpret_cast<uint4 *>(dsm + L.dmat + (size_t)(q / per) * A.dm_stride + 16 * (q % per)) =
+                    __ldg(reinterpret_cast<const uint4 *>(A.dmat + (size_t)lo * A.d_pad) + q);
+        }
     }
     if (kc_on) {
         // empty directory: no valid rows (direct), no tags and zero stamps (4-way sets)
@@ -1332,51 +1338,82 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                     // is column 32b + 8t + 4h + i and k = 2t + 8 + i column
                     // 32b + 8t + 4h + 2 + i; the targets use the same map, so
                     // the dot products are those of the rows. Each warp takes
-                    // 32 active rows (two tiles) at a time and hands each
+                    // one or two tiles of active rows at a time and hands each
                     // row's two sums to one lane, which finishes the row as
                     // the CUDA-core pass does.
                     tiles_done = true;
                     const int g = lane >> 2, t4 = lane & 3;
                     const int nblk = A.d_pad >> 5;
                     uint2 *frag = reinterpret_cast<uint2 *>(dsm + L.frag);   // [2 nblk k-steps][32 lanes]
-                    if (warp == 1) {
-                        for (int ks = 0; ks < 2 * nblk; ++ks) {
-                            const int b = ks >> 1, h = ks & 1;
-                            uint32_t w0 = 0, w1 = 0;
-                            if (!first && g < 2) {
-                                const int c = 32 * b + 8 * t4 + 4 * h;
-                                float e[4];
+                    // packed by the row warps together, before their barrier
+                    for (int ks = warp - 1; ks < 2 * nblk; ks += kRowWarps) {
+                        const int b = ks >> 1, h = ks & 1;
+                        uint32_t w0 = 0, w1 = 0;
+                        if (!first && g < 2) {
+                            const int c = 32 * b + 8 * t4 + 4 * h;
+                            float e[4];
 #pragma unroll
-                                for (int x = 0; x < 4; ++x) {
-                                    const int cx = c + x;
-                                    e[x] = cx < d ? (g == 0 ? T[cx].x : T[cx].y) : 0.f;
-                                }
-                                const __nv_bfloat162 p0 = __floats2bfloat162_rn(e[0], e[1]);
-                                const __nv_bfloat162 p1 = __floats2bfloat162_rn(e[2], e[3]);
-                                w0 = *reinterpret_cast<const uint32_t *>(&p0);
-                                w1 = *reinterpret_cast<const uint32_t *>(&p1);
+                            for (int x = 0; x < 4; ++x) {
+                                const int cx = c + x;
+                                e[x] = cx < d ? (g == 0 ? T[cx].x : T[cx].y) : 0.f;
                             }
-                            frag[ks * 32 + lane] = make_uint2(w0, w1);
+                            const __nv_bfloat162 p0 = __floats2bfloat162_rn(e[0], e[1]);
+                            const __nv_bfloat162 p1 = __floats2bfloat162_rn(e[2], e[3]);
+                            w0 = *reinterpret_cast<const uint32_t *>(&p0);
+                            w1 = *reinterpret_cast<const uint32_t *>(&p1);
                         }
+                        frag[ks * 32 + lane] = make_uint2(w0, w1);
                     }
                     rows_bar_sync();
-                    for (int base = rw * 32;; base += kRowWarps * 32) {   // warp-uniform
-                        const bool round0 = base == rw * 32;
+                    // Few rows: one tile per warp, so that twice the warps share
+                    // them. Rows on chip when they fit beside the segment
+                    // (their CTAs' strides keep two rows of a read apart in the
+                    // banks), else four blocks' loads from L2 at a time: one
+                    // block after the other, 100 rows x 100 columns a CTA took
+                    // 4,800 cycles from the pair step to the candidates.
+                    const int ntile = cnt <= kRowWarps * 16 ? 1 : 2;
+                    const bool chip = RES && A.dm_stride > 0;
+                    for (int base = rw * 16 * ntile;; base += kRowWarps * 16 * ntile) {   // warp-uniform
+                        const bool round0 = base == rw * 16 * ntile;
                         if (!round0 && base >= cnt) break;
                         float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
                         if (!first) {
 #pragma unroll
                             for (int q = 0; q < 2; ++q) {
+                                if (q >= ntile) break;
                                 const int ka = base + 16 * q + g, kb2 = ka + 8;
-                                const __nv_bfloat16 *pa = nullptr, *pb = nullptr;
-                                if (ka < cnt) pa = A.dmat + (size_t)(lo + (ident ? ka : ACT(ka))) * A.d_pad + 8 * t4;
-                                if (kb2 < cnt) pb = A.dmat + (size_t)(lo + (ident ? kb2 : ACT(kb2))) * A.d_pad + 8 * t4;
-                                for (int b = 0; b < nblk; ++b) {
-                                    const uint4 u = pa ? __ldg(reinterpret_cast<const uint4 *>(pa + 32 * b)) : make_uint4(0, 0, 0, 0);
-                                    const uint4 v = pb ? __ldg(reinterpret_cast<const uint4 *>(pb + 32 * b)) : make_uint4(0, 0, 0, 0);
-                                    const uint2 f0 = frag[(2 * b) * 32 + lane], f1 = frag[(2 * b + 1) * 32 + lane];
-                                    mma_bf16_16816(acc[q], u.x, v.x, u.y, v.y, f0.x, f0.y);
-                                    mma_bf16_16816(acc[q], u.z, v.z, u.w, v.w, f1.x, f1.y);
+                                const int ra = ka < cnt ? (ident ? ka : ACT(ka)) : -1, rb = kb2 < cnt ? (ident ? kb2 : ACT(kb2)) : -1;
+                                if (chip) {
+                                    const unsigned char *pa = dsm + L.dmat + (size_t)(ra < 0 ? 0 : ra) * A.dm_stride + 16 * t4;
+                                    const unsigned char *pb = dsm + L.dmat + (size_t)(rb < 0 ? 0 : rb) * A.dm_stride + 16 * t4;
+#pragma unroll 4
+                                    for (int b = 0; b < nblk; ++b) {
+                                        uint4 u = *reinterpret_cast<const uint4 *>(pa + 64 * b);
+                                        uint4 v = *reinterpret_cast<const uint4 *>(pb + 64 * b);
+                                        const uint2 f0 = frag[(2 * b) * 32 + lane], f1 = frag[(2 * b + 1) * 32 + lane];
+                                        mma_bf16_16816(acc[q], u.x, v.x, u.y, v.y, f0.x, f0.y);
+                                        mma_bf16_16816(acc[q], u.z, v.z, u.w, v.w, f1.x, f1.y);
+                                    }
+                                } else {
+                                    const __nv_bfloat16 *pa = ra >= 0 ? A.dmat + (size_t)(lo + ra) * A.d_pad + 8 * t4 : nullptr;
+                                    const __nv_bfloat16 *pb = rb >= 0 ? A.dmat + (size_t)(lo + rb) * A.d_pad + 8 * t4 : nullptr;
+                                    for (int b0 = 0; b0 < nblk; b0 += 4) {
+                                        uint4 u[4], v[4];
+#pragma unroll
+                                        for (int j = 0; j < 4; ++j) {
+                                            const bool in = b0 + j < nblk;
+                                            u[j] = pa && in ? __ldg(reinterpret_cast<const uint4 *>(pa + 32 * (b0 + j))) : make_uint4(0, 0, 0, 0);
+                                            v[j] = pb && in ? __ldg(reinterpret_cast<const uint4 *>(pb + 32 * (b0 + j))) : make_uint4(0, 0, 0, 0);
+                                        }
+#pragma unroll
+                                        for (int j = 0; j < 4; ++j) {
+                                            if (b0 + j >= nblk) break;
+                                            const int b = b0 + j;
+                                            const uint2 f0 = frag[(2 * b) * 32 + lane], f1 = frag[(2 * b + 1) * 32 + lane];
+                                            mma_bf16_16816(acc[q], u[j].x, v[j].x, u[j].y, v[j].y, f0.x, f0.y);
+                                            mma_bf16_16816(acc[q], u[j].z, v[j].z, u[j].w, v[j].w, f1.x, f1.y);
+                                        }
+                                    }
                                 }
                             }
                         }
@@ -1396,7 +1433,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                             }
                         }
                         const int k = base + lane;
-                        const bool valid = k < cnt;
+                        const bool valid = k < cnt && lane < 16 * ntile;
                         int r = 0;
                         double fi = 0.0;
                         uint8_t sb = 0;

@@ -439,6 +439,7 @@ __global__ void k_iota(int64_t n, int32_t *out);
 constexpr int kChunkRows = 4096;
 // largest FP64-mode problem (rows, non-binary input) solved by one 16-CTA cluster
 constexpr int64_t kFp64OneClusterRows = 8192;
+constexpr int64_t kFp64OneClusterLate = 12288;   // ... of a re-layout level with the kernel-row cache
 // smallest FP64-mode problem that takes one CTA per SM with the flat exchange
 // even when its segments fit in shared memory
 constexpr int64_t kFp64FlatRows = 200000;
@@ -1146,6 +1147,7 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
         int G, cs, resident, seg_rows_max;
         int64_t seg_nnz_max;
         size_t smem;
+        int dm_stride;   // row tiles: the dense rows on chip too, this many bytes apart (0: not)
     };
     int64_t *segnnz_d = ar.alloc<int64_t>(256);
     auto pick_shape = [&](int64_t n_l, int64_t nnz_l, const int64_t *indptr_l, size_t kdir_l) -> Shape {
@@ -1165,7 +1167,13 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
             // issue per clock per SM here), so above a few thousand rows 16 SMs
             // are slower than clusters of 8 over the whole GPU despite their
             // cheaper exchange (measured crossover ~7,000 covtype-shaped rows)
-            const int64_t one_cluster_max = kmode == MODE_FP64 ? kFp64OneClusterRows : 200000;
+            // The small levels of a re-layout find nine rows of ten in the
+            // kernel-row cache and are then bound by the exchange (short rows,
+            // 9,000 / 12,000 of them: 4.6 / 4.9 us a step on one cluster, 5.5 /
+            // 5.7 on clusters of 8; 16,000: 6.4 against 5.8; without cached
+            // rows 9.1 / 10.2 against 6.1 / 6.4)
+            const bool late = kdir_l > 0 && n_l < n && (double)nnz_l <= 16.0 * (double)n_l;
+            const int64_t one_cluster_max = kmode == MODE_FP64 ? (late ? kFp64OneClusterLate : kFp64OneClusterRows) : 200000;
             if (L16.total <= lim_dyn && smo_max_clusters(kmode, lpr, 2, L16.total, 16) >= 1 &&
                 (P->ctas == 16 || n_l <= one_cluster_max)) {
                 single = true;
@@ -1245,6 +1253,17 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
         sh.seg_rows_max = seg_rows_max_l;
         sh.seg_nnz_max = seg_nnz_max_l;
         sh.smem = resident_l ? Lr.total : Ls.total;
+        sh.dm_stride = 0;
+        if (row_tiles && resident_l) {
+            // two rows of one read 64 bytes apart in the banks
+            const int stride = 2 * d_pad + (2 * d_pad % 128 == 0 ? 64 : 0);
+            const SmoLayout Ld = smo_layout(kmode, (int)D.d, kt, D.maxnnz, 1, seg_rows_max_l, seg_nnz_max_l, kdir_l, stride);
+            if (Ld.total <= lim_dyn &&
+                smo_max_clusters(kmode, lpr, G_l == cs_l ? 2 : 1, Ld.total, cs_l) * cs_l >= G_l) {
+                sh.smem = Ld.total;
+                sh.dm_stride = stride;
+            }
+        }
         if (sh.smem > lim_dyn) {
             set_err("d = %lld exceeds the shared-memory target rows of this mode", (long long)D.d);
             throw Fail{SVM_ERR_UNSUPPORTED};
@@ -1512,6 +1531,7 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
         A.gmap = L.gmap;
         A.dmat = L.dmat;
         A.d_pad = d_pad;
+        A.dm_stride = L.shape.dm_stride;
         A.kc = L.kc.slots > 0 ? kc_buf : nullptr;
         A.kc_ld = L.kc.ld;
         A.kc_slots = L.kc.slots;

@@ -149,6 +149,7 @@ struct SmoArgs {
     // row pass on the CUDA cores
     const __nv_bfloat16 *dmat;
     int32_t d_pad;
+    int32_t dm_stride;         // > 0: the segments' rows on chip too, this many bytes apart
     // optional: (step, active rows) after each shrink event, 2 per event
     int64_t *atrace;
     int64_t atrace_len;
@@ -228,13 +229,14 @@ cudaError_t launch_smo_batch(int mode, int lpr, int dense, const BatchArgs &a, s
 
 // Dynamic shared-memory layout of the step kernel (byte offsets).
 struct SmoLayout {
-    size_t tgt, tcol, ktab, f, alpha, nrm, rowptr, act, st, col, val, bits, dist, kdir, frag, total;
+    size_t tgt, tcol, ktab, f, alpha, nrm, rowptr, act, st, col, val, bits, dist, kdir, frag, dmat, total;
 };
 
 __host__ __device__ inline size_t smo_align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 __host__ __device__ inline SmoLayout smo_layout(int mode, int d, int ktab_len, int maxnnz,
-                                                int resident, int rows, int64_t nnz, size_t kdir_bytes = 0)
+                                                int resident, int rows, int64_t nnz, size_t kdir_bytes = 0,
+                                                int dm_stride = 0)
 {
     SmoLayout L;
     const bool bits = mode_bits(mode);
@@ -260,6 +262,8 @@ __host__ __device__ inline SmoLayout smo_layout(int mode, int d, int ktab_len, i
     L.kdir = o;   o = smo_align16(o + kdir_bytes);                     // kernel-row cache directory
     // mixed mode: B fragments of the tensor-core row tiles (16 k-steps x 32 lanes x 8 B)
     L.frag = o;   o = smo_align16(o + (mode == 2 ? (size_t)16 * 32 * 8 : 0));
+    // ... and the segment's dense BF16 rows for them, dm_stride bytes each
+    L.dmat = o;   o = smo_align16(o + (size_t)rows * dm_stride);
     L.total = o;
     return L;
 }

@@ -36,3 +36,17 @@ def test_ragged_rows_with_empty_ones(n):
     a = pkg.svm_train(p.X, p.y, p.C, p.gamma, p.tau, trace_len=300)
     b = pkg.svm_train(p.X, p.y, p.C, p.gamma, p.tau, trace_len=300, flags=pkg.SVM_FLAG_STREAM_ROWS)
     assert np.array_equal(a["trace"], b["trace"]) and np.array_equal(a["alpha"], b["alpha"])
+
+
+@pytest.mark.parametrize("d", [32, 64, 100, 200])
+@pytest.mark.parametrize("n", [530, 3840, 4100])
+def test_row_tiles_on_chip_equal_streamed_ones(n, d):
+    # one and two tiles per warp, rows on chip, on chip without their dense
+    # copy (d = 200, the larger sizes) and from L2
+    p = synth.small_dense(n, d, seed=n + d, sep=0.15, C=2.0, gamma=1.0 / d)
+    kw = dict(precision=pkg.SVM_MIXED_BF16, shrink=pkg.POLICIES["Multi500"], trace_len=300, max_iter=3000)
+    a = pkg.svm_train(p.X, p.y, p.C, p.gamma, p.tau, flags=pkg.SVM_FLAG_TENSOR_ROWS, **kw)
+    b = pkg.svm_train(p.X, p.y, p.C, p.gamma, p.tau, flags=pkg.SVM_FLAG_TENSOR_ROWS | pkg.SVM_FLAG_STREAM_ROWS, **kw)
+    assert a["stats"]["row_tiles"] == b["stats"]["row_tiles"] == 1 and b["stats"]["resident"] == 0
+    assert a["iters"] == b["iters"] and np.array_equal(a["trace"], b["trace"])
+    assert np.array_equal(a["alpha"], b["alpha"]) and a["b"] == b["b"]
