@@ -236,8 +236,11 @@ Plan plan_of(const RbfContract &c)
 
 }  // namespace
 
+// K in Q63 is as exact as a double down to 2^-11: only kernels whose smallest
+// table value (the largest distance) is at least that.
 bool rbf_bits_supported(const RbfContract &c)
 {
+    if (!(c.gamma * (double)(c.ktab_len - 1) <= 7.5)) return false;
     return c.mode == MODE_BINARY && c.d <= 256 && !c.keep_order && !c.out_by_row && !c.yq && !c.accumulate && !c.q;
 }
 

@@ -68,3 +68,21 @@ def test_two_query_tiles_per_cta():
     for lo, hi in ((0, 700), (19000, 19300), (m - 500, m)):
         part = pkg.svm_decision(p.X, p.y, a, 0.25, p.gamma, p.Z.take(np.arange(lo, hi)), precision=pkg.SVM_MIXED_BF16)
         assert np.abs(part - got[lo:hi]).max() <= bound
+
+
+@pytest.mark.parametrize("gamma", [0.03, 1.0])
+def test_binary_decision_keeps_small_kernel_values(gamma):
+    # one class and b = 0, so nothing cancels and the bound is relative to the
+    # decision itself: K and its exponent's rounding, a term each, and the sum
+    # of n terms. At gamma = 1 the largest K of a query is near e^-20.
+    n, m = 400, 40
+    p = synth.random_sparse(n=n + m, d=200, density=0.08, seed=11, binary=True)
+    Z, X = p.X.take(np.arange(n, n + m)), p.X.take(np.arange(n))
+    y, a = np.ones(n, p.y.dtype), np.full(n, 1.0)
+    got = pkg.svm_decision(X, y, a, 0.0, gamma, Z, precision=pkg.SVM_FP64)
+    D = lambda M: np.array([np.bincount(M.indices[M.indptr[i]:M.indptr[i + 1]], minlength=200) for i in range(M.n)])  # noqa: E731
+    dx, dz = D(X), D(Z)
+    dist = dz.sum(1)[:, None] + dx.sum(1)[None, :] - 2 * (dz @ dx.T)
+    ref = np.exp(-gamma * dist.astype(np.float64)).sum(1)
+    rel = (n + 4 + gamma * dist.max()) * 2.0 ** -52
+    assert np.all(np.abs(got - ref) <= rel * ref), (np.abs(got - ref) / ref).max()
