@@ -61,7 +61,9 @@ struct BatchShared {
     Side wup[kWarps], wlow[kWarps];
     unsigned long long wkup[kWarps], wklow[kWarps];
     int wiup[kWarps], wilow[kWarps];
-    CandFull ccand[kMaxCluster];   // cluster leader: its CTAs' candidates
+    CandFull xc[2][kMaxCluster];   // every CTA's candidate, by epoch parity
+    unsigned long long xbar[2];    // mbarriers of the two parities
+    Side none[2];                  // empty I_up / I_low sides
     ResultArea res;
     BatchFinish fin[kMaxCluster];  // cluster leader: its CTAs' partial sums
     BatchFinish wfin[kWarps];
@@ -69,7 +71,8 @@ struct BatchShared {
     unsigned char st_u, st_l;
     PairPre pre;
     unsigned long long stage_bar[kWarps];   // packed units: a row warp's unit has landed
-    int stage_bad;                          // a wait for one gave up
+    int bad;                                // a wait gave up: status 2 from here on
+    int stop;                               // the gap is closed, the step is not taken
     int job;
 };
 
@@ -105,16 +108,23 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
     unsigned char *stage0 = reinterpret_cast<unsigned char *>(
         ((uintptr_t)(kdir + B.kdir_words) + 127) & ~(uintptr_t)127);
     uint32_t stage_parity = 0;
-    if constexpr (PACK_MODE) {
-        if (tid == 0) {
-            for (int w = 0; w < kWarps; ++w) mbar_init(smem_u32(&sh.stage_bar[w]), 1);
-            sh.stage_bad = 0;
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            fence_async_proxy();
-        }
+    if (tid == 0) {
+        for (int w = 0; w < kWarps; ++w) mbar_init(smem_u32(&sh.stage_bar[w]), 1);
+        mbar_init(smem_u32(&sh.xbar[0]), 1);
+        mbar_init(smem_u32(&sh.xbar[1]), 1);
+        side_empty(sh.none[0], true);
+        side_empty(sh.none[1], false);
+        sh.bad = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_async_proxy();
     }
+    cluster.sync();   // the barriers exist before any CTA of the cluster sends
+    unsigned epoch = 0;
 
     for (;;) {
+        // a wait of this cluster gave up: its further jobs only report that
+        // (read before the barrier below, so every thread and CTA sees the same)
+        const bool dead = sh.bad != 0;
         // ---- next job from the work-list, broadcast to the cluster
         if (crank == 0 && tid == 0) {
             int j = INT_MAX;
@@ -246,12 +256,12 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
         };
         auto wait_unit = [&]() {
             if (!in_flight) return;
-            const int bad = mbar_wait_bounded(stage_bar, stage_parity, 10ll * 1000 * 1000 * 1000, &sh.stage_bad);
-            if (__any_sync(0xffffffffu, bad) && lane == 0) sh.stage_bad = 1;
+            const int bad = mbar_wait_bounded(stage_bar, stage_parity, 10ll * 1000 * 1000 * 1000, &sh.bad);
+            if (__any_sync(0xffffffffu, bad) && lane == 0) sh.bad = 1;
             stage_parity ^= 1u;
             in_flight = false;
         };
-        if (warp >= 1 && warp <= stage_warps && warp - 1 < units) issue_unit(warp - 1);
+        if (!dead && warp >= 1 && warp <= stage_warps && warp - 1 < units) issue_unit(warp - 1);
 
         Side up, low;
         side_empty(up, true);
@@ -259,9 +269,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
         bool first = true;
         int64_t iter = 0;
         int prev_valid = 0, prev_len_u = 0, prev_len_l = 0;
-        int64_t prev_pu = 0, prev_pl = 0;
-        int status_code = 0;
-        for (;;) {
+        int status_code = dead ? 2 : 0;
+        while (!dead) {
             const int buf = (int)(iter & 1);
             Tgt *T = tbuf + (size_t)buf * dmax;
             int *tcu = tcol + (size_t)(buf * 2 + 0) * maxnnz;
@@ -269,16 +278,15 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             bool hu = false, hl = false;   // x_up's / x_low's kernel row is in the cache
             uint32_t kd_wu = 0, kd_wl = 0;
             if (!first) {
-                if (!dless(thr, low.f - up.f)) { status_code = 0; break; }
-                if (iter >= J.max_iter) { status_code = 1; break; }
+                // (the gap is tested beside the pair step, below)
+                if (up.i == INT_MAX || low.i == INT_MAX) { status_code = 0; break; }
+                if (iter >= J.max_iter) { status_code = dless(thr, low.f - up.f) ? 1 : 0; break; }
                 if (kc_on) {
                     kd_wu = kdir[up.i >> 5];
                     kd_wl = kdir[low.i >> 5];
                     hu = (kd_wu >> (up.i & 31)) & 1u;
                     hl = (kd_wl >> (low.i & 31)) & 1u;
                 }
-                // the pair step's part that K(up, low) does not enter
-                if (warp >= kPre0) pair_pre<MODE == MODE_FP64>(&sh.pre, warp - kPre0, lane, up, low, C);
                 // ---- 1. targets into the shared-memory buffer
                 if (dense) {
                     if constexpr (MODE == MODE_MIXED) {
@@ -311,10 +319,22 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                         }
                     }
                 }
-                __syncthreads();
+                // the warps of the pair step's bounds only arrive; with both
+                // kernel rows cached no row warp needs the targets
+                const bool both = hu && hl;
+                if (warp >= kPre0 || (both && warp != 0)) fill_bar_arrive();
+                else fill_bar_sync();
+                if (warp == 0 && !both) filled_arrive();
+                if (warp >= kPre0) {
+                    // the pair step's part that K(up, low) does not enter
+                    pair_pre<MODE == MODE_FP64>(&sh.pre, warp - kPre0, lane, up, low, C);
+                    pre_bar_arrive();
+                    if (!both) filled_sync();
+                }
             }
             unsigned long long bku = kNoKey, bkl = kNoKey;
             int biu = INT_MAX, bil = INT_MAX, bru = 0, brl = 0;
+            bool stop = false;   // the gap is closed: nothing of this step is taken
             if (warp == 0) {
                 // ---- 2. pair step (Eq. alphaup with rho = -eta, Platt clip)
                 if (!first) {
@@ -345,7 +365,9 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
 #pragma unroll
                         for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
                     }
+                    pre_bar_sync();
                     const PairPre pre = sh.pre;
+                    stop = !bits_less(thr, neg_if(pre.slope.x, low.y > 0));   // Eq. (kktterm)
                     bool curved;
                     double q;
                     if constexpr (MODE == MODE_BINARY) {
@@ -370,6 +392,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                     }
                     const PairStep ps = pair_solve(pre, up, low, curved, q, C, snap, c_snap);
                     if (lane == 0) {
+                        sh.stop = stop;
                         sh.du = ps.du;
                         sh.dl = ps.dl;
                         sh.au_new = ps.au;
@@ -392,6 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                         du = sh.du; dl = sh.dl;
                         st_u = sh.st_u; st_l = sh.st_l;
                         au_new = sh.au_new; al_new = sh.al_new;
+                        stop = sh.stop != 0;
                         have_step = true;
                     }
                 };
@@ -399,6 +423,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 double *kcl = kc_on && !first ? kc + (size_t)low.i * kc_ld : nullptr;
                 // FP64 update of Eq. (fup) and selection keys of one row
                 auto update_row = [&](int r, double ku, double kl, double fi, uint8_t sb) {
+                    if (stop) return;
                     if (!first) {
                         fi = fma(dl, kl, fma(du, ku, fi));
                         fj[r] = fi;
@@ -721,14 +746,33 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                                 }
                             } else if (xd) {
                                 if constexpr (MODE == MODE_FP64) {
+                                    // four entries' loads at a time; a side
+                                    // whose row is cached is left out
                                     const int4 *T4 = reinterpret_cast<const int4 *>(T);
-                                    for (int64_t p = p0 + gl; p < p1; p += LPR) {
-                                        const uint32_t u = __float_as_uint(values[p]);
-                                        const int32_t mx = xd_mant(u);
-                                        const int e = xd_exp(u, xd_tmin) + xd_bias;
-                                        const int4 t = T4[indices[p]];
-                                        xd_add(au, mx, t.x, e + t.y);
-                                        xd_add(al, mx, t.z, e + t.w);
+                                    const int2 *T2 = reinterpret_cast<const int2 *>(T) + (hu ? 1 : 0);
+                                    for (int64_t pb = p0 + gl; pb < p1; pb += 4 * LPR) {
+                                        int cb[4];
+                                        uint32_t ub[4];
+#pragma unroll
+                                        for (int j = 0; j < 4; ++j) {
+                                            const int64_t p = pb + (int64_t)j * LPR;
+                                            cb[j] = p < p1 ? indices[p] : 0;
+                                            ub[j] = p < p1 ? __float_as_uint(values[p]) : 0u;
+                                        }
+#pragma unroll
+                                        for (int j = 0; j < 4; ++j) {
+                                            if (pb + (int64_t)j * LPR >= p1) break;
+                                            const int32_t mx = xd_mant(ub[j]);
+                                            const int e = xd_exp(ub[j], xd_tmin) + xd_bias;
+                                            if (!hu && !hl) {
+                                                const int4 t = T4[cb[j]];
+                                                xd_add(au, mx, t.x, e + t.y);
+                                                xd_add(al, mx, t.z, e + t.w);
+                                            } else {
+                                                const int2 t = T2[2 * cb[j]];
+                                                xd_add(au, mx, t.x, e + t.y);
+                                            }
+                                        }
                                     }
                                 }
                             } else {
@@ -755,9 +799,11 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                         if (!first && xd) {
                             if constexpr (MODE == MODE_FP64) {
                                 xd_lane_sum<LPR>(au);
-                                xd_lane_sum<LPR>(al);
-                                su = xd_round(au, xd_unit);
-                                sl = xd_round(al, xd_unit);
+                                su = sl = xd_round(au, xd_unit);
+                                if (!hu && !hl) {
+                                    xd_lane_sum<LPR>(al);
+                                    sl = xd_round(al, xd_unit);
+                                }
                             }
                         } else if (!first) {
 #pragma unroll
@@ -774,6 +820,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 }
                 }
             }
+            if (stop) { status_code = 0; break; }   // (every CTA sees the same pair)
             // payload of a job row (job-local index r)
             auto make_side = [&](int r) {
                 Side sd;
@@ -810,76 +857,85 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             }
             __syncthreads();
             // both rows are stored from here on (all threads have read this
-            // step's bits; the cluster barriers order the next step's reads)
+            // step's bits; the barrier after the exchange orders the next step's reads)
             if (kc_on && !first && tid == 0) {
                 const uint32_t bu = 1u << (up.i & 31), bl = 1u << (low.i & 31);
                 const bool same = (up.i >> 5) == (low.i >> 5);
                 kdir[up.i >> 5] = kd_wu | bu | (same ? bl : 0u);
                 if (!same) kdir[low.i >> 5] = kd_wl | bl;
             }
-            // ---- 4. candidate exchange inside the cluster
+            // ---- 4. candidate exchange inside the cluster: every CTA's
+            //         candidate into every CTA's shared memory, as asynchronous
+            //         stores counted on its mbarrier (lanes q and 16 + q send
+            //         the first 48 bytes of the I_up and I_low sides to CTA q);
+            //         every CTA reduces them in the same order. With the
+            //         gap test beside the pair step, no target fill once both
+            //         rows are cached and four entries' loads in flight, 7 FP64
+            //         problems of 300 to 3000 rows took 28.7 instead of 35.0 ms
+            //         (two cluster barriers a step before, 530 cycles each).
+            ++epoch;
+            const int par = (int)(epoch & 1);
             if (warp == 0) {
                 unsigned long long k1 = lane < kWarps ? sh.wkup[lane] : kNoKey;
                 unsigned long long k2 = lane < kWarps ? sh.wklow[lane] : kNoKey;
                 int i1 = lane < kWarps ? sh.wiup[lane] : INT_MAX;
                 int i2 = lane < kWarps ? sh.wilow[lane] : INT_MAX;
-                const unsigned long long k1s = k1, k2s = k2;
                 const int i1s = i1, i2s = i2;
                 warp_min_ki(k1, i1);
                 warp_min_ki(k2, i2);
-                const unsigned mu = __ballot_sync(0xffffffffu, i1 != INT_MAX && k1s == k1 && i1s == i1);
-                const unsigned ml = __ballot_sync(0xffffffffu, i2 != INT_MAX && k2s == k2 && i2s == i2);
-                if (lane == 0) {
-                    CandFull cf;
-                    if (mu) cf.up = sh.wup[__ffs(mu) - 1]; else side_empty(cf.up, true);
-                    if (ml) cf.low = sh.wlow[__ffs(ml) - 1]; else side_empty(cf.low, false);
-                    cf.count = hi - lo;
-                    cf.pad[0] = cf.pad[1] = cf.pad[2] = 0;
-                    *(cluster.map_shared_rank(sh.ccand, 0) + crank) = cf;
+                const int w1 = __ffs(__ballot_sync(0xffffffffu, i1s == i1)) - 1;
+                const int w2 = __ffs(__ballot_sync(0xffffffffu, i2s == i2)) - 1;
+                const bool side_low = lane >= 16;
+                const int q = lane & 15;
+                const Side *sd = side_low ? (i2 != INT_MAX ? &sh.wlow[w2] : &sh.none[1])
+                                          : (i1 != INT_MAX ? &sh.wup[w1] : &sh.none[0]);
+                if (q < csize) {
+                    const uint4 *sv = reinterpret_cast<const uint4 *>(sd);
+                    const uint32_t dst = cluster_addr(smem_u32(side_low ? &sh.xc[par][crank].low : &sh.xc[par][crank].up), q);
+                    const uint32_t rbar = cluster_addr(smem_u32(&sh.xbar[par]), q);
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) st_async_v4(dst + 16 * j, sv[j], rbar);
                 }
+                if (lane == 0) mbar_arrive_expect_tx(smem_u32(&sh.xbar[par]), (uint32_t)(csize * 2 * 48));
             }
-            if (prev_valid && warp >= 8) {
+            if (prev_valid && !dense && warp >= 8) {
                 Tgt *P = tbuf + (size_t)(1 - buf) * dmax;
-                if (dense) {
-                    (void)prev_pu;
-                    (void)prev_pl;
-                } else {
-                    const int *pcu = tcol + (size_t)((1 - buf) * 2 + 0) * maxnnz;
-                    const int *pcl = tcol + (size_t)((1 - buf) * 2 + 1) * maxnnz;
-                    for (int k = tid - 256; k < prev_len_u; k += kThreads - 256) P[pcu[k]] = tclear;
-                    for (int k = tid - 256; k < prev_len_l; k += kThreads - 256) P[pcl[k]] = tclear;
-                }
+                const int *pcu = tcol + (size_t)((1 - buf) * 2 + 0) * maxnnz;
+                const int *pcl = tcol + (size_t)((1 - buf) * 2 + 1) * maxnnz;
+                for (int k = tid - 256; k < prev_len_u; k += kThreads - 256) P[pcu[k]] = tclear;
+                for (int k = tid - 256; k < prev_len_l; k += kThreads - 256) P[pcl[k]] = tclear;
             }
-            cluster.sync();
-            if (crank == 0 && warp == 0) {
-                CandFull c;
-                if (lane < csize) c = sh.ccand[lane];
-                else { side_empty(c.up, true); side_empty(c.low, false); c.count = 0; }
-                unsigned long long k1 = c.up.i == INT_MAX ? kNoKey : key_up(c.up.f);
-                unsigned long long k2 = c.low.i == INT_MAX ? kNoKey : key_low(c.low.f);
-                int i1 = c.up.i, i2 = c.low.i;
-                const unsigned long long k1s = k1, k2s = k2;
+            if (warp == 0) {
+                const uint32_t parity = (uint32_t)((epoch - 1) >> 1) & 1u;
+                int bad = mbar_wait_bounded(smem_u32(&sh.xbar[par]), parity, 10ll * 1000 * 1000 * 1000, &sh.bad);
+                bad = __any_sync(0xffffffffu, bad);
+                unsigned long long k1 = kNoKey, k2 = kNoKey;
+                int i1 = INT_MAX, i2 = INT_MAX;
+                long long cc = 0;
+                if (lane < csize && !bad) cand_keys(sh.xc[par][lane], k1, i1, k2, i2, cc);
                 const int i1s = i1, i2s = i2;
                 warp_min_ki(k1, i1);
                 warp_min_ki(k2, i2);
-                const unsigned mu = __ballot_sync(0xffffffffu, i1 != INT_MAX && k1s == k1 && i1s == i1);
-                const unsigned ml = __ballot_sync(0xffffffffu, i2 != INT_MAX && k2s == k2 && i2s == i2);
-                if (lane < csize) {
-                    ResultArea res;
-                    if (mu) res.up = sh.ccand[__ffs(mu) - 1].up; else side_empty(res.up, true);
-                    if (ml) res.low = sh.ccand[__ffs(ml) - 1].low; else side_empty(res.low, false);
-                    res.total = m;
-                    res.flag = 0;
-                    res.gap_open = 1;   // the batch kernel tests the gap itself
-                    *cluster.map_shared_rank(&sh.res, lane) = res;
+                // (without any candidate lane 0 wins, whose side is the empty one)
+                const int w1 = __ffs(__ballot_sync(0xffffffffu, i1s == i1)) - 1;
+                const int w2 = __ffs(__ballot_sync(0xffffffffu, i2s == i2)) - 1;
+                if (lane < 12) {
+                    const bool u = lane < 6;
+                    const int w = u ? lane : lane - 6;
+                    reinterpret_cast<unsigned long long *>(u ? &sh.res.up : &sh.res.low)[w] =
+                        reinterpret_cast<const unsigned long long *>(u ? &sh.xc[par][w1].up : &sh.xc[par][w2].low)[w];
                 }
+                if (lane == 0) sh.res.flag = bad;
             }
-            cluster.sync();
+            __syncthreads();
+            if (sh.res.flag) {
+                if (tid == 0) sh.bad = 1;
+                status_code = 2;
+                break;
+            }
             prev_valid = first ? 0 : 1;
             prev_len_u = up.len;
             prev_len_l = low.len;
-            prev_pu = up.p0;
-            prev_pl = low.p0;
             up = sh.res.up;
             low = sh.res.low;
             if (!first) ++iter;
@@ -920,6 +976,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                     t.nsv += sh.wfin[w].nsv;
                 }
                 *(cluster.map_shared_rank(sh.fin, 0) + crank) = t;
+                if (sh.bad)
+                    for (int r = 0; r < csize; ++r) *cluster.map_shared_rank(&sh.bad, r) = 1;
             }
             cluster.sync();
             if (crank == 0 && tid == 0) {
@@ -937,7 +995,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 R.b = t.n0 > 0 ? t.sum_f0 / (double)t.n0 : 0.5 * (up.f + low.f);
                 R.objective = t.sum_a - 0.5 * t.sum_ayfy;
                 R.iters = iter;
-                R.status = PACK_MODE && sh.stage_bad ? 2 : status_code;
+                R.status = sh.bad ? 2 : status_code;
                 R.n_sv = (int32_t)t.nsv;
                 B.results[job] = R;
                 if (B.done) {
