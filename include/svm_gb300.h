@@ -25,7 +25,9 @@
  *   - All calls are synchronous with respect to the host unless stated: on
  *     return, outputs are written and the library's device work is done.
  *   - The library allocates its own device workspace (stream-ordered) and
- *     frees it before returning; inputs are only read, never kept.
+ *     frees it before returning, into a pool of its own that keeps up to 4 GiB
+ *     for later calls (given back when an allocation would fail otherwise);
+ *     inputs are only read, never kept.
  */
 #ifndef SVM_GB300_H
 #define SVM_GB300_H

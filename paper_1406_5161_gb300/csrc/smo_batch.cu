@@ -7,7 +7,7 @@
 // bminmax, kktterm, alphaup) exactly as the single-job fused step does:
 // target rows in shared memory, the FP64 pair step on warp 0 overlapped with
 // the row sums of warps 1.., FP64 f updates, integer selection keys. The
-// candidate exchange stays inside the cluster (distributed shared memory),
+// candidate exchange stays inside the cluster (asynchronous stores),
 // so clusters never wait on one another and need no co-residency. When a
 // job converges, the cluster reduces b (Section III-A) and the objective,
 // writes the job's result and takes the next job.
@@ -870,9 +870,11 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             //         the first 48 bytes of the I_up and I_low sides to CTA q);
             //         every CTA reduces them in the same order. With the
             //         gap test beside the pair step, no target fill once both
-            //         rows are cached and four entries' loads in flight, 7 FP64
-            //         problems of 300 to 3000 rows took 28.7 instead of 35.0 ms
-            //         (two cluster barriers a step before, 530 cycles each).
+            //         rows are cached and four entries' loads in flight, 45 FP64
+            //         problems of 1,500 rows (d = 20, clusters of 4 CTAs) took
+            //         28.7 instead of 35.0 ms (two cluster barriers a step
+            //         before, 530 cycles each); 90 mixed ones of about 4,000
+            //         rows (d = 256, 2 CTAs) 104.6 ms as before.
             ++epoch;
             const int par = (int)(epoch & 1);
             if (warp == 0) {
