@@ -546,7 +546,17 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                         // sums are handed to one lane, so that the exponentials
                         // and the FP64 updates run on whole warps
                         const int step_warps = packed ? stage_warps : kRowWarps;
-                        for (int u = warp - 1; u < units && warp <= step_warps; u += step_warps) {
+                        // Packed units are walked forwards and backwards in
+                        // turn: a step begins with the unit that its stage
+                        // still holds, and the units read last are in L2 (76
+                        // problems' rows, 152 MB, are more than L2 and came
+                        // from HBM in every step when always walked forwards:
+                        // 90 problems of 4,000 x 256, 104.6 -> 97.0 ms). The
+                        // selection does not depend on the order.
+                        const bool rev = packed && (iter & 1);
+                        const int nu = warp <= step_warps && warp <= units ? (units - warp) / step_warps + 1 : 0;
+                        for (int k = 0; k < nu; ++k) {
+                            const int u = warp - 1 + (rev ? nu - 1 - k : k) * step_warps;
                             const int base = lo + 32 * u;
                             const int r = base + lane;
                             const bool valid = r < hi;
@@ -574,13 +584,11 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                                     }
                                 }
                                 // the next unit while this one's rows are
-                                // finished (a warp's first unit again at the
-                                // end: it lands before the next step begins)
+                                // finished
                                 __syncwarp();
-                                const int next = u + step_warps < units ? u + step_warps : warp - 1;
-                                if (next != u) {
+                                if (k + 1 < nu) {
                                     fence_async_proxy();
-                                    issue_unit(next);
+                                    issue_unit(rev ? u - step_warps : u + step_warps);
                                 }
                             } else if (!first) {
 #pragma unroll
