@@ -57,11 +57,23 @@ struct __align__(16) BatchFinish {
 // 16 k-steps x 32 lanes of packed BF16 target pairs (uint2)
 constexpr size_t kFragBytes = (size_t)16 * 32 * sizeof(uint2);
 
+// What a step needs of a candidate: the first 48 bytes of its two sides.
+struct __align__(16) SideHead {
+    double f, a, nrm;
+    int64_t p0;
+    int32_t i, len, y, owner;
+};
+static_assert(sizeof(SideHead) == 48 && offsetof(SideHead, p0) == offsetof(Side, p0) && offsetof(SideHead, i) == offsetof(Side, i) &&
+              offsetof(SideHead, len) == offsetof(Side, len) && offsetof(SideHead, y) == offsetof(Side, y), "SideHead is Side's head");
+struct CandSlot {
+    SideHead up, low;
+};
+
 struct BatchShared {
     Side wup[kWarps], wlow[kWarps];
     unsigned long long wkup[kWarps], wklow[kWarps];
     int wiup[kWarps], wilow[kWarps];
-    CandFull xc[2][kMaxCluster];   // every CTA's candidate, by epoch parity
+    CandSlot xc[2][kMaxCluster];   // every CTA's candidate, by epoch parity
     unsigned long long xbar[2];    // mbarriers of the two parities
     Side none[2];                  // empty I_up / I_low sides
     ResultArea res;
@@ -75,6 +87,9 @@ struct BatchShared {
     int stop;                               // the gap is closed, the step is not taken
     int job;
 };
+// with the FP64 mode's table of the exponential, within what the launch plans
+// (svm_api.cu) leave for static shared memory
+static_assert(sizeof(BatchShared) + sizeof(uint64_t) * kExpfxTabLen <= 12288 - 64, "static shared memory of the batch kernel");
 
 template <int MODE, int LPR>
 __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
@@ -921,8 +936,13 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 bad = __any_sync(0xffffffffu, bad);
                 unsigned long long k1 = kNoKey, k2 = kNoKey;
                 int i1 = INT_MAX, i2 = INT_MAX;
-                long long cc = 0;
-                if (lane < csize && !bad) cand_keys(sh.xc[par][lane], k1, i1, k2, i2, cc);
+                if (lane < csize && !bad) {
+                    const CandSlot &cs = sh.xc[par][lane];
+                    i1 = cs.up.i;
+                    i2 = cs.low.i;
+                    k1 = i1 == INT_MAX ? kNoKey : key_up(cs.up.f);
+                    k2 = i2 == INT_MAX ? kNoKey : key_low(cs.low.f);
+                }
                 const int i1s = i1, i2s = i2;
                 warp_min_ki(k1, i1);
                 warp_min_ki(k2, i2);

@@ -975,6 +975,16 @@ void contract_tc(Arena &ar, const RbfContract &c, const void *sv, int *err, cuda
     CK(launch_rbf_contract_tc(c, sv, ws, err, st));
 }
 
+// What a launch leaves free besides the kernel's static and dynamic shared
+// memory. With the static part it fixes the largest d that is accepted: the
+// two add up to 14,544 bytes (16,592 in the FP64 mode).
+constexpr size_t kSmemSlack = 976;
+
+// What the batched solver's plans leave free: its static part and, in the
+// mixed mode, 60 KB that keep the accepted d where it was when every warp had
+// target fragments of its own (packed units use that room where d is small).
+size_t batch_smem_limit(int mode);
+
 size_t smem_limit()
 {
     int dev = 0, v = 0;
@@ -982,6 +992,8 @@ size_t smem_limit()
     CK(cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     return (size_t)v;
 }
+
+size_t batch_smem_limit(int mode) { return smem_limit() - 12288 - (mode == MODE_MIXED ? 61440 : 0); }
 
 double elapsed_ms(std::chrono::steady_clock::time_point t0)
 {
@@ -1088,7 +1100,7 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
     }
     const int sms = device_sms();
     const int kt = mode == MODE_BINARY ? ktab_len : 0;
-    const size_t lim_dyn = smem_limit() - smo_static_smem(kmode) - 1024;
+    const size_t lim_dyn = smem_limit() - smo_static_smem(kmode) - kSmemSlack;
     // kernel-row cache (FP64 and mixed inputs): every slot holds one kernel
     // row over all n samples; all n rows when they fit (direct), else up to
     // 8192 rows in 4-way sets; the directory goes into each CTA's shared
@@ -2345,7 +2357,7 @@ void batch_prepare(Arena &ar, const svm_csr *X, int precision, cudaStream_t st, 
     }
     B.ktab_len = B.mode == MODE_BINARY ? 2 * D.maxnnz + 1 : 0;
     B.smem = smo_batch_smem(B.mode, B.d_eff, B.ktab_len, D.maxnnz, 0);
-    if (B.smem > smem_limit() - 12288) {
+    if (B.smem > batch_smem_limit(B.mode)) {
         set_err("d = %lld exceeds the shared-memory target rows of the batched solver", (long long)D.d);
         throw Fail{SVM_ERR_UNSUPPORTED};
     }
@@ -3045,7 +3057,7 @@ int train_fixed_impl(const svm_csr *X, const int8_t *y, const svm_params *P, dou
         throw Fail{SVM_ERR_UNSUPPORTED};
     }
     // (the larger of the two modes' static shared memory: the mode is decided below)
-    const size_t lim_dyn = smem_limit() - std::max(smo_static_smem(MODE_BINARY), smo_static_smem(MODE_FP64)) - 1024;
+    const size_t lim_dyn = smem_limit() - std::max(smo_static_smem(MODE_BINARY), smo_static_smem(MODE_FP64)) - kSmemSlack;
     // binary input whose distance tables do not fit in shared memory takes
     // the generic FP64 row pass with norms, as svm_train does
     bool binary = !h.not_binary;
@@ -3407,7 +3419,7 @@ int svm_server_create(const svm_server_config *config, svm_server **out)
         V.cfg = c;
         V.mode = c.precision == SVM_FP64 ? MODE_FP64 : MODE_MIXED;
         V.smem = smo_batch_smem(V.mode, c.max_d, 0, c.max_d, 0);
-        if (V.smem > smem_limit() - 12288) ARG_FAIL("max_d = %d does not fit the engine's shared memory", c.max_d);
+        if (V.smem > batch_smem_limit(V.mode)) ARG_FAIL("max_d = %d does not fit the engine's shared memory", c.max_d);
         V.nclusters = smo_batch_max_clusters(V.mode, c.lanes_per_row, 0, V.smem, c.cluster_size);
         if (V.nclusters < 1) ARG_FAIL("cluster_size %d does not fit this device", c.cluster_size);
         CK(cudaGetDevice(&V.device));
