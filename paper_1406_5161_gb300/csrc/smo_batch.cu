@@ -18,6 +18,7 @@
 // value instead of 8 for index + value).
 #include <cuda_bf16.h>
 
+#include "batch_status.cuh"
 #include "smo_step.cuh"
 
 namespace svmgb {
@@ -54,6 +55,9 @@ struct __align__(16) BatchFinish {
     int pad[2];
 };
 
+// limit of every wait of the kernel
+constexpr int64_t kWaitNs = 10ll * 1000 * 1000 * 1000;
+
 // 16 k-steps x 32 lanes of packed BF16 target pairs (uint2)
 constexpr size_t kFragBytes = (size_t)16 * 32 * sizeof(uint2);
 
@@ -83,7 +87,7 @@ struct BatchShared {
     unsigned char st_u, st_l;
     PairPre pre;
     unsigned long long stage_bar[kWarps];   // packed units: a row warp's unit has landed
-    int bad;                                // a wait gave up: status 2 from here on
+    int bad;                                // a wait of the CTA, from the job's end on of the cluster, gave up
     int stop;                               // the gap is closed, the step is not taken
     int job;
 };
@@ -137,13 +141,13 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
     unsigned epoch = 0;
 
     for (;;) {
-        // a wait of this cluster gave up: its further jobs only report that
-        // (read before the barrier below, so every thread and CTA sees the same)
-        const bool dead = sh.bad != 0;
-        // ---- next job from the work-list, broadcast to the cluster
+        // ---- next job from the work-list, broadcast to the cluster; none once
+        //      a wait of this cluster gave up (agreed on at the end of that
+        //      job): other clusters, or the host, take what is left
         if (crank == 0 && tid == 0) {
             int j = INT_MAX;
-            if (!B.ring) {
+            if (sh.bad) {
+            } else if (!B.ring) {
                 j = atomicAdd(B.next_job, 1);
                 if (j >= B.njobs) j = INT_MAX;
             } else {
@@ -271,12 +275,14 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
         };
         auto wait_unit = [&]() {
             if (!in_flight) return;
-            const int bad = mbar_wait_bounded(stage_bar, stage_parity, 10ll * 1000 * 1000 * 1000, &sh.bad);
+            // (for the copy itself, whatever else failed: none is in flight
+            // when the CTA leaves)
+            const int bad = mbar_wait_bounded(stage_bar, stage_parity, kWaitNs, nullptr);
             if (__any_sync(0xffffffffu, bad) && lane == 0) sh.bad = 1;
             stage_parity ^= 1u;
             in_flight = false;
         };
-        if (!dead && warp >= 1 && warp <= stage_warps && warp - 1 < units) issue_unit(warp - 1);
+        if (warp >= 1 && warp <= stage_warps && warp - 1 < units) issue_unit(warp - 1);
 
         Side up, low;
         side_empty(up, true);
@@ -284,8 +290,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
         bool first = true;
         int64_t iter = 0;
         int prev_valid = 0, prev_len_u = 0, prev_len_l = 0;
-        int status_code = dead ? 2 : 0;
-        while (!dead) {
+        int status_code = JOB_CONVERGED;
+        for (;;) {
             const int buf = (int)(iter & 1);
             Tgt *T = tbuf + (size_t)buf * dmax;
             int *tcu = tcol + (size_t)(buf * 2 + 0) * maxnnz;
@@ -294,8 +300,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             uint32_t kd_wu = 0, kd_wl = 0;
             if (!first) {
                 // (the gap is tested beside the pair step, below)
-                if (up.i == INT_MAX || low.i == INT_MAX) { status_code = 0; break; }
-                if (iter >= J.max_iter) { status_code = dless(thr, low.f - up.f) ? 1 : 0; break; }
+                if (up.i == INT_MAX || low.i == INT_MAX) { status_code = JOB_CONVERGED; break; }
+                if (iter >= J.max_iter) { status_code = dless(thr, low.f - up.f) ? JOB_ITER_LIMIT : JOB_CONVERGED; break; }
                 if (kc_on) {
                     kd_wu = kdir[up.i >> 5];
                     kd_wl = kdir[low.i >> 5];
@@ -843,7 +849,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 }
                 }
             }
-            if (stop) { status_code = 0; break; }   // (every CTA sees the same pair)
+            if (stop) { status_code = JOB_CONVERGED; break; }   // (every CTA sees the same pair)
             // payload of a job row (job-local index r)
             auto make_side = [&](int r) {
                 Side sd;
@@ -932,8 +938,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             }
             if (warp == 0) {
                 const uint32_t parity = (uint32_t)((epoch - 1) >> 1) & 1u;
-                int bad = mbar_wait_bounded(smem_u32(&sh.xbar[par]), parity, 10ll * 1000 * 1000 * 1000, &sh.bad);
-                bad = __any_sync(0xffffffffu, bad);
+                int bad = mbar_wait_bounded(smem_u32(&sh.xbar[par]), parity, kWaitNs, nullptr);
+                bad = __any_sync(0xffffffffu, bad || *(volatile int *)&sh.bad);
                 unsigned long long k1 = kNoKey, k2 = kNoKey;
                 int i1 = INT_MAX, i2 = INT_MAX;
                 if (lane < csize && !bad) {
@@ -960,7 +966,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             __syncthreads();
             if (sh.res.flag) {
                 if (tid == 0) sh.bad = 1;
-                status_code = 2;
+                status_code = JOB_WAIT_GAVE_UP;
                 break;
             }
             prev_valid = first ? 0 : 1;
@@ -1025,7 +1031,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 R.b = t.n0 > 0 ? t.sum_f0 / (double)t.n0 : 0.5 * (up.f + low.f);
                 R.objective = t.sum_a - 0.5 * t.sum_ayfy;
                 R.iters = iter;
-                R.status = sh.bad ? 2 : status_code;
+                R.status = sh.bad ? JOB_WAIT_GAVE_UP : status_code;
                 R.n_sv = (int32_t)t.nsv;
                 B.results[job] = R;
                 if (B.done) {

@@ -207,7 +207,7 @@ __device__ __forceinline__ uint64_t global_ns()
 
 // Waits for the phase of the given parity of a CTA-local mbarrier, giving up
 // after timeout_ns of %globaltimer, or at once when another CTA has flagged
-// an error; returns 1 when it gave up (the caller records the error and
+// an error in *err (NULL: only by time); returns 1 when it gave up (the caller records the error and
 // leaves its loop, so that no wait of the library can outlast its limit).
 __device__ __forceinline__ int mbar_wait_bounded(uint32_t bar, uint32_t parity, int64_t timeout_ns, const int *err)
 {
@@ -219,7 +219,7 @@ __device__ __forceinline__ int mbar_wait_bounded(uint32_t bar, uint32_t parity, 
             const uint64_t now = global_ns();
             if (t0 == 0) t0 = now;
             else if (now - t0 > (uint64_t)timeout_ns) return 1;
-            if (*(volatile const int *)err) return 1;
+            if (err && *(volatile const int *)err) return 1;
         }
     }
     return 0;

@@ -26,6 +26,7 @@
 #include <string>
 #include <vector>
 
+#include "batch_status.cuh"
 #include "svm_internal.cuh"
 
 using namespace svmgb;
@@ -2544,6 +2545,16 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
         q.smem += 128 + (size_t)a.stage_warps * unit;
     };
 
+    // a cluster whose wait gave up takes no further job, so one such job may
+    // leave others without a result: the records are read only when none has
+    auto check_jobs = [](const std::vector<BatchResultDev> &rec) {
+        for (const BatchResultDev &r : rec) {
+            if (r.status != JOB_WAIT_GAVE_UP) continue;
+            set_err("%s", kJobWaitMessage);
+            throw Fail{SVM_ERR_TIMEOUT};
+        }
+    };
+
     // ---- launch shape: given, or picked by timing candidates on a sample
     int cs = cfg->cluster_size, lpr = cfg->lanes_per_row;
     if (lpr > 0) {
@@ -2581,6 +2592,7 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
                 set_pack(SQ, Q, l, c, std::min(maxc, ns));
                 const float ms = batch_run(Q, SQ, l, c, std::min(maxc, ns), next_job, st, &launches);
                 CK(cudaMemcpy(sres.data(), dres, sizeof(BatchResultDev) * ns, cudaMemcpyDeviceToHost));
+                check_jobs(sres);
                 int64_t it = 0;
                 for (auto &r : sres) it += r.iters;
                 const double rate = (double)it / (double)std::max(ms, 1e-3f);
@@ -2653,24 +2665,18 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
         for (int j = 0; j < n_jobs; ++j)
             std::memcpy(jobs[j].alpha_out, ha.data() + offs[j], 8 * jobs[j].n_rows);
     }
+    check_jobs(lres);
     for (int k = 0; k < n_jobs; ++k) hres[order[k]] = lres[k];
     int64_t iters = 0;
     int rc = SVM_OK;
     for (int j = 0; j < n_jobs; ++j) {
-        if (hres[j].status == 2) {
-            set_err("a wait in the batched SMO kernel exceeded its time limit");
-            throw Fail{SVM_ERR_TIMEOUT};
+        const int code = job_result(hres[j], results[j]);
+        if (code < 0) {
+            set_err("job %d: the kernel left no valid result", j);
+            throw Fail{code};
         }
-        svm_result &R = results[j];
-        R.b = hres[j].b;
-        R.b_up = hres[j].b_up;
-        R.b_low = hres[j].b_low;
-        R.objective = hres[j].objective;
-        R.iters = hres[j].iters;
-        R.status = hres[j].status == 1 ? SVM_NOT_CONVERGED : SVM_OK;
-        R.n_sv = hres[j].n_sv;
+        if (code != SVM_OK) rc = code;
         iters += hres[j].iters;
-        if (R.status != SVM_OK) rc = SVM_NOT_CONVERGED;
     }
     cfg->ms_kernel = ms;
     cfg->iters_total = iters;
@@ -2878,20 +2884,17 @@ void srv_admit(Server &S, const std::shared_ptr<SrvJob> &J)
 // collect a finished job (lock held)
 void srv_finish(Server &S, const std::shared_ptr<SrvJob> &J)
 {
-    const BatchResultDev &R = S.res_h[J->slot];
-    J->res.b = R.b;
-    J->res.b_up = R.b_up;
-    J->res.b_low = R.b_low;
-    J->res.objective = R.objective;
-    J->res.iters = R.iters;
-    J->res.status = R.status == 1 ? SVM_NOT_CONVERGED : SVM_OK;
-    J->res.n_sv = R.n_sv;
-    J->alpha.resize(J->n);
-    CK(cudaMemcpyAsync(J->alpha.data(), J->alpha_d, 8 * J->n, cudaMemcpyDeviceToHost, S.s_side));
+    const int rc = job_result(S.res_h[J->slot], J->res);
+    if (rc >= 0) {
+        J->alpha.resize(J->n);
+        CK(cudaMemcpyAsync(J->alpha.data(), J->alpha_d, 8 * J->n, cudaMemcpyDeviceToHost, S.s_side));
+    } else if (!J->cancelled) {
+        J->err = rc == SVM_ERR_TIMEOUT ? kJobWaitMessage : "the engine left no valid result";
+    }
     CK(cudaFreeAsync(J->mem, S.s_side));
     CK(cudaStreamSynchronize(S.s_side));
     J->mem = nullptr;
-    J->rc = J->cancelled ? SVM_ERR_CANCELLED : J->res.status;
+    J->rc = J->cancelled ? SVM_ERR_CANCELLED : rc;
     J->state = 2;
     J->t_done = std::chrono::steady_clock::now();
     S.used -= J->bytes;

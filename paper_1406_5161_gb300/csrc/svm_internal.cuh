@@ -186,7 +186,7 @@ struct BatchJobDev {
 struct BatchResultDev {
     double b, b_up, b_low, objective;
     int64_t iters;
-    int32_t status;            // 0 converged, 1 iteration limit, 2 a wait gave up
+    int32_t status;            // how it ended (batch_status.cuh)
     int32_t n_sv;
 };
 
