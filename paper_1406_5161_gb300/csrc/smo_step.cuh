@@ -747,36 +747,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
     Side up, low;
     side_empty(up, true);
     side_empty(low, false);
-    auto load_mask = [&](Side &sd) {
-        if constexpr (BITS) {
-#pragma unroll
-            for (int q = 0; q < W4; ++q) {
-                const uint4 v = bits_g[(size_t)sd.i * W4 + q];
-                sd.m[4 * q] = v.x; sd.m[4 * q + 1] = v.y; sd.m[4 * q + 2] = v.z; sd.m[4 * q + 3] = v.w;
-            }
-        }
-    };
-    bool first = A.select_only != 0;
-    if (!first) {
-        up.f = C0.b_up; up.a = C0.a_up; up.i = C0.i_up;
-        low.f = C0.b_low; low.a = C0.a_low; low.i = C0.i_low;
-        if (up.i >= 0 && up.i < A.n) {
-            up.p0 = A.indptr[up.i];
-            up.len = (int)(A.indptr[up.i + 1] - up.p0);
-            up.y = A.y[up.i];
-            if constexpr (MODE == MODE_MIXED) up.nrm = norm_bits(A.normf[up.i]);
-            if constexpr (MODE == MODE_FP64) up.nrm = A.norm[up.i];
-            load_mask(up);
-        }
-        if (low.i >= 0 && low.i < A.n) {
-            low.p0 = A.indptr[low.i];
-            low.len = (int)(A.indptr[low.i + 1] - low.p0);
-            low.y = A.y[low.i];
-            if constexpr (MODE == MODE_MIXED) low.nrm = norm_bits(A.normf[low.i]);
-            if constexpr (MODE == MODE_FP64) low.nrm = A.norm[low.i];
-            load_mask(low);
-        }
-    }
+    bool first = true;   // every launch begins with a selection pass
     // one cluster over the whole grid: candidates go to every CTA as
     // asynchronous stores whose bytes each CTA counts on its own mbarrier
     // (one per epoch parity; the CTA's own arrival sets the expected bytes)
@@ -807,21 +778,6 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
         cluster.sync();
     } else {
         __syncthreads();
-    }
-
-    if constexpr (LEAN) {
-        // a pair handed over from an earlier launch: its rows' owners
-        auto locate = [&](Side &sd) {
-            if (sd.i < 0 || sd.i >= A.n) { sd.i = INT_MAX; return; }
-            int o = (int)((int64_t)sd.i * G / A.n);
-            while (o + 1 < G && seg_lo(A.n, G, o + 1) <= sd.i) ++o;
-            sd.owner = o;
-            sd.p0 -= A.indptr[seg_lo(A.n, G, o)];
-        };
-        if (!first) {
-            locate(up);
-            locate(low);
-        }
     }
 
     // ---- accessors (segment-local row r, global sample lo + r)
@@ -919,7 +875,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
     unsigned kd_need = 0;
     bool filled = false;   // this step filled its target buffer
     int exit_reason = 0;
-    bool gap_open = first || dless(A.thr, low.f - up.f);   // stopping test of the pair in up / low
+    bool gap_open = true;            // stopping test of the pair in up / low
     int prev_valid = 0;              // buffer (1 - buf) holds the previous targets
     int prev_len_u = 0, prev_len_l = 0;
     // optional per-phase cycle counts of CTA 0 (one clock read per phase)
@@ -2476,10 +2432,6 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
         SmoCtrl *c = A.ctrl;
         c->b_up = up.f;
         c->b_low = low.f;
-        c->a_up = up.a;
-        c->a_low = low.a;
-        c->i_up = up.i == INT_MAX ? -1 : (A.gmap ? A.gmap[up.i] : up.i);
-        c->i_low = low.i == INT_MAX ? -1 : (A.gmap ? A.gmap[low.i] : low.i);
         c->iter = iter;
         c->counter = counter;
         c->active = total;

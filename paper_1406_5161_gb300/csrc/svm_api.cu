@@ -1407,7 +1407,6 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
     std::memset(&hc, 0, sizeof hc);
     hc.counter = h;
     hc.active = n;
-    hc.i_up = hc.i_low = -1;
 
     SmoArgs A;
     std::memset(&A, 0, sizeof A);
@@ -1520,7 +1519,7 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
     lv.push_back(Level{n, D.nnz, D.indptr, D.indices, vals_fp32, D.vmix, D.normf, D.norm, D.y, bits,
                        alpha, f, status, act, seg_cnt, nullptr, nullptr, top, dmat, top_kc, ew, ew64});
     int64_t relayouts = 0;
-    auto launch_level = [&](const Level &L, int select_only, double thr, int64_t hh, int64_t limit) {
+    auto launch_level = [&](const Level &L, double thr, int64_t hh, int64_t limit) {
         A.n = L.n;
         A.G = L.shape.G;
         A.indptr = L.indptr;
@@ -1558,7 +1557,6 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
         A.thr = thr;
         A.h = hh;
         A.iter_limit = limit;
-        A.select_only = select_only;
         CK(cudaEventRecord(e0, st));
         CK(launch_smo_persistent(kmode, lpr, A, L.shape.smem, st, L.shape.cs));
         CK(cudaEventRecord(e1, st));
@@ -1695,13 +1693,12 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
     const int32_t *inc_idx = nullptr;
     int64_t inc_m = 0;
     double *inc_a0 = nullptr;
-    auto run = [&](int select_only, double thr, int64_t hh, int64_t limit) {
-        int sel = select_only;
+    auto run = [&](double thr, int64_t hh, int64_t limit) {
         bool top = true;
         if (inc_track) inc_ok = false;
         for (;;) {
             const int64_t se0 = hc.shrink_events;
-            launch_level(lv.back(), sel, thr, hh, limit);
+            launch_level(lv.back(), thr, hh, limit);
             if (hc.exit_reason != 2) break;
             const bool one_event = top && hc.shrink_events - se0 == 1;
             // the same state continues on the gathered rows (a selection
@@ -1717,7 +1714,6 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
                 inc_ok = true;
             }
             top = false;
-            sel = 1;
         }
         while (lv.size() > 1) pop_level();
         relayout_ok = relayout_on;
@@ -1735,7 +1731,7 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
     int64_t inc_recons = 0;
     for (;;) {
         inc_track = inc_allowed && shrinking;
-        run(1, thr, shrinking ? h : 0, max_iter);
+        run(thr, shrinking ? h : 0, max_iter);
         inc_track = false;
         if (hc.exit_reason == 1) {
             status_code = SVM_NOT_CONVERGED;
@@ -1851,7 +1847,7 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
         ++launches;
         hc.active = n;
         // b_up / b_low over all samples (a selection pass, no steps)
-        run(1, 2.0 * P->tau, 0, hc.iter);
+        run(2.0 * P->tau, 0, hc.iter);
         if (!(hc.b_low - hc.b_up > 2.0 * P->tau)) break;
         if (sp.recon == SVM_RECON_SINGLE) shrinking = false;
         else hc.counter = h;
@@ -3125,7 +3121,6 @@ int train_fixed_impl(const svm_csr *X, const int8_t *y, const svm_params *P, dou
     SmoCtrl hc;
     std::memset(&hc, 0, sizeof hc);
     hc.active = n;
-    hc.i_up = hc.i_low = -1;
     SmoArgs A;
     std::memset(&A, 0, sizeof A);
     A.n = n;
@@ -3154,7 +3149,6 @@ int train_fixed_impl(const svm_csr *X, const int8_t *y, const svm_params *P, dou
     A.thr = 2.0 * P->tau;
     A.iter_limit = P->max_iter > 0 ? P->max_iter : 100 * n + 1000000;
     A.h = 0;
-    A.select_only = 1;
     A.wss2 = (P->flags & SVM_FLAG_WSS2) != 0;
     A.timeout_ns = 10ll * 1000 * 1000 * 1000;
     // every call starts from a zeroed exchange area and a fresh control block

@@ -62,13 +62,11 @@ __host__ __device__ constexpr int mode_words(int m) { return m == MODE_BITS8 ? 8
 
 // Solver state carried between launches of the persistent step kernel.
 struct SmoCtrl {
-    double b_up, b_low;        // f at i_up / i_low over the active set
-    double a_up, a_low;        // alpha of i_up / i_low
+    double b_up, b_low;        // extremes of f over the active set (Eq. bminmax)
     int64_t iter;              // SMO steps done
     int64_t counter;           // shrink counter
     int64_t active;            // active-set size
     int64_t row_visits;        // sum of active-set sizes over the steps
-    int32_t i_up, i_low;
     int32_t exit_reason;       // 0: gap <= thr, 1: iteration limit, 2: active set
                                // below SmoArgs::compact_below
     int32_t err;               // 0 ok, 1 timeout in a grid-wide wait
@@ -122,7 +120,6 @@ struct SmoArgs {
     double C, gamma, thr;
     int64_t iter_limit;
     int64_t h;                 // shrink counter reset value (0: no shrinking)
-    int32_t select_only;       // start with a selection pass
     int32_t phase_times;       // record per-phase cycle counts (CTA 0)
     int64_t *cta_cycles;       // with phase_times: per-CTA cycles of work per launch (G)
     int64_t timeout_ns;
