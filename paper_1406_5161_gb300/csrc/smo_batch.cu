@@ -217,7 +217,9 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
         if constexpr (MODE == MODE_FP64) {
             if (xd) tclear = make_double2(__hiloint2double(xd_tmin, 0), __hiloint2double(xd_tmin, 0));
         }
-        // ---- job set-up: tables, empty target buffers, alpha = 0, f = -y
+        // ---- job set-up: tables, empty target buffers, and alpha = 0, f = -y
+        //      unless an earlier launch left them after iter0 steps (the
+        //      selection pass below then finds the pair that one had chosen)
         for (int c = tid; c < 2 * dmax; c += kThreads) tbuf[c] = tclear;
         if constexpr (MODE == MODE_BINARY) {
             for (int k = tid; k < B.ktab_len; k += kThreads) {
@@ -227,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 ktab[B.ktab_len + k] = eta > 1e-12 ? 1.0 / eta : 0.0;
             }
         }
-        for (int r = lo + tid; r < hi; r += kThreads) {
+        for (int r = lo + tid; r < hi && J.iter0 == 0; r += kThreads) {
             const int8_t yr = yj[r];
             aj[r] = 0.0;
             fj[r] = -(double)yr;
@@ -288,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
         side_empty(up, true);
         side_empty(low, false);
         bool first = true;
-        int64_t iter = 0;
+        int64_t iter = J.iter0;
         int prev_valid = 0, prev_len_u = 0, prev_len_l = 0;
         int status_code = JOB_CONVERGED;
         for (;;) {

@@ -76,6 +76,7 @@ struct Fail {
 // back too when an allocation fails for want of memory. The driver orders its
 // reuse across streams and threads.
 constexpr size_t kPoolKeepBytes = (size_t)4 << 30;
+constexpr size_t kBatchCacheFree = (size_t)3 << 30;   // a buffer the pool keeps beside a call's others
 constexpr int kPoolDevices = 64;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kPoolDevices] = {};
@@ -2621,34 +2622,103 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
     int ncl = in_flight(maxc);
     // Kernel-row cache (FP64): each cluster's job keeps the kernel rows it
     // computes, all of them when its kernel matrix fits the cluster's part of
-    // the budget (svm_train's). 45 jobs of 1,500 x 20 rows: 54 ms without, 33
-    // with it. Mixed rows gain nothing: of the rows of the 90 one-vs-one jobs
-    // (2,200-5,800 x 256) a quarter of the steps find both, 140 -> 126 ms, and
-    // mapping the 10 GB takes the difference.
-    if (P.mode == MODE_FP64) {
-        auto matrix_bytes = [&](int64_t m) { return m * ((m + 31) / 32 * 32) * 8; };
-        const int words = (int)std::min<int64_t>((most_rows + 31) / 32, 4096);
-        BatchPlan Q = P;
-        Q.smem = smo_batch_smem(P.mode, P.d_eff, P.ktab_len, D.maxnnz, words);
-        const int qmax = Q.smem <= smem_limit() - 12288 ? batch_clusters(Q, lpr, cs) : 0;
+    // the budget (svm_train's). 45 jobs of 1,500 x 20 rows: 27.5 ms of kernel
+    // without, 18.9 with it. Mixed rows gain nothing: of the rows of the 90
+    // one-vs-one jobs (2,200-5,800 x 256) a quarter of the steps find both, 140
+    // -> 126 ms, and mapping the 10 GB takes the difference.
+    struct CachePlan {
+        size_t bytes, smem;
+        int64_t stride;
+        int words;
+    };
+    void *kc_buf = nullptr;
+    size_t kc_have = 0;
+    auto plan_cache = [&](const BatchPlan &q, int l, int c, int ncl) {
+        CachePlan k = {0, 0, 0, 0};
+        if (P.mode != MODE_FP64) return k;
+        auto matrix_bytes = [](int64_t m) { return m * ((m + 31) / 32 * 32) * 8; };
+        k.words = (int)std::min<int64_t>((most_rows + 31) / 32, 4096);
+        BatchPlan Q = q;
+        Q.smem = k.smem = smo_batch_smem(P.mode, P.d_eff, P.ktab_len, D.maxnnz, k.words);
         size_t fr = 0, tot = 0;
-        if (qmax >= maxc && cudaMemGetInfo(&fr, &tot) == cudaSuccess) {
-            const int64_t stride = std::min<int64_t>(matrix_bytes(most_rows),
-                                                     (int64_t)std::min<size_t>(fr / 2, (size_t)32 << 30) / ncl) / 256 * 256;
-            if (stride >= matrix_bytes(least_rows)) {
-                if (void *kc = try_alloc((size_t)stride * ncl)) {
-                    P.smem = Q.smem;
-                    A.kc = kc;
-                    A.kc_stride = stride;
-                    A.kdir_words = words;
-                }
-            }
+        if (Q.smem > smem_limit() - 12288 || batch_clusters(Q, l, c) < batch_clusters(q, l, c)) return k;
+        if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return k;
+        k.stride = std::min<int64_t>(matrix_bytes(most_rows),
+                                     (int64_t)std::min<size_t>((fr + kc_have) / 2, (size_t)32 << 30) / ncl) / 256 * 256;
+        if (k.stride >= matrix_bytes(least_rows)) k.bytes = (size_t)k.stride * ncl;
+        return k;
+    };
+    auto set_cache = [&](BatchArgs &a, BatchPlan &q, const CachePlan &k) {
+        if (k.bytes > kc_have) {
+            kc_buf = try_alloc(k.bytes);
+            kc_have = kc_buf ? k.bytes : 0;
         }
-    }
-    set_pack(A, P, lpr, cs, ncl);
-    const float ms = batch_run(P, A, lpr, cs, ncl, next_job, st, &launches);
+        if (!k.bytes || !kc_buf) return;
+        q.smem = k.smem;
+        a.kc = kc_buf;
+        a.kc_stride = k.stride;
+        a.kdir_words = k.words;
+    };
+
+    // One launch over the jobs of the list still in `todo`, each for at most
+    // `steps` further steps; what it leaves unfinished stays in `todo`.
     std::vector<BatchResultDev> lres(n_jobs), hres(n_jobs);
-    CK(cudaMemcpyAsync(lres.data(), dres, sizeof(BatchResultDev) * n_jobs, cudaMemcpyDeviceToHost, st));
+    std::vector<int> todo(n_jobs);
+    for (int k = 0; k < n_jobs; ++k) todo[k] = k;
+    float ms = 0.f;
+    auto run_jobs = [&](BatchArgs a, BatchPlan q, int64_t steps) {
+        const bool resumed = (int)todo.size() < n_jobs || lres[todo[0]].iters > 0;
+        if (resumed || steps < INT64_MAX) {
+            std::vector<BatchJobDev> part;
+            for (int k : todo) {
+                part.push_back(list[k]);
+                part.back().iter0 = lres[k].iters;
+                part.back().max_iter = list[k].max_iter - lres[k].iters > steps ? lres[k].iters + steps : list[k].max_iter;
+            }
+            CK(cudaMemcpyAsync(djobs, part.data(), sizeof(BatchJobDev) * part.size(), cudaMemcpyHostToDevice, st));
+        }
+        a.njobs = (int)todo.size();
+        ms += batch_run(q, a, lpr, cs, std::min(ncl, a.njobs), next_job, st, &launches);
+        std::vector<BatchResultDev> rec(todo.size());
+        CK(cudaMemcpyAsync(rec.data(), dres, sizeof(BatchResultDev) * rec.size(), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        check_jobs(rec);
+        std::vector<int> left;
+        for (size_t i = 0; i < rec.size(); ++i) {
+            const int k = todo[i];
+            lres[k] = rec[i];
+            if (rec[i].status == JOB_ITER_LIMIT && rec[i].iters < list[k].max_iter) left.push_back(k);
+        }
+        todo = std::move(left);
+    };
+    set_pack(A, P, lpr, cs, ncl);
+    CachePlan kp = plan_cache(P, lpr, cs, ncl);
+    if (kp.bytes > kBatchCacheFree) {
+        // More kernel rows than the pool keeps between calls are paid for in
+        // every call: mapping and giving back take 1.7 ms per GB (20 easy
+        // problems of 16,000 rows, 283 steps each: 22 ms without a cache, 65
+        // with whole kernel matrices in 32 GB). So the jobs run without a cache
+        // until that has taken as long as the mapping would, and only what is
+        // then unfinished continues with one, if its step limit leaves it time
+        // to save as much: never much more than twice the better of the two.
+        const double map_ms = 1.7e-9 * (double)kp.bytes;
+        for (int64_t steps = 250; !todo.empty() && ms < map_ms;) {
+            const float before = ms;
+            run_jobs(A, P, steps);
+            steps = std::max<int64_t>(50, (int64_t)((double)steps * (map_ms - ms) / std::max(ms - before, 1e-3f)));
+        }
+        int64_t taken = 1, still = 0;   // steps of the longest job so far, and at most from here on
+        for (int k : todo) {
+            taken = std::max<int64_t>(taken, lres[k].iters);
+            still = std::max<int64_t>(still, list[k].max_iter - lres[k].iters);
+        }
+        kp.bytes = 0;
+        if ((double)still * ms > 2.0 * map_ms * (double)taken) kp = plan_cache(P, lpr, cs, std::min<int>(ncl, (int)todo.size()));
+    }
+    if (!todo.empty()) {
+        set_cache(A, P, kp);
+        run_jobs(A, P, INT64_MAX);
+    }
     if (X->on_device) {
         for (int j = 0; j < n_jobs; ++j)
             CK(cudaMemcpyAsync(jobs[j].alpha_out, alpha + offs[j], 8 * jobs[j].n_rows, cudaMemcpyDeviceToDevice,
@@ -2661,7 +2731,6 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
         for (int j = 0; j < n_jobs; ++j)
             std::memcpy(jobs[j].alpha_out, ha.data() + offs[j], 8 * jobs[j].n_rows);
     }
-    check_jobs(lres);
     for (int k = 0; k < n_jobs; ++k) hres[order[k]] = lres[k];
     int64_t iters = 0;
     int rc = SVM_OK;

@@ -177,6 +177,7 @@ struct BatchJobDev {
     int32_t pad;
     double C, gamma, tau;
     int64_t max_iter;
+    int64_t iter0;             // > 0: continue after that many steps of an earlier launch
     XdFormat xd;               // FP64 mode: exact inner products (xd.on)
 };
 
