@@ -2542,6 +2542,46 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
         q.smem += 128 + (size_t)a.stage_warps * unit;
     };
 
+    // Kernel-row cache (FP64): each cluster's job keeps the kernel rows it
+    // computes, all of them when its kernel matrix fits the cluster's part of
+    // the budget (svm_train's). 45 jobs of 1,500 x 20 rows: 27.5 ms of kernel
+    // without, 18.9 with it. Mixed rows gain nothing: of the rows of the 90
+    // one-vs-one jobs (2,200-5,800 x 256) a quarter of the steps find both, 140
+    // -> 126 ms, and mapping the 10 GB takes the difference.
+    struct CachePlan {
+        size_t bytes, smem;
+        int64_t stride;
+        int words;
+    };
+    void *kc_buf = nullptr;
+    size_t kc_have = 0;
+    auto plan_cache = [&](const BatchPlan &q, int l, int c, int ncl) {
+        CachePlan k = {0, 0, 0, 0};
+        if (P.mode != MODE_FP64) return k;
+        auto matrix_bytes = [](int64_t m) { return m * ((m + 31) / 32 * 32) * 8; };
+        k.words = (int)std::min<int64_t>((most_rows + 31) / 32, 4096);
+        BatchPlan Q = q;
+        Q.smem = k.smem = smo_batch_smem(P.mode, P.d_eff, P.ktab_len, D.maxnnz, k.words);
+        size_t fr = 0, tot = 0;
+        if (Q.smem > smem_limit() - 12288 || batch_clusters(Q, l, c) < batch_clusters(q, l, c)) return k;
+        if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return k;
+        k.stride = std::min<int64_t>(matrix_bytes(most_rows),
+                                     (int64_t)std::min<size_t>((fr + kc_have) / 2, (size_t)32 << 30) / ncl) / 256 * 256;
+        if (k.stride >= matrix_bytes(least_rows)) k.bytes = (size_t)k.stride * ncl;
+        return k;
+    };
+    auto set_cache = [&](BatchArgs &a, BatchPlan &q, const CachePlan &k) {
+        if (k.bytes > kc_have) {
+            kc_buf = try_alloc(k.bytes);
+            kc_have = kc_buf ? k.bytes : 0;
+        }
+        if (!k.bytes || !kc_buf) return;
+        q.smem = k.smem;
+        a.kc = kc_buf;
+        a.kc_stride = k.stride;
+        a.kdir_words = k.words;
+    };
+
     // a cluster whose wait gave up takes no further job, so one such job may
     // leave others without a result: the records are read only when none has
     auto check_jobs = [](const std::vector<BatchResultDev> &rec) {
@@ -2587,6 +2627,9 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
                 BatchPlan Q = P;
                 BatchArgs SQ = S;
                 set_pack(SQ, Q, l, c, std::min(maxc, ns));
+                // (with the cache where the solve begins with it)
+                const CachePlan k = plan_cache(P, l, c, std::min(maxc, ns));
+                if (k.bytes <= kBatchCacheFree) set_cache(SQ, Q, k);
                 const float ms = batch_run(Q, SQ, l, c, std::min(maxc, ns), next_job, st, &launches);
                 CK(cudaMemcpy(sres.data(), dres, sizeof(BatchResultDev) * ns, cudaMemcpyDeviceToHost));
                 check_jobs(sres);
@@ -2620,46 +2663,6 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
         return cfg->clusters > 0 ? std::min(k, cfg->clusters) : k;
     };
     int ncl = in_flight(maxc);
-    // Kernel-row cache (FP64): each cluster's job keeps the kernel rows it
-    // computes, all of them when its kernel matrix fits the cluster's part of
-    // the budget (svm_train's). 45 jobs of 1,500 x 20 rows: 27.5 ms of kernel
-    // without, 18.9 with it. Mixed rows gain nothing: of the rows of the 90
-    // one-vs-one jobs (2,200-5,800 x 256) a quarter of the steps find both, 140
-    // -> 126 ms, and mapping the 10 GB takes the difference.
-    struct CachePlan {
-        size_t bytes, smem;
-        int64_t stride;
-        int words;
-    };
-    void *kc_buf = nullptr;
-    size_t kc_have = 0;
-    auto plan_cache = [&](const BatchPlan &q, int l, int c, int ncl) {
-        CachePlan k = {0, 0, 0, 0};
-        if (P.mode != MODE_FP64) return k;
-        auto matrix_bytes = [](int64_t m) { return m * ((m + 31) / 32 * 32) * 8; };
-        k.words = (int)std::min<int64_t>((most_rows + 31) / 32, 4096);
-        BatchPlan Q = q;
-        Q.smem = k.smem = smo_batch_smem(P.mode, P.d_eff, P.ktab_len, D.maxnnz, k.words);
-        size_t fr = 0, tot = 0;
-        if (Q.smem > smem_limit() - 12288 || batch_clusters(Q, l, c) < batch_clusters(q, l, c)) return k;
-        if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return k;
-        k.stride = std::min<int64_t>(matrix_bytes(most_rows),
-                                     (int64_t)std::min<size_t>((fr + kc_have) / 2, (size_t)32 << 30) / ncl) / 256 * 256;
-        if (k.stride >= matrix_bytes(least_rows)) k.bytes = (size_t)k.stride * ncl;
-        return k;
-    };
-    auto set_cache = [&](BatchArgs &a, BatchPlan &q, const CachePlan &k) {
-        if (k.bytes > kc_have) {
-            kc_buf = try_alloc(k.bytes);
-            kc_have = kc_buf ? k.bytes : 0;
-        }
-        if (!k.bytes || !kc_buf) return;
-        q.smem = k.smem;
-        a.kc = kc_buf;
-        a.kc_stride = k.stride;
-        a.kdir_words = k.words;
-    };
-
     // One launch over the jobs of the list still in `todo`, each for at most
     // `steps` further steps; what it leaves unfinished stays in `todo`.
     std::vector<BatchResultDev> lres(n_jobs), hres(n_jobs);
