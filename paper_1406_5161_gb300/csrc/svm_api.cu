@@ -2857,7 +2857,7 @@ void srv_admit(Server &S, const std::shared_ptr<SrvJob> &J)
     const bool mixed = S.mode == MODE_MIXED;
     const bool dense = mixed && J->nnz == J->n * J->d;
     const int dpad = (int)((J->d + 7) & ~7ll);
-    CK(cudaMallocAsync(&J->mem, J->bytes, st));
+    J->mem = pool_alloc(J->bytes, st);
     unsigned char *p = static_cast<unsigned char *>(J->mem);
     auto take = [&](size_t x) {
         unsigned char *r = p;
