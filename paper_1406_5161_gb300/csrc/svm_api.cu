@@ -121,6 +121,23 @@ void *pool_alloc(size_t bytes, cudaStream_t st)
     return p;
 }
 
+// Device memory that an allocation of this library can have: what the device
+// has free and what the pool keeps unused (0 where the runtime cannot tell).
+size_t available_bytes()
+{
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    uint64_t reserved = 0, used = 0;
+    cudaMemPool_t pool = device_pool();
+    if (pool && cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
+        fr += reserved - used;
+    return fr;
+}
+
 // Stream-ordered device allocations released when the scope ends; small ones
 // are cut from slabs.
 struct Arena {
@@ -1139,9 +1156,7 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
     if ((kmode == MODE_FP64 && P->cache_mb >= 0) || (kmode == MODE_MIXED && P->cache_mb > 0)) {
         size_t budget = (size_t)P->cache_mb << 20;
         if (P->cache_mb == 0) {
-            size_t fr = 0, tot = 0;
-            if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) fr = 0;
-            budget = std::min<size_t>(fr / 2, (size_t)32 << 30);
+            budget = std::min<size_t>(available_bytes() / 2, (size_t)32 << 30);
         }
         top_kc = plan_kc(n, budget);
         if (top_kc.slots > 0) {
@@ -2562,11 +2577,9 @@ int train_batch_impl(const svm_csr *X, const svm_job *jobs, int32_t n_jobs, svm_
         k.words = (int)std::min<int64_t>((most_rows + 31) / 32, 4096);
         BatchPlan Q = q;
         Q.smem = k.smem = smo_batch_smem(P.mode, P.d_eff, P.ktab_len, D.maxnnz, k.words);
-        size_t fr = 0, tot = 0;
         if (Q.smem > smem_limit() - 12288 || batch_clusters(Q, l, c) < batch_clusters(q, l, c)) return k;
-        if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return k;
         k.stride = std::min<int64_t>(matrix_bytes(most_rows),
-                                     (int64_t)std::min<size_t>((fr + kc_have) / 2, (size_t)32 << 30) / ncl) / 256 * 256;
+                                     (int64_t)std::min<size_t>((available_bytes() + kc_have) / 2, (size_t)32 << 30) / ncl) / 256 * 256;
         if (k.stride >= matrix_bytes(least_rows)) k.bytes = (size_t)k.stride * ncl;
         return k;
     };

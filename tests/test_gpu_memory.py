@@ -52,3 +52,11 @@ def test_served_job_takes_the_memory_that_is_kept():
         with _Filled(400 * MiB):   # the job needs 640 MB
             out = srv.wait(srv.submit(X, y, 1.0, 1e-3, max_iter=5), timeout=30.0)
     assert out is not None and out["status"] == pkg.SVM_NOT_CONVERGED
+
+
+def test_repeated_call_gets_the_same_cache():
+    p = synth.small_dense(20000, 8, seed=3, sep=0.5)
+    X, y = pkg.to_device(p.X), torch.as_tensor(p.y, device="cuda")
+    with _Filled(6 << 30):
+        slots = [pkg.svm_train(X, y, 1.0, 0.1, 1e-3, max_iter=100)["stats"]["cache_slots"] for _ in range(3)]
+    assert slots[0] > 0 and slots == [slots[0]] * 3, slots
