@@ -26,8 +26,9 @@
  *     return, outputs are written and the library's device work is done.
  *   - The library allocates its own device workspace (stream-ordered) and
  *     frees it before returning, into a pool of its own that keeps up to 4 GiB
- *     for later calls (given back when an allocation would fail otherwise);
- *     inputs are only read, never kept.
+ *     per device for later calls. What it keeps serves this library's
+ *     allocations alone; svm_trim_memory gives it back to the device. Inputs
+ *     are only read, never kept.
  */
 #ifndef SVM_GB300_H
 #define SVM_GB300_H
@@ -523,6 +524,14 @@ int svm_diag_wait_timeout(int64_t limit_ns, void *stream);
  * that the contraction can be reported against the exp rate it is bound by.
  * ex2_per_s receives instructions per second. Synchronous. */
 int svm_diag_sfu_rate(double *ex2_per_s, void *stream);
+
+/* Gives the device memory that the library keeps for later calls on the
+ * current device back to it (up to 4 GiB, see above), for callers whose other
+ * allocators need it; memory in use (models, served jobs, calls of other
+ * threads) stays. The next call maps what it needs anew (0.85 ms per GB).
+ *   stream   the stream of the calls before, which is waited for
+ * Returns SVM_OK or SVM_ERR_CUDA. */
+int svm_trim_memory(void *stream);
 
 /* Message for the last failing call on this thread ("" if none). */
 const char *svm_last_error(void);

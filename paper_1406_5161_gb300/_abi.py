@@ -126,6 +126,8 @@ def load(build_if_missing: bool = True):
             lib.svm_train_fixed_workspace.argtypes = [P, P, P, P, P, P]
             lib.svm_diag_wait_timeout.restype = ct.c_int
             lib.svm_diag_wait_timeout.argtypes = [ct.c_int64, P]
+            lib.svm_trim_memory.restype = ct.c_int
+            lib.svm_trim_memory.argtypes = [P]
             lib.svm_diag_sfu_rate.restype = ct.c_int
             lib.svm_diag_sfu_rate.argtypes = [P, P]
             lib.svm_model_create.restype = ct.c_int
@@ -157,6 +159,13 @@ def svm_diag_wait_timeout(limit_ns: int, stream=None) -> int:
     """Runs the library's bounded device-side wait on a barrier that nothing
     completes; returns the status (SVM_ERR_TIMEOUT expected)."""
     return int(load().svm_diag_wait_timeout(int(limit_ns), _stream_ptr(stream)))
+
+
+def svm_trim_memory(stream=None) -> None:
+    """Give the device memory that the library keeps for later calls back."""
+    rc = load().svm_trim_memory(_stream_ptr(stream))
+    if rc < 0:
+        raise SvmError(rc, svm_last_error())
 
 
 def svm_last_error() -> str:

@@ -73,8 +73,9 @@ struct Fail {
 // so each call paid for mapping it again (the 32 MB kernel-row cache of a
 // 2,000-row solve alone about 0.3 ms of 6.4). This one keeps up to
 // kPoolKeepBytes between calls and gives back the rest; what it keeps is given
-// back too when an allocation fails for want of memory. The driver orders its
-// reuse across streams and threads.
+// back when one of the library's own allocations fails for want of memory, and
+// by svm_trim_memory (other allocators of the process cannot reach it). The
+// driver orders its reuse across streams and threads.
 constexpr size_t kPoolKeepBytes = (size_t)4 << 30;
 constexpr size_t kBatchCacheFree = (size_t)3 << 30;   // a buffer the pool keeps beside a call's others
 constexpr int kPoolDevices = 64;
@@ -3744,6 +3745,21 @@ int svm_train_fixed_workspace(const svm_csr *X, const int8_t *y, const svm_param
     g_err.clear();
     try {
         return train_fixed_impl(X, y, params, alpha_out, b_out, iters_out);
+    } catch (const Fail &f) {
+        return f.code;
+    } catch (...) {
+        set_err("unexpected host exception");
+        return SVM_ERR_CUDA;
+    }
+}
+
+int svm_trim_memory(void *stream)
+{
+    g_err.clear();
+    try {
+        CK(cudaStreamSynchronize(as_stream(stream)));
+        if (cudaMemPool_t pool = device_pool()) CK(cudaMemPoolTrimTo(pool, 0));
+        return SVM_OK;
     } catch (const Fail &f) {
         return f.code;
     } catch (...) {

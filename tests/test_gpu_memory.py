@@ -60,3 +60,14 @@ def test_repeated_call_gets_the_same_cache():
     with _Filled(6 << 30):
         slots = [pkg.svm_train(X, y, 1.0, 0.1, 1e-3, max_iter=100)["stats"]["cache_slots"] for _ in range(3)]
     assert slots[0] > 0 and slots == [slots[0]] * 3, slots
+
+
+def test_trim_gives_the_kept_memory_back():
+    _keep_some()
+    torch.cuda.synchronize()
+    before, _ = torch.cuda.mem_get_info()
+    pkg.svm_trim_memory()
+    after, _ = torch.cuda.mem_get_info()
+    assert after - before >= 2 << 30, (before, after)
+    p = synth.small_dense(300, 8, seed=1)   # and the library goes on
+    assert pkg.svm_train(p.X, p.y, 1.0, 0.1, 1e-3)["status"] == pkg.SVM_OK
