@@ -5,6 +5,7 @@
 // prediction runs in the library's CUDA kernels. The host reads a small
 // control block between phases (after each persistent launch) to apply the
 // phase logic of Algorithm 5.
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -68,6 +69,37 @@ struct Fail {
         throw Fail{SVM_ERR_ARG};      \
     } while (0)
 
+// Identifies the device's current context. What the library keeps between
+// calls belongs to one context; a process that resets its device goes on with
+// another, where the old pool and page-locked buffers no longer exist.
+// 0: there is none yet.
+unsigned long long current_context()
+{
+    using GetId = CUresult (*)(CUcontext, unsigned long long *);
+    static std::atomic<GetId> fn{nullptr};   // the driver's entry, once found
+    GetId f = fn.load();
+    if (!f) {
+        void *q = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &q, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            (void)cudaGetLastError();
+            return 0;
+        }
+        fn = f = reinterpret_cast<GetId>(q);
+    }
+    unsigned long long id = 0;
+    return f(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+// ... made by the runtime where there is none
+unsigned long long context_id()
+{
+    unsigned long long id = current_context();
+    if (id) return id;
+    CK(cudaFree(nullptr));
+    return current_context();
+}
+
 // The library's own pool of stream-ordered device memory, one per device. The
 // default pool gives its memory back to the system at every synchronisation,
 // so each call paid for mapping it again (the 32 MB kernel-row cache of a
@@ -80,15 +112,20 @@ constexpr size_t kPoolKeepBytes = (size_t)4 << 30;
 constexpr size_t kBatchCacheFree = (size_t)3 << 30;   // a buffer the pool keeps beside a call's others
 constexpr int kPoolDevices = 64;
 std::mutex g_pool_mu;
-cudaMemPool_t g_pool[kPoolDevices] = {};
+struct DevicePool {
+    cudaMemPool_t pool;
+    unsigned long long context;
+};
+DevicePool g_pool[kPoolDevices] = {};
 
 cudaMemPool_t device_pool()
 {
     int dev = 0;
     CK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kPoolDevices) return nullptr;
+    const unsigned long long context = context_id();
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    if (!g_pool[dev]) {
+    if (!g_pool[dev].pool || g_pool[dev].context != context) {
         cudaMemPoolProps props;
         std::memset(&props, 0, sizeof props);
         props.allocType = cudaMemAllocationTypePinned;
@@ -98,9 +135,9 @@ cudaMemPool_t device_pool()
         CK(cudaMemPoolCreate(&pool, &props));
         uint64_t keep = kPoolKeepBytes;
         CK(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
-        g_pool[dev] = pool;
+        g_pool[dev] = {pool, context};
     }
-    return g_pool[dev];
+    return g_pool[dev].pool;
 }
 
 void *pool_alloc(size_t bytes, cudaStream_t st)
@@ -188,8 +225,20 @@ struct HostBox {
     static constexpr size_t kBytes = 4096;
     void *p = nullptr;
     bool locked = false;
-    HostBox()
+    int device = -1;                  // where it was allocated (any device uses it)
+    unsigned long long context = 0;
+    // gone with that device's context
+    bool lost() const
     {
+        int dev = -1;
+        return locked && cudaGetDevice(&dev) == cudaSuccess && dev == device && current_context() != context;
+    }
+    void open()
+    {
+        const unsigned long long id = context_id();   // (a current context, also after a reset)
+        if (p && !lost()) return;
+        CK(cudaGetDevice(&device));
+        context = id;
         locked = cudaHostAlloc(&p, kBytes, cudaHostAllocPortable) == cudaSuccess;
         if (!locked) {
             (void)cudaGetLastError();
@@ -198,8 +247,8 @@ struct HostBox {
     }
     ~HostBox()
     {
-        if (locked) cudaFreeHost(p);
-        else ::operator delete(p);
+        if (!locked) ::operator delete(p);
+        else if (!lost()) cudaFreeHost(p);
     }
 };
 enum { BOX_INFO_X = 0, BOX_INFO_Z = 256, BOX_COUNT = 512, BOX_ERR = 520 };
@@ -207,6 +256,7 @@ template <class T>
 T *host_box(int at)
 {
     static thread_local HostBox box;
+    box.open();
     return reinterpret_cast<T *>(static_cast<unsigned char *>(box.p) + at);
 }
 
