@@ -32,10 +32,16 @@ constexpr int kBWarps = kBThreads / 32;
 constexpr int kTQ = 8;
 constexpr int kTabMax = 257;   // d <= 256
 
-// Rows list[0 .. m) (or 0 .. m-1) as bit masks of W words; emax: the largest
-// exponent field of coef (NULL: none).
+// What the sum needs to know of the coefficients (zeroed).
+struct CoefInfo {
+    int emax;       // largest exponent field of a finite one (subnormals count as 1)
+    int infinite;   // 1: a positive one is infinite, 2: a negative one
+};
+
+// Rows list[0 .. m) (or 0 .. m-1) as bit masks of W words; info: of coef
+// (NULL: none).
 __global__ void k_mask_rows(int64_t m, int W, const int32_t *list, const int64_t *indptr, const int32_t *indices,
-                            uint32_t *bits, const double *coef, int *emax)
+                            uint32_t *bits, const double *coef, CoefInfo *info)
 {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int e = 0;
@@ -51,11 +57,18 @@ __global__ void k_mask_rows(int64_t m, int W, const int32_t *list, const int64_t
         uint4 *dst = reinterpret_cast<uint4 *>(bits + (size_t)k * W);
         dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
         if (W == 8) dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-        if (coef) e = (int)(double_to_bits(coef[k]) >> 52) & 0x7ff;
+        if (coef) {
+            const uint64_t b = double_to_bits(coef[k]);
+            e = max((int)(b >> 52) & 0x7ff, 1);
+            if (e == 0x7ff) {
+                atomicOr(&info->infinite, b >> 63 ? 2 : 1);
+                e = 0;
+            }
+        }
     }
     if (coef) {
         e = __reduce_max_sync(0xffffffffu, e);
-        if ((threadIdx.x & 31) == 0 && e > *(volatile int *)emax) atomicMax(emax, e);
+        if ((threadIdx.x & 31) == 0 && e > *(volatile int *)&info->emax) atomicMax(&info->emax, e);
     }
 }
 
@@ -63,7 +76,7 @@ struct BitsArgs {
     int64_t nq, nsv;
     const uint32_t *xbits, *zbits;
     const double *coef;
-    const int *emax;
+    const CoefInfo *info;
     const double *ktab;
     int ktab_len;
     double add_scalar;
@@ -120,7 +133,7 @@ __global__ void __launch_bounds__(kBThreads) rbf_bits_kernel(BitsArgs a)
     for (int k = tid; k < kTQ * W; k += kBThreads)
         zq[k / W][k % W] = k / W < nt ? a.zbits[(size_t)(q0 + k / W) * W + k % W] : 0u;
     __syncthreads();
-    const int emax = *a.emax;
+    const int emax = a.info->emax;
     const int splits = gridDim.y;
     const int64_t k1 = a.nsv * (int64_t)(blockIdx.y + 1) / splits;
     XdAcc acc[kTQ];
@@ -134,11 +147,11 @@ __global__ void __launch_bounds__(kBThreads) rbf_bits_kernel(BitsArgs a)
             const uint4 v = __ldg(xs + j);
             x[4 * j] = v.x; x[4 * j + 1] = v.y; x[4 * j + 2] = v.z; x[4 * j + 3] = v.w;
         }
-        // |coef| 2^(1084 - emax), below 2^62
+        // |coef| 2^(1084 - emax), below 2^62 (infinite ones: see the end)
         const uint64_t cb = double_to_bits(a.coef[k]);
-        const int e = (int)(cb >> 52) & 0x7ff, sh = emax - e - 9;
-        const uint64_t m = (cb & 0x000fffffffffffffull) | (e ? 0x0010000000000000ull : 0ull);
-        const uint64_t cq = sh <= 0 ? m << -sh : (sh < 64 ? m >> sh : 0ull);
+        const int field = (int)(cb >> 52) & 0x7ff, sh = emax - max(field, 1) - 9;
+        const uint64_t m = (cb & 0x000fffffffffffffull) | (field ? 0x0010000000000000ull : 0ull);
+        const uint64_t cq = field == 0x7ff ? 0ull : (sh <= 0 ? m << -sh : (sh < 64 ? m >> sh : 0ull));
         const uint32_t neg = (uint32_t)((int32_t)(uint32_t)(cb >> 32) >> 31);
 #pragma unroll
         for (int q = 0; q < kTQ; ++q) {
@@ -204,7 +217,13 @@ __global__ void __launch_bounds__(kBThreads) rbf_bits_kernel(BitsArgs a)
     }
     // the sum counts units of 2^(emax - 1115) (rounded to 53 bits where no
     // exponent can leave the normal range, then scaled)
-    if (tid < nt) a.out[q0 + tid] = ldexp(xd_round(sum, -64), emax - 1115 + 64) + a.add_scalar;
+    if (tid < nt) {
+        double v = ldexp(xd_round(sum, -64), emax - 1115 + 64);
+        // (every K is positive, so infinite coefficients alone decide)
+        if (const int inf = a.info->infinite)
+            v = bits_to_double(inf == 1 ? 0x7ff0000000000000ull : (inf == 2 ? 0xfff0000000000000ull : 0x7ff8000000000000ull));
+        a.out[q0 + tid] = v + a.add_scalar;
+    }
 }
 
 struct Plan {
@@ -229,7 +248,7 @@ Plan plan_of(const RbfContract &c)
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     p.xbits = up(4 * (size_t)p.W * std::max<int64_t>(c.nsv, 1));
     p.zbits = up(4 * (size_t)p.W * c.nq);
-    p.head = up(sizeof(int) * (1 + (size_t)p.tiles));
+    p.head = up(sizeof(CoefInfo) + sizeof(unsigned) * (size_t)p.tiles);
     p.part = up(p.splits > 1 ? 16 * (size_t)p.splits * c.nq : 0);
     return p;
 }
@@ -257,8 +276,8 @@ cudaError_t launch_rbf_bits(const RbfContract &c, void *ws, cudaStream_t st)
     unsigned char *w = static_cast<unsigned char *>(ws);
     uint32_t *xbits = reinterpret_cast<uint32_t *>(w);
     uint32_t *zbits = reinterpret_cast<uint32_t *>(w + p.xbits);
-    int *head = reinterpret_cast<int *>(w + p.xbits + p.zbits);
-    cudaError_t e = cudaMemsetAsync(head, 0, sizeof(int) * (1 + (size_t)p.tiles), st);
+    CoefInfo *head = reinterpret_cast<CoefInfo *>(w + p.xbits + p.zbits);
+    cudaError_t e = cudaMemsetAsync(head, 0, sizeof(CoefInfo) + sizeof(unsigned) * (size_t)p.tiles, st);
     if (e != cudaSuccess) return e;
     if (c.nsv > 0)
         k_mask_rows<<<(unsigned)((c.nsv + 127) / 128), 128, 0, st>>>(c.nsv, p.W, c.sv, c.x_indptr, c.x_indices, xbits,
@@ -271,12 +290,12 @@ cudaError_t launch_rbf_bits(const RbfContract &c, void *ws, cudaStream_t st)
     a.xbits = xbits;
     a.zbits = zbits;
     a.coef = c.coef;
-    a.emax = head;
+    a.info = head;
     a.ktab = c.ktab;
     a.ktab_len = c.ktab_len;
     a.add_scalar = c.add_scalar;
     a.out = c.out;
-    a.done = reinterpret_cast<unsigned *>(head) + 1;
+    a.done = reinterpret_cast<unsigned *>(head + 1);
     a.part = reinterpret_cast<uint4 *>(w + p.xbits + p.zbits + p.head);
     const dim3 grid((unsigned)p.tiles, (unsigned)p.splits);
     if (p.W == 4) rbf_bits_kernel<4><<<grid, kBThreads, 0, st>>>(a);
