@@ -140,10 +140,9 @@ cudaMemPool_t device_pool()
     return g_pool[dev].pool;
 }
 
-void *pool_alloc(size_t bytes, cudaStream_t st)
+void *pool_alloc(cudaMemPool_t pool, size_t bytes, cudaStream_t st)
 {
     void *p = nullptr;
-    cudaMemPool_t pool = device_pool();
     if (!pool) {
         CK(cudaMallocAsync(&p, bytes, st));
         return p;
@@ -185,7 +184,8 @@ struct Arena {
     unsigned char *slab = nullptr;
     size_t slab_used = 0;
     int exceptions;
-    explicit Arena(cudaStream_t s) : st(s), exceptions(std::uncaught_exceptions()) {}
+    cudaMemPool_t pool;
+    explicit Arena(cudaStream_t s) : st(s), exceptions(std::uncaught_exceptions()), pool(device_pool()) {}
     Arena(const Arena &) = delete;
     Arena &operator=(const Arena &) = delete;
     template <class T>
@@ -194,14 +194,14 @@ struct Arena {
         const size_t bytes = ((count ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
         if (bytes <= kSmall) {
             if (!slab || slab_used + bytes > kSlab) {
-                slab = static_cast<unsigned char *>(keep(pool_alloc(kSlab, st)));
+                slab = static_cast<unsigned char *>(keep(pool_alloc(pool, kSlab, st)));
                 slab_used = 0;
             }
             unsigned char *p = slab + slab_used;
             slab_used += bytes;
             return reinterpret_cast<T *>(p);
         }
-        return static_cast<T *>(keep(pool_alloc(bytes, st)));
+        return static_cast<T *>(keep(pool_alloc(pool, bytes, st)));
     }
     ~Arena()
     {
@@ -227,16 +227,16 @@ struct HostBox {
     bool locked = false;
     int device = -1;                  // where it was allocated (any device uses it)
     unsigned long long context = 0;
-    // gone with that device's context
-    bool lost() const
+    // gone with that device's context; id: the current one
+    bool lost(unsigned long long id) const
     {
         int dev = -1;
-        return locked && cudaGetDevice(&dev) == cudaSuccess && dev == device && current_context() != context;
+        return locked && id != context && cudaGetDevice(&dev) == cudaSuccess && dev == device;
     }
     void open()
     {
         const unsigned long long id = context_id();   // (a current context, also after a reset)
-        if (p && !lost()) return;
+        if (p && !lost(id)) return;
         CK(cudaGetDevice(&device));
         context = id;
         locked = cudaHostAlloc(&p, kBytes, cudaHostAllocPortable) == cudaSuccess;
@@ -248,7 +248,7 @@ struct HostBox {
     ~HostBox()
     {
         if (!locked) ::operator delete(p);
-        else if (!lost()) cudaFreeHost(p);
+        else if (!lost(current_context())) cudaFreeHost(p);
     }
 };
 enum { BOX_INFO_X = 0, BOX_INFO_Z = 256, BOX_COUNT = 512, BOX_ERR = 520 };
@@ -2921,7 +2921,7 @@ void srv_admit(Server &S, const std::shared_ptr<SrvJob> &J)
     const bool mixed = S.mode == MODE_MIXED;
     const bool dense = mixed && J->nnz == J->n * J->d;
     const int dpad = (int)((J->d + 7) & ~7ll);
-    J->mem = pool_alloc(J->bytes, st);
+    J->mem = pool_alloc(device_pool(), J->bytes, st);
     unsigned char *p = static_cast<unsigned char *>(J->mem);
     auto take = [&](size_t x) {
         unsigned char *r = p;
