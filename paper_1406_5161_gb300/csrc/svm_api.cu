@@ -220,35 +220,69 @@ private:
 };
 
 // Page-locked host memory of the calling thread for small results read back
-// between launches (a copy to pageable memory is staged by the driver).
-struct HostBox {
-    static constexpr size_t kBytes = 4096;
-    void *p = nullptr;
+// between launches (a copy to pageable memory is staged by the driver). Boxes
+// are cut from one allocation, lent to a thread until it ends, and never freed:
+// page-locked memory that one thread freed made the next allocation wait for
+// all running kernels, so that a call from a new thread waited seconds for the
+// persistent engine of a busy server.
+struct HostBoxes {
+    static constexpr size_t kBytes = 1024, kCount = 64;
+    std::mutex mu;
+    std::vector<void *> free;
     bool locked = false;
-    int device = -1;                  // where it was allocated (any device uses it)
+    int device = -1;                  // where they were allocated (any device uses them)
     unsigned long long context = 0;
-    // gone with that device's context; id: the current one
-    bool lost(unsigned long long id) const
+    unsigned generation = 0;          // one per allocation that is still valid
+
+    // a box, keeping `p` of `gen` while that is valid; id: the current context
+    void *take(void *p, unsigned &gen, unsigned long long id)
     {
+        std::lock_guard<std::mutex> lk(mu);
         int dev = -1;
-        return locked && id != context && cudaGetDevice(&dev) == cudaSuccess && dev == device;
-    }
-    void open()
-    {
-        const unsigned long long id = context_id();   // (a current context, also after a reset)
-        if (p && !lost(id)) return;
-        CK(cudaGetDevice(&device));
-        context = id;
-        locked = cudaHostAlloc(&p, kBytes, cudaHostAllocPortable) == cudaSuccess;
-        if (!locked) {
-            (void)cudaGetLastError();
-            p = ::operator new(kBytes);
+        CK(cudaGetDevice(&dev));
+        if (locked && dev == device && id != context) {   // gone with that device's context
+            free.clear();
+            locked = false;
+            ++generation;
         }
+        if (p && gen == generation) return p;
+        if (free.empty()) {
+            unsigned char *q = nullptr;
+            if (cudaHostAlloc(reinterpret_cast<void **>(&q), kBytes * kCount, cudaHostAllocPortable) == cudaSuccess) {
+                if (!locked) {
+                    locked = true;
+                    device = dev;
+                    context = id;
+                }
+            } else {
+                (void)cudaGetLastError();
+                q = static_cast<unsigned char *>(::operator new(kBytes * kCount));
+            }
+            for (size_t k = 0; k < kCount; ++k) free.push_back(q + k * kBytes);
+        }
+        gen = generation;
+        p = free.back();
+        free.pop_back();
+        return p;
     }
+    void give(void *p, unsigned gen)
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        if (gen == generation) free.push_back(p);
+    }
+};
+HostBoxes &host_boxes()
+{
+    static HostBoxes *boxes = new HostBoxes;   // threads may end after the process's statics
+    return *boxes;
+}
+struct HostBox {
+    void *p = nullptr;
+    unsigned generation = 0;
+    unsigned long long context = 0;   // the one it was last taken under
     ~HostBox()
     {
-        if (!locked) ::operator delete(p);
-        else if (!lost(current_context())) cudaFreeHost(p);
+        if (p) host_boxes().give(p, generation);
     }
 };
 enum { BOX_INFO_X = 0, BOX_INFO_Z = 256, BOX_COUNT = 512, BOX_ERR = 520 };
@@ -256,7 +290,11 @@ template <class T>
 T *host_box(int at)
 {
     static thread_local HostBox box;
-    box.open();
+    const unsigned long long id = context_id();   // (a current context, also after a reset)
+    if (!box.p || box.context != id) {
+        box.p = host_boxes().take(box.p, box.generation, id);
+        box.context = id;
+    }
     return reinterpret_cast<T *>(static_cast<unsigned char *>(box.p) + at);
 }
 
@@ -1251,7 +1289,9 @@ int train_impl(const svm_csr *X, const int8_t *y, const svm_params *P, const svm
             // kernel-row cache and are then bound by the exchange (short rows,
             // 9,000 / 12,000 of them: 4.6 / 4.9 us a step on one cluster, 5.5 /
             // 5.7 on clusters of 8; 16,000: 6.4 against 5.8; without cached
-            // rows 9.1 / 10.2 against 6.1 / 6.4)
+            // rows 9.1 / 10.2 against 6.1 / 6.4). Measured on rows of 12
+            // entries; longer rows than 16 stay where they were. The steps
+            // are the same bit for bit on either side of the line.
             const bool late = kdir_l > 0 && n_l < n && (double)nnz_l <= 16.0 * (double)n_l;
             const int64_t one_cluster_max = kmode == MODE_FP64 ? (late ? kFp64OneClusterLate : kFp64OneClusterRows) : 200000;
             if (L16.total <= lim_dyn && smo_max_clusters(kmode, lpr, 2, L16.total, 16) >= 1 &&
