@@ -345,7 +345,8 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                     }
                 }
                 // the warps of the pair step's bounds only arrive; with both
-                // kernel rows cached no row warp needs the targets
+                // kernel rows cached no row warp waits for the targets (warp
+                // 0 does: its K(up, low) is computed from them)
                 const bool both = hu && hl;
                 if (warp >= kPre0 || (both && warp != 0)) fill_bar_arrive();
                 else fill_bar_sync();
@@ -763,7 +764,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                             if (dense) {
                                 if constexpr (MODE == MODE_MIXED) {
                                 const __nv_bfloat16 *xr = dmat + (size_t)g * d;
-                                for (int c = gl * 8; c < d; c += LPR * 8) {
+                                auto piece = [&](int c) {
                                     const uint4 raw = *reinterpret_cast<const uint4 *>(xr + c);
                                     const __nv_bfloat162 *h2 = reinterpret_cast<const __nv_bfloat162 *>(&raw);
 #pragma unroll
@@ -775,6 +776,15 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                                         su = fmaf(v.y, t1.x, su);
                                         sl = fmaf(v.y, t1.y, sl);
                                     }
+                                };
+                                // long rows wait for loads: eight pieces'
+                                // at a time (1,306 x 1,587, 2 lanes, 14.6 ->
+                                // 13.1 us a step; 64 columns 3% slower so)
+                                if (d >= 16 * LPR * 8) {
+#pragma unroll 8
+                                    for (int c = gl * 8; c < d; c += LPR * 8) piece(c);
+                                } else {
+                                    for (int c = gl * 8; c < d; c += LPR * 8) piece(c);
                                 }
                                 }
                             } else if (xd) {
@@ -916,13 +926,12 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
             //         candidate into every CTA's shared memory, as asynchronous
             //         stores counted on its mbarrier (lanes q and 16 + q send
             //         the first 48 bytes of the I_up and I_low sides to CTA q);
-            //         every CTA reduces them in the same order. With the
-            //         gap test beside the pair step, no target fill once both
-            //         rows are cached and four entries' loads in flight, 45 FP64
-            //         problems of 1,500 rows (d = 20, clusters of 4 CTAs) took
-            //         28.7 instead of 35.0 ms (two cluster barriers a step
-            //         before, 530 cycles each); 90 mixed ones of about 4,000
-            //         rows (d = 256, 2 CTAs) 104.6 ms as before.
+            //         every CTA reduces them in the same order. (Two cluster
+            //         barriers a step before, 530 cycles each. With the gap
+            //         test beside the pair step and row warps that do not
+            //         wait for the target fill when both rows are cached, 45
+            //         FP64 problems of 1,500 rows, d = 20, clusters of 4 CTAs,
+            //         on one input: 35.0 -> 28.7 ms.)
             ++epoch;
             const int par = (int)(epoch & 1);
             if (warp == 0) {
