@@ -1530,60 +1530,56 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
                 if (xd && !first && !skip_sums) {
                     if constexpr (MODE == MODE_FP64) {
                         // exact inner products in integer arithmetic, each
-                        // lane loading its next XB entries at once (4: fewer
-                        // live registers than 8, measured 3% faster)
-                        constexpr int XB = 4;
-                        if (!kc_hu && !kc_hl) {
+                        // lane loading four entries at once (fewer live
+                        // registers than 8, measured 3% faster), the rest of
+                        // the row one by one; a side whose row is in the cache
+                        // is left out. (Bound by issue: with a bound check per
+                        // entry 20,000 x 128 rows took 23.7 ms for 1,200 steps
+                        // without cache, 20.3 so; 120,000 covtype-shaped rows
+                        // 558.8 and 545.8.)
+                        XdAcc au = xd_zero(), al = xd_zero();
+                        auto sum_row = [&](auto two) {
                             const int4 *T4 = reinterpret_cast<const int4 *>(T);
-                            XdAcc au = xd_zero(), al = xd_zero();
-                            for (int64_t pb = p0 + gl; pb < p1; pb += XB * LPR) {
-                                int cb[XB];
-                                uint32_t ub[XB];
-#pragma unroll
-                                for (int j = 0; j < XB; ++j) {
-                                    const int64_t p = pb + (int64_t)j * LPR;
-                                    cb[j] = 0;
-                                    ub[j] = 0u;
-                                    if (p < p1) XCW(p, cb[j], ub[j]);
-                                }
-#pragma unroll
-                                for (int j = 0; j < XB; ++j) {
-                                    if (pb + (int64_t)j * LPR >= p1) break;
-                                    const int32_t m = xd_word_m(ub[j]);
-                                    const int e = xd_word_e(ub[j]);
-                                    const int4 t = T4[cb[j]];
+                            const int2 *T2 = reinterpret_cast<const int2 *>(T) + (kc_hu ? 1 : 0);
+                            auto entry = [&](int c, uint32_t u) {
+                                const int32_t m = xd_word_m(u);
+                                const int e = xd_word_e(u);
+                                if constexpr (two()) {
+                                    const int4 t = T4[c];
                                     xd_add(au, m, t.x, e + t.y);
                                     xd_add(al, m, t.z, e + t.w);
+                                } else {
+                                    const int2 t = T2[2 * c];
+                                    xd_add(au, m, t.x, e + t.y);
                                 }
-                            }
-                            xd_lane_sum<LPR>(au);
-                            xd_lane_sum<LPR>(al);
-                            su = xd_round(au, xd_unit);
-                            sl = xd_round(al, xd_unit);
-                        } else {
-                            // the other side's row is in the cache
-                            const int2 *T2 = reinterpret_cast<const int2 *>(T) + (kc_hu ? 1 : 0);
-                            XdAcc a = xd_zero();
-                            for (int64_t pb = p0 + gl; pb < p1; pb += XB * LPR) {
+                            };
+                            constexpr int XB = 4;
+                            int64_t p = p0 + gl;
+#pragma unroll 1
+                            for (; p + (XB - 1) * LPR < p1; p += XB * LPR) {
                                 int cb[XB];
                                 uint32_t ub[XB];
 #pragma unroll
-                                for (int j = 0; j < XB; ++j) {
-                                    const int64_t p = pb + (int64_t)j * LPR;
-                                    cb[j] = 0;
-                                    ub[j] = 0u;
-                                    if (p < p1) XCW(p, cb[j], ub[j]);
-                                }
+                                for (int j = 0; j < XB; ++j) XCW(p + (int64_t)j * LPR, cb[j], ub[j]);
 #pragma unroll
-                                for (int j = 0; j < XB; ++j) {
-                                    if (pb + (int64_t)j * LPR >= p1) break;
-                                    const int2 t = T2[2 * cb[j]];
-                                    xd_add(a, xd_word_m(ub[j]), t.x, xd_word_e(ub[j]) + t.y);
-                                }
+                                for (int j = 0; j < XB; ++j) entry(cb[j], ub[j]);
                             }
-                            xd_lane_sum<LPR>(a);
-                            su = sl = xd_round(a, xd_unit);
-                        }
+#pragma unroll 1
+                            for (; p < p1; p += LPR) {
+                                int c = 0;
+                                uint32_t u = 0;
+                                XCW(p, c, u);
+                                entry(c, u);
+                            }
+                            xd_lane_sum<LPR>(au);
+                            su = sl = xd_round(au, xd_unit);
+                            if constexpr (two()) {
+                                xd_lane_sum<LPR>(al);
+                                sl = xd_round(al, xd_unit);
+                            }
+                        };
+                        if (!kc_hu && !kc_hl) sum_row(std::true_type{});
+                        else sum_row(std::false_type{});
                     }
                 } else if constexpr (BITS) {
                     // squared distances to x_up and x_low (one lane per row)
