@@ -295,6 +295,11 @@ int svm_train(const svm_csr *X, const int8_t *y, const svm_params *params,
  *   Z            m query rows with Z->d == X->d (space of Z; out in that space)
  *   precision    enum svm_precision (SVM_MIXED_BF16 uses the tensor cores)
  *   stream       cudaStream_t or NULL
+ * The sum over the support vectors is split over the device by the number of
+ * queries: a query's value may differ in its last bits between calls that
+ * score different numbers of rows, or on devices with another number of SMs
+ * (not where binary rows are summed exactly, as bit masks). The same call gives
+ * the same bits. svm_decision_kernel and svm_model_decision alike.
  */
 int svm_decision(const svm_csr *X, const int8_t *y, const double *alpha, double b,
                  double gamma, const svm_csr *Z, int32_t precision, void *stream,
@@ -366,7 +371,9 @@ typedef struct svm_result {
     double b_up, b_low;      /* Eq. (bminmax) at exit */
     double objective;        /* dual objective W */
     int64_t iters;
-    int32_t status;          /* SVM_OK or SVM_NOT_CONVERGED */
+    int32_t status;          /* SVM_OK or SVM_NOT_CONVERGED; from the server also an
+                                error (a wait gave up: SVM_ERR_TIMEOUT), the other
+                                fields then 0 */
     int32_t n_sv;
 } svm_result;
 
@@ -390,8 +397,11 @@ typedef struct svm_batch_config {
  * each job's rows are split over the CTAs of one cluster, which exchange
  * their candidates through distributed shared memory. X is ingested once for
  * all jobs. Results and multipliers are those each job would get alone with
- * svm_train at the same precision (no shrinking). Returns SVM_OK,
- * SVM_NOT_CONVERGED (some job hit max_iter) or an error.
+ * svm_train at the same precision (no shrinking). FP64 jobs keep kernel rows
+ * in device memory while the call runs: up to half of what is available, at
+ * most 32 GiB, more than 3 GiB only when the solve takes long enough to gain by
+ * it. Returns SVM_OK, SVM_NOT_CONVERGED (some job hit max_iter) or an error
+ * (SVM_ERR_TIMEOUT when a wait of the kernel gave up).
  */
 int svm_train_batch(const svm_csr *X, const svm_job *jobs, int32_t n_jobs,
                     svm_batch_config *config, svm_result *results);

@@ -178,6 +178,7 @@ struct BatchJobDev {
     double C, gamma, tau;
     int64_t max_iter;
     int64_t iter0;             // > 0: continue after that many steps of an earlier launch
+                               // (jobs without packed rows)
     XdFormat xd;               // FP64 mode: exact inner products (xd.on)
 };
 
