@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                 ktab[B.ktab_len + k] = eta > 1e-12 ? 1.0 / eta : 0.0;
             }
         }
-        for (int r = lo + tid; r < hi && J.iter0 == 0; r += kThreads) {
+        for (int r = lo + tid; r < hi && (MODE != MODE_FP64 || J.iter0 == 0); r += kThreads) {
             const int8_t yr = yj[r];
             aj[r] = 0.0;
             fj[r] = -(double)yr;
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
         side_empty(up, true);
         side_empty(low, false);
         bool first = true;
-        int64_t iter = J.iter0;
+        int64_t iter = MODE == MODE_FP64 ? J.iter0 : 0;   // (only FP64 jobs are continued)
         int prev_valid = 0, prev_len_u = 0, prev_len_l = 0;
         int status_code = JOB_CONVERGED;
         for (;;) {
@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(kThreads, 1) smo_batch_kernel(BatchArgs B)
                                 // long rows wait for loads: eight pieces'
                                 // at a time (1,306 x 1,587, 2 lanes, 14.6 ->
                                 // 13.1 us a step; 64 columns 3% slower so)
-                                if (d >= 16 * LPR * 8) {
+                                if (LPR <= 8 && d >= 16 * LPR * 8) {
 #pragma unroll 8
                                     for (int c = gl * 8; c < d; c += LPR * 8) piece(c);
                                 } else {
