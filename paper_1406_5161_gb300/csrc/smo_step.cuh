@@ -747,9 +747,9 @@ __global__ void __launch_bounds__(kThreads, 1) smo_persistent_kernel(SmoArgs A)
     Side up, low;
     side_empty(up, true);
     side_empty(low, false);
-    // every launch begins with a selection pass (not a constant to the
-    // compiler, whose code for the steps is 1% slower on mixed rows with one)
-    bool first = A.n > 0;
+    // every launch begins with a selection pass (always true, but no constant
+    // to the compiler, whose code for the mixed steps is 1% slower with one)
+    bool first = C0.iter >= 0;
     // one cluster over the whole grid: candidates go to every CTA as
     // asynchronous stores whose bytes each CTA counts on its own mbarrier
     // (one per epoch parity; the CTA's own arrival sets the expected bytes)
